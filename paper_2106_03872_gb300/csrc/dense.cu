@@ -63,7 +63,8 @@ __global__ void __launch_bounds__(256) k_gemm_cn(const cplx<T>* __restrict__ A, 
     }
 }
 
-__global__ void k_reduce_parts(const double2* __restrict__ part, int nks, size_t mn, double2* __restrict__ out) {
+__global__ void k_reduce_parts(const double2* __restrict__ part, int nks, size_t mn, double2* __restrict__ out,
+                               float2* __restrict__ out32) {
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < mn; e += (size_t)gridDim.x * blockDim.x) {
     double2 s = make_double2(0.0, 0.0);
     for (int k = 0; k < nks; ++k) {
@@ -72,12 +73,13 @@ __global__ void k_reduce_parts(const double2* __restrict__ part, int nks, size_t
       s.y += p.y;
     }
     out[e] = s;
+    if (out32) out32[e] = make_float2((float)s.x, (float)s.y);
   }
 }
 
 // Y[i][k] = sum_j M[i][j] X[j][k]; tile 32 rows x 64 columns, each thread 2 x 4 outputs.
-template <typename T>
-__global__ void __launch_bounds__(256) k_rotate(const double2* __restrict__ M, int nin, const cplx<T>* __restrict__ X,
+template <typename T, typename MC>
+__global__ void __launch_bounds__(256) k_rotate(const MC* __restrict__ M, int nin, const cplx<T>* __restrict__ X,
                                                 const cplx<T>* __restrict__ X2, int nin1, int ldx, cplx<T>* __restrict__ Y,
                                                 int ldy, int m, int K) {
   using C = cplx<T>;
@@ -89,8 +91,12 @@ __global__ void __launch_bounds__(256) k_rotate(const double2* __restrict__ M, i
   for (int j0 = 0; j0 < nin; j0 += KT) {
     for (int e = threadIdx.x; e < 32 * KT; e += 256) {
       const int r = e / KT, jj = e % KT;
-      const double2 v = (i0 + r < m && j0 + jj < nin) ? M[(size_t)(i0 + r) * nin + j0 + jj] : make_double2(0.0, 0.0);
-      Ms[r][jj] = mk<C>(T(v.x), T(v.y));
+      C v = mk<C>(T(0), T(0));
+      if (i0 + r < m && j0 + jj < nin) {
+        const MC q = M[(size_t)(i0 + r) * nin + j0 + jj];
+        v = mk<C>(T(q.x), T(q.y));
+      }
+      Ms[r][jj] = v;
     }
     for (int e = threadIdx.x; e < KT * 64; e += 256) {
       const int jj = e / 64, c = e % 64;
@@ -313,138 +319,43 @@ __global__ void __launch_bounds__(1024) k_jacobi(double2* __restrict__ A, double
   }
 }
 
-// The same parallel round-robin Jacobi in FP32 for the mixed path's subspace problems of
-// 128 < n <= 256 (the one-CTA Householder solver holds n <= 128 in shared memory): A (FP32,
-// destroyed) and the eigenvector columns V in global memory, L2-resident; rotations of pairs
-// whose coupling is below 1e-6 |A|_F are skipped (FP32 rounding of a rotated entry is ~6e-8
-// |A|), so the sweeps stop once the off-diagonal part is at FP32 level.  No sorting: the caller
-// takes FP64 Rayleigh quotients of the vectors, then sorts (eigh_jacobi_mixed).
-__device__ __forceinline__ float2 cmulf(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
-__device__ __forceinline__ float2 cconjf(float2 a) { return make_float2(a.x, -a.y); }
-__device__ __forceinline__ float2 cscalef(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
-
-__global__ void __launch_bounds__(1024) k_jacobi32(float2* __restrict__ A, float2* __restrict__ V, int n) {
-  __shared__ int sp[256], sq[256];
-  __shared__ float sc[256], ss[256];
-  __shared__ float2 se[256];
-  __shared__ int srot;
-  __shared__ float sthr;
-  __shared__ float red[32];
-  const int P = n + (n & 1);
-  const int np = P / 2;
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) V[e] = make_float2((e / n == e % n) ? 1.f : 0.f, 0.f);
-  float f = 0.f;
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) f += A[e].x * A[e].x + A[e].y * A[e].y;
-  for (int o = 16; o > 0; o >>= 1) f += __shfl_down_sync(0xffffffffu, f, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = f;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float t = 0.f;
-    for (int w = 0; w < (int)((blockDim.x + 31) >> 5); ++w) t += red[w];
-    sthr = 1e-6f * sqrtf(t);
-  }
-  __syncthreads();
-  for (int sweep = 0; sweep < 40; ++sweep) {
-    if (threadIdx.x == 0) srot = 0;
-    __syncthreads();
-    for (int r = 0; r < P - 1; ++r) {
-      if (threadIdx.x < np) {
-        const int k = threadIdx.x;
-        const int pa = k, pb = P - 1 - k;
-        const int ua = (pa == 0) ? 0 : 1 + ((pa - 1 + r) % (P - 1));
-        const int ub = (pb == 0) ? 0 : 1 + ((pb - 1 + r) % (P - 1));
-        const int p = min(ua, ub), q = max(ua, ub);
-        int active = 0;
-        if (q < n) {
-          const float2 b = A[(size_t)p * n + q];
-          const float mag = hypotf(b.x, b.y);
-          if (mag > sthr) {
-            const float alpha = A[(size_t)p * n + p].x, gamma = A[(size_t)q * n + q].x;
-            const float tau = (gamma - alpha) / (2.f * mag);
-            const float t = (tau >= 0.f ? 1.f : -1.f) / (fabsf(tau) + sqrtf(1.f + tau * tau));
-            const float c = 1.f / sqrtf(1.f + t * t);
-            sc[k] = c;
-            ss[k] = t * c;
-            se[k] = make_float2(b.x / mag, b.y / mag);
-            active = 1;
-            srot = 1;
-          }
-        }
-        sp[k] = p;
-        sq[k] = active ? q : -1;
-      }
-      __syncthreads();
-      for (int job = threadIdx.x; job < np * n; job += blockDim.x) {     // rows: A <- J^H A
-        const int k = job / n, j = job % n;
-        const int q = sq[k];
-        if (q < 0) continue;
-        const int p = sp[k];
-        const float c = sc[k], sv = ss[k];
-        const float2 e = se[k];
-        const float2 ap = A[(size_t)p * n + j], aq = A[(size_t)q * n + j];
-        A[(size_t)p * n + j] = cscalef(ap, c) - cscalef(cmulf(e, aq), sv);
-        A[(size_t)q * n + j] = cscalef(cmulf(cconjf(e), ap), sv) + cscalef(aq, c);
-      }
-      __syncthreads();
-      for (int job = threadIdx.x; job < np * n; job += blockDim.x) {     // columns: A <- A J, V <- V J
-        const int k = job / n, i = job % n;
-        const int q = sq[k];
-        if (q < 0) continue;
-        const int p = sp[k];
-        const float c = sc[k], sv = ss[k];
-        const float2 e = se[k];
-        float2 ap = A[(size_t)i * n + p], aq = A[(size_t)i * n + q];
-        A[(size_t)i * n + p] = cscalef(ap, c) - cscalef(cmulf(cconjf(e), aq), sv);
-        A[(size_t)i * n + q] = cscalef(cmulf(e, ap), sv) + cscalef(aq, c);
-        ap = V[(size_t)i * n + p];
-        aq = V[(size_t)i * n + q];
-        V[(size_t)i * n + p] = cscalef(ap, c) - cscalef(cmulf(cconjf(e), aq), sv);
-        V[(size_t)i * n + q] = cscalef(cmulf(e, ap), sv) + cscalef(aq, c);
-      }
-      __syncthreads();
-    }
-    if (srot == 0) break;
-    __syncthreads();
-  }
-}
-
-__global__ void k_c128_to_c64(const double2* __restrict__ in, float2* __restrict__ out, size_t n) {
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
-    out[e] = make_float2((float)in[e].x, (float)in[e].y);
-}
-__global__ void k_c64_to_c128(const float2* __restrict__ in, double2* __restrict__ out, size_t n) {
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
-    out[e] = make_double2((double)in[e].x, (double)in[e].y);
-}
-
-// lam[i] = v_i^H H v_i / v_i^H v_i in FP64 (column i of V), one CTA per i.
-__global__ void k_rayleigh_quotients(const double2* __restrict__ H, const double2* __restrict__ V, int n,
-                                     double* __restrict__ lam) {
-  const int i = blockIdx.x;
+// lam[i] = v_i^H H v_i / v_i^H v_i in FP64 (column i of V), one CTA per i; a warp per row of the
+// upper triangle (H is Hermitian: the FP64 products bound this kernel, and half of them do).
+__global__ void __launch_bounds__(256) k_rayleigh_quotients(const double2* __restrict__ H, const double2* __restrict__ V,
+                                                            int n, double* __restrict__ lam) {
+  const int i = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   __shared__ double2 vi[512];
-  __shared__ double red[2][32];
+  __shared__ double red[2][8];
   for (int k = threadIdx.x; k < n; k += blockDim.x) vi[k] = V[(size_t)k * n + i];
   __syncthreads();
   double num = 0.0, den = 0.0;
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-    const int j = e / n, k = e % n;
-    // conj(v_j) H_jk v_k
-    const double2 hv = zmul(H[e], vi[k]);
-    num += vi[j].x * hv.x + vi[j].y * hv.y;
-    if (j == k) den += vi[k].x * vi[k].x + vi[k].y * vi[k].y;
+  for (int j = warp; j < n; j += 8) {
+    const double2 vj = vi[j];
+    double2 s = make_double2(0.0, 0.0);
+    for (int k = j + 1 + lane; k < n; k += 32) {
+      const double2 h = H[(size_t)j * n + k], x = vi[k];
+      s.x = fma(h.x, x.x, fma(-h.y, x.y, s.x));
+      s.y = fma(h.x, x.y, fma(h.y, x.x, s.y));
+    }
+    num += 2.0 * (vj.x * s.x + vj.y * s.y);                          // Re(conj(v_j) H_jk v_k), twice
+    if (lane == 0) {
+      const double m = vj.x * vj.x + vj.y * vj.y;
+      num += H[(size_t)j * n + j].x * m;
+      den += m;
+    }
   }
   for (int o = 16; o > 0; o >>= 1) {
     num += __shfl_down_sync(0xffffffffu, num, o);
     den += __shfl_down_sync(0xffffffffu, den, o);
   }
-  if ((threadIdx.x & 31) == 0) {
-    red[0][threadIdx.x >> 5] = num;
-    red[1][threadIdx.x >> 5] = den;
+  if (lane == 0) {
+    red[0][warp] = num;
+    red[1][warp] = den;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     double a = 0, b = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+    for (int w = 0; w < 8; ++w) {
       a += red[0][w];
       b += red[1][w];
     }
@@ -460,9 +371,12 @@ template <bool MIXED>
 __global__ void __launch_bounds__(64) k_small_product(const double2* __restrict__ A, const double2* __restrict__ B,
                                                       int n, int flags, double2* __restrict__ C) {
   constexpr int KC = 32;
+  // MIXED operands are rounded as they are staged (64 conversions per element at the FP64 rate were
+  // most of the kernel when every product converted its own)
   using R = typename std::conditional<MIXED, float, double>::type;
-  __shared__ double2 As[8][KC + 1];
-  __shared__ double2 Bs[8][KC + 1];                                  // Bs[j][k] = opB(B)_kj
+  using C2 = cplx<R>;
+  __shared__ C2 As[8][KC + 1];
+  __shared__ C2 Bs[8][KC + 1];                                       // Bs[j][k] = opB(B)_kj
   const int ty = threadIdx.x >> 3, tx = threadIdx.x & 7;
   const int I = blockIdx.y * 8, J = blockIdx.x * 8;
   const bool ca = flags & 1, tb = flags & 2, cb = flags & 4;
@@ -472,7 +386,7 @@ __global__ void __launch_bounds__(64) k_small_product(const double2* __restrict_
       const int r = e / KC, k = kc + e % KC;
       double2 a = (I + r < n && k < n) ? A[(size_t)(I + r) * n + k] : make_double2(0.0, 0.0);
       if (ca) a.y = -a.y;
-      As[r][e % KC] = a;
+      As[r][e % KC] = mk<C2>((R)a.x, (R)a.y);
       double2 b;
       int jj, kk;
       if (tb) {                                                      // opB(B)_kj = B_jk: rows J..J+7
@@ -485,16 +399,15 @@ __global__ void __launch_bounds__(64) k_small_product(const double2* __restrict_
         b = (kc + kk < n && J + jj < n) ? B[(size_t)(kc + kk) * n + J + jj] : make_double2(0.0, 0.0);
       }
       if (cb) b.y = -b.y;
-      Bs[jj][kk] = b;
+      Bs[jj][kk] = mk<C2>((R)b.x, (R)b.y);
     }
     __syncthreads();
     R cr = 0, ci = 0;
 #pragma unroll 8
     for (int kk = 0; kk < KC; ++kk) {
-      const double2 a = As[ty][kk], b = Bs[tx][kk];
-      const R ax = (R)a.x, ay = (R)a.y, bx = (R)b.x, by = (R)b.y;
-      cr += ax * bx - ay * by;
-      ci += ax * by + ay * bx;
+      const C2 a = As[ty][kk], b = Bs[tx][kk];
+      cr += a.x * b.x - a.y * b.y;
+      ci += a.x * b.y + a.y * b.x;
     }
     re += (double)cr;
     im += (double)ci;
@@ -517,38 +430,73 @@ __global__ void k_sd_matrix(const double2* __restrict__ C, const double* __restr
   }
 }
 
-// Sort by lam (ties by index), normalise, fix phases; Vt row r = eigenvector of rank r.
-__global__ void k_sort_vectors(const double* __restrict__ lam, const double2* __restrict__ V, int n,
-                               double* __restrict__ eig, double2* __restrict__ Vt) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double li = lam[i];
-    int rank = 0;
-    for (int j = 0; j < n; ++j) rank += (lam[j] < li) || (lam[j] == li && j < i);
-    int kmax = 0;
-    double best = -1.0, nrm = 0.0;
-    for (int j = 0; j < n; ++j) {
-      const double2 v = V[(size_t)j * n + i];
-      const double m2 = v.x * v.x + v.y * v.y;
-      nrm += m2;
-      if (m2 > best) {
-        best = m2;
-        kmax = j;
-      }
+// Sort by lam (ties by index), normalise, fix phases; Vt row r = eigenvector of rank r.  One CTA
+// per vector (one thread per vector took the column's dependent loads one by one: 128 threads of
+// one SM for the whole matrix).
+constexpr int SV_THREADS = 128;
+__global__ void __launch_bounds__(SV_THREADS) k_sort_vectors(const double* __restrict__ lam, const double2* __restrict__ V,
+                                                             int n, double* __restrict__ eig, double2* __restrict__ Vt) {
+  constexpr int NW = SV_THREADS / 32;
+  __shared__ double sb[NW], sn[NW];
+  __shared__ int sk[NW], sr[NW];
+  const int i = blockIdx.x, t = threadIdx.x;
+  const double li = lam[i];
+  int rank = 0, kmax = n;
+  double best = -1.0, nrm = 0.0;
+  for (int j = t; j < n; j += SV_THREADS) {
+    rank += (lam[j] < li) || (lam[j] == li && j < i);
+    const double2 v = V[(size_t)j * n + i];
+    const double m2 = v.x * v.x + v.y * v.y;
+    nrm += m2;
+    if (m2 > best) {
+      best = m2;
+      kmax = j;
     }
-    const double2 vk = V[(size_t)kmax * n + i];
-    const double mag = sqrt(best);
-    const double sc = 1.0 / (mag * sqrt(nrm));
-    const double2 ph = make_double2(vk.x * sc, -vk.y * sc);
-    eig[rank] = li;
-    for (int j = 0; j < n; ++j) Vt[(size_t)rank * n + j] = zmul(V[(size_t)j * n + i], ph);
   }
+  // the largest component, the lowest index on ties
+  for (int o = 16; o > 0; o >>= 1) {
+    rank += __shfl_xor_sync(0xffffffffu, rank, o);
+    nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
+    const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+    const int ok = __shfl_xor_sync(0xffffffffu, kmax, o);
+    if (ob > best || (ob == best && ok < kmax)) {
+      best = ob;
+      kmax = ok;
+    }
+  }
+  if ((t & 31) == 0) {
+    sb[t >> 5] = best;
+    sn[t >> 5] = nrm;
+    sk[t >> 5] = kmax;
+    sr[t >> 5] = rank;
+  }
+  __syncthreads();
+  rank = 0;
+  nrm = 0.0;
+  best = -1.0;
+  kmax = n;
+  for (int w = 0; w < NW; ++w) {
+    rank += sr[w];
+    nrm += sn[w];
+    if (sb[w] > best || (sb[w] == best && sk[w] < kmax)) {
+      best = sb[w];
+      kmax = sk[w];
+    }
+  }
+  if (kmax >= n) kmax = 0;                                           // every component NaN
+  const double2 vk = V[(size_t)kmax * n + i];
+  const double mag = sqrt(best);
+  const double sc = 1.0 / (mag * sqrt(nrm));
+  const double2 ph = make_double2(vk.x * sc, -vk.y * sc);
+  if (t == 0) eig[rank] = li;
+  for (int j = t; j < n; j += SV_THREADS) Vt[(size_t)rank * n + j] = zmul(V[(size_t)j * n + i], ph);
 }
 
 }  // namespace
 
 template <typename T>
 void gemm_cn(const cplx<T>* A, int lda, const cplx<T>* B, int ldb, int m, int n, int K, double2* part,
-             size_t part_elems, double2* out, cudaStream_t s) {
+             size_t part_elems, double2* out, cudaStream_t s, float2* out32) {
   const int tm = (m + GT - 1) / GT, tn = (n + GT - 1) / GT;
   int ks = std::max(1, 304 / (tm * tn));
   ks = std::min(ks, std::max(1, K / 256));
@@ -561,16 +509,16 @@ void gemm_cn(const cplx<T>* A, int lda, const cplx<T>* B, int ldb, int m, int n,
   k_gemm_cn<T><<<g, 256, 0, s>>>(A, lda, B, ldb, m, n, K, kchunk, part);
   KS_CHECK_LAUNCH();
   const size_t mn = (size_t)m * n;
-  k_reduce_parts<<<(unsigned)std::min<size_t>((mn + 255) / 256, 1024), 256, 0, s>>>(part, ks, mn, out);
+  k_reduce_parts<<<(unsigned)std::min<size_t>((mn + 255) / 256, 1024), 256, 0, s>>>(part, ks, mn, out, out32);
   KS_CHECK_LAUNCH();
 }
 
-template <typename T>
-void rotate(const double2* M, int nin, const cplx<T>* X, const cplx<T>* X2, int nin1, int ldx, cplx<T>* Y, int ldy,
+template <typename T, typename MC>
+void rotate(const MC* M, int nin, const cplx<T>* X, const cplx<T>* X2, int nin1, int ldx, cplx<T>* Y, int ldy,
             int m, int K, cudaStream_t s) {
   if (!X2) nin1 = nin;
   dim3 g((K + 63) / 64, (m + 31) / 32);
-  k_rotate<T><<<g, 256, 0, s>>>(M, nin, X, X2, nin1, ldx, Y, ldy, m, K);
+  k_rotate<T, MC><<<g, 256, 0, s>>>(M, nin, X, X2, nin1, ldx, Y, ldy, m, K);
   KS_CHECK_LAUNCH();
 }
 
@@ -590,30 +538,12 @@ void cholesky_inverse_tol(double2* A, double2* M, int n, double tol, int* status
   KS_CHECK_LAUNCH();
 }
 
-void eigh_jacobi_mixed(const double2* A, double2* V, double* lam, double* eig, double2* Vt, float2* work, int n,
-                       cudaStream_t s) {
-  if (n > 256 || n < 1) fail(KS_ERR_ARG, "eigh_jacobi_mixed: n=%d not in [1, 256]", n);
-  const size_t nn = (size_t)n * n;
-  float2* A32 = work;
-  float2* V32 = work + nn;
-  const unsigned nb = (unsigned)std::min<size_t>((nn + 255) / 256, 1024);
-  k_c128_to_c64<<<nb, 256, 0, s>>>(A, A32, nn);
-  KS_CHECK_LAUNCH();
-  k_jacobi32<<<1, 1024, 0, s>>>(A32, V32, n);
-  KS_CHECK_LAUNCH();
-  k_c64_to_c128<<<nb, 256, 0, s>>>(V32, V, nn);
-  KS_CHECK_LAUNCH();
+void eigh_mixed(const double2* A, double2* V, double* lam, double* eig, double2* Vt, void* work, int n,
+                cudaStream_t s) {
+  eigh_vectors_f32(A, V, n, work, Vt, s);                              // Vt is scratch until the sort
   k_rayleigh_quotients<<<n, 256, 0, s>>>(A, V, n, lam);
   KS_CHECK_LAUNCH();
-  k_sort_vectors<<<1, 128, 0, s>>>(lam, V, n, eig, Vt);
-  KS_CHECK_LAUNCH();
-}
-
-void eigh_mixed(const double2* A, double2* V, double* lam, double* eig, double2* Vt, int n, cudaStream_t s) {
-  eigh_householder_f32(A, V, n, s);
-  k_rayleigh_quotients<<<n, 256, 0, s>>>(A, V, n, lam);
-  KS_CHECK_LAUNCH();
-  k_sort_vectors<<<1, 128, 0, s>>>(lam, V, n, eig, Vt);
+  k_sort_vectors<<<n, SV_THREADS, 0, s>>>(lam, V, n, eig, Vt);
   KS_CHECK_LAUNCH();
 }
 
@@ -638,12 +568,14 @@ void jacobi_eigh(double2* A, double2* V, double* eig, double2* Vt, int n, cudaSt
 }
 
 template void gemm_cn<float>(const float2*, int, const float2*, int, int, int, int, double2*, size_t, double2*,
-                             cudaStream_t);
+                             cudaStream_t, float2*);
 template void gemm_cn<double>(const double2*, int, const double2*, int, int, int, int, double2*, size_t, double2*,
-                              cudaStream_t);
-template void rotate<float>(const double2*, int, const float2*, const float2*, int, int, float2*, int, int, int,
-                            cudaStream_t);
-template void rotate<double>(const double2*, int, const double2*, const double2*, int, int, double2*, int, int, int,
-                             cudaStream_t);
+                              cudaStream_t, float2*);
+template void rotate<float, double2>(const double2*, int, const float2*, const float2*, int, int, float2*, int, int,
+                                     int, cudaStream_t);
+template void rotate<float, float2>(const float2*, int, const float2*, const float2*, int, int, float2*, int, int,
+                                    int, cudaStream_t);
+template void rotate<double, double2>(const double2*, int, const double2*, const double2*, int, int, double2*, int,
+                                      int, int, cudaStream_t);
 
 }  // namespace ks

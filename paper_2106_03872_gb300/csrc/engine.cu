@@ -303,7 +303,7 @@ template <typename T> class Engine final : public EngineBase {
     }
     // ---- dense LA
     const size_t nn = (size_t)ns_ * ns_;
-    part_elems_ = std::max<size_t>(nn * 8, 4096);
+    part_elems_ = std::max<size_t>(nn * (small_block() ? 304 : 8), 4096);
     if (use_tc()) {
       part_elems_ = std::max(part_elems_, tc_overlap_part_elems(ns_, ns_));
       rotws_bytes_ = tc_rotation_workspace_bytes(ns_, 2 * ns_);
@@ -320,6 +320,7 @@ template <typename T> class Engine final : public EngineBase {
     mCat_ = alloc<double2>(2 * nn);
     eig_ = alloc<double>(ns_);
     lam_ = alloc<double>(ns_);
+    if (mixed_eigh()) ehw_ = arena_.alloc(eigh_workspace(ns_));
     if (mixed_cholesky()) chw_ = alloc<double2>(cholesky_mixed_workspace(ns_));
     if (fused_rr()) {
       hraw32_ = alloc<float2>(nn);
@@ -603,9 +604,9 @@ template <typename T> class Engine final : public EngineBase {
     //    Mcat = [(I + alpha Lambda) C | -alpha C] run on the side stream (one SM), while
     //  - the main stream applies H to H psi (H^2 psi);
     //  - then psi <- Mcat [psi; H psi] and H psi <- Mcat [H psi; H^2 psi].
-    // On the bf16x3 path with n <= 128 the side stream's Rayleigh-Ritz step is one CTA
-    // (rr_step_mixed: subspace matrix, eigenpairs, C and Mcat in FP32, rows in ascending order
-    // of the FP32 eigenvalues); the reported FP64 Rayleigh quotients follow on the side
+    // On the mixed path with n <= 128 the side stream's Rayleigh-Ritz step runs in FP32
+    // (rr_step_mixed: subspace matrix, eigenpairs, C and Mcat, rows in ascending order of the
+    // FP32 eigenvalues); the reported FP64 Rayleigh quotients follow on the side
     // stream while the main stream rotates.
     // H psi enters the next iteration without a new application of H to psi; it is recomputed
     // directly on entry to a call whose block changed and every HPSI_REFRESH iterations.
@@ -637,9 +638,9 @@ template <typename T> class Engine final : public EngineBase {
       if (frr) {
         {
           ProfScope p(prof, "rr_step", aux_);
-          rr_step_mixed(hraw32_, m32_, alpha, n, mcat32_, aexp_, vexp_, perm_, aux_);
+          rr_step_mixed(hraw32_, m32_, alpha, n, mcat32_, aexp_, vexp_, perm_, ehw_, aux_);
         }
-        {
+        if (use_tc()) {
           ProfScope p(prof, "rot_prep", aux_);
           tc_rotate_prepare(mcat32_, n, 2 * n, rotws_, rotws_bytes_, aux_);
         }
@@ -1425,24 +1426,28 @@ template <typename T> class Engine final : public EngineBase {
       if (buf_[i] != a && buf_[i] != b) return buf_[i];
     fail(KS_ERR_STATE, "internal: no spare state buffer");
   }
-  bool use_tc() const { return sizeof(T) == 4 && prec_ == KS_MIXED_BF16X3; }
+  // Blocks of at most 16 states take the CUDA-core FP32 overlap and rotation instead of the
+  // tensor-core kernels: an eighth of a 128-row operand tile would be states, and the unsplit FP32
+  // products are exact to 24 bits where the split ones carry 16 (an orthonormalised block of 7 states
+  // is off by 5e-6 with them).
+  static constexpr int SMALL_BLOCK = 16;
+  bool small_block() const { return sizeof(T) == 4 && ns_ <= SMALL_BLOCK; }
+  bool use_tc() const { return sizeof(T) == 4 && prec_ == KS_MIXED_BF16X3 && !small_block(); }
   bool mixed_cholesky() const { return sizeof(T) == 4 && ns_ <= 256; }
-  // the mixed path's FP32 eigensolver: one-CTA Householder for n <= 128, one-CTA FP32 Jacobi up
-  // to 256 (both finished by FP64 Rayleigh quotients); FP64 Jacobi beyond, or with
-  // KS_OPT_FP64_SUBSPACE
+  bool mixed_eigh() const { return sizeof(T) == 4 && ns_ <= 256; }
+  // the mixed path's FP32 Householder eigensolver up to 256 states (finished by FP64 Rayleigh
+  // quotients); FP64 Jacobi beyond, or with KS_OPT_FP64_SUBSPACE
   void eigh_sub(int n, double2* Vt, cudaStream_t s) {
-    if (sizeof(T) == 4 && !fp64_subspace_ && n <= 128)
-      eigh_mixed(mA_, mV_, lam_, eig_, Vt, n, s);
-    else if (sizeof(T) == 4 && !fp64_subspace_ && n <= 256)
-      eigh_jacobi_mixed(mA_, mV_, lam_, eig_, Vt, reinterpret_cast<float2*>(mF_), n, s);
+    if (mixed_eigh() && !fp64_subspace_)
+      eigh_mixed(mA_, mV_, lam_, eig_, Vt, ehw_, n, s);
     else
       jacobi_eigh(mA_, mV_, eig_, Vt, n, s);
   }
   // KS_OPT_FP64_SUBSPACE on a mixed handle: the Cholesky factor of S, the subspace products and
   // the Rayleigh-Ritz eigensolver in FP64 (as on the FP64 path), the states and their GEMMs mixed
   bool fp64_subspace_ = false;
-  // the block iteration's Rayleigh-Ritz step runs in one CTA (rr_step_mixed)
-  bool fused_rr() const { return use_tc() && ns_ <= 128; }
+  // the block iteration's Rayleigh-Ritz step runs in FP32 (rr_step_mixed)
+  bool fused_rr() const { return sizeof(T) == 4 && ns_ <= 128; }
 
   // out = A^H B over the sphere (n x n), tensor cores on the bf16x3 mixed path
   void overlap(const C* A, const C* B, int n, double2* out, cudaStream_t s, float2* out32 = nullptr) {
@@ -1452,7 +1457,7 @@ template <typename T> class Engine final : public EngineBase {
         return;
       }
     }
-    gemm_cn<T>(A, g_.nG, B, g_.nG, n, n, g_.nG, part_, part_elems_, out, s);
+    gemm_cn<T>(A, g_.nG, B, g_.nG, n, n, g_.nG, part_, part_elems_, out, s, out32);
   }
 
   // Y = M X (rows of states); with X2, M is n x 2n and X = [X; X2]
@@ -1464,14 +1469,18 @@ template <typename T> class Engine final : public EngineBase {
         return;
       }
     }
-    rotate<T>(M, nin, X, X2, ns_, g_.nG, Y, g_.nG, ns_, g_.nG, s);
+    rotate<T, double2>(M, nin, X, X2, ns_, g_.nG, Y, g_.nG, ns_, g_.nG, s);
   }
 
-  // Y = Mcat [X; X2] from the split image of mcat32_ that tc_rotate_prepare left in rotws_
+  // Y = Mcat [X; X2] from the split image of mcat32_ that tc_rotate_prepare left in rotws_ (small
+  // blocks: from mcat32_ itself)
   void rot_prepared(const C* X, const C* X2, C* Y, cudaStream_t s) {
-    if constexpr (std::is_same<T, float>::value)
-      tc_rotate_prepared(rotws_, 2 * ns_, X, X2, ns_, g_.nG, Y, g_.nG, ns_, g_.nG, status_ + 1, s);
-    else
+    if constexpr (std::is_same<T, float>::value) {
+      if (use_tc())
+        tc_rotate_prepared(rotws_, 2 * ns_, X, X2, ns_, g_.nG, Y, g_.nG, ns_, g_.nG, status_ + 1, s);
+      else
+        rotate<float, float2>(mcat32_, 2 * ns_, X, X2, ns_, g_.nG, Y, g_.nG, ns_, g_.nG, s);
+    } else
       fail(KS_ERR_STATE, "internal: prepared rotation on the FP64 path");
   }
 
@@ -1529,6 +1538,7 @@ template <typename T> class Engine final : public EngineBase {
   double2 *mS_ = nullptr, *mA_ = nullptr, *mM_ = nullptr, *mV_ = nullptr;
   double* eig_ = nullptr;
   double* lam_ = nullptr;
+  void* ehw_ = nullptr;      // workspace of the FP32 eigensolver
   double2* chw_ = nullptr;   // two-pass FP32 Cholesky workspace (mixed path)
   double2 *mT_ = nullptr, *mC_ = nullptr, *mF_ = nullptr;   // subspace products, FP64 factor scratch
   double2* mCat_ = nullptr;                                   // [n][2n] steepest-descent step matrix

@@ -134,13 +134,15 @@ template <typename T> void real_to_double(const T* in, double* out, size_t n, cu
 
 // ---- dense linear algebra (dense.cu) ----------------------------------------------------------
 // out[i][j] = sum_k conj(A[i][k]) B[j][k] for i < m, j < n (row-major, FP64 out); split-K with
-// deterministic reduction through `part` (>= gemm_cn_parts(...) double2 elements).
+// deterministic reduction through `part` (>= gemm_cn_parts(...) double2 elements); out32, when given,
+// receives an FP32 copy.
 template <typename T> void gemm_cn(const cplx<T>* A, int lda, const cplx<T>* B, int ldb, int m, int n, int K,
-                                   double2* part, size_t part_elems, double2* out, cudaStream_t s);
+                                   double2* part, size_t part_elems, double2* out, cudaStream_t s,
+                                   float2* out32 = nullptr);
 // Y[i][k] = sum_j M[i][j] X[j][k], i < m, j < nin, k < K; rows j >= nin1 of X come from X2
 // (row j - nin1) when X2 is non-NULL.  Y must not overlap X or X2.
-template <typename T> void rotate(const double2* M, int nin, const cplx<T>* X, const cplx<T>* X2, int nin1, int ldx,
-                                  cplx<T>* Y, int ldy, int m, int K, cudaStream_t s);
+template <typename T, typename MC> void rotate(const MC* M, int nin, const cplx<T>* X, const cplx<T>* X2, int nin1,
+                                               int ldx, cplx<T>* Y, int ldy, int m, int K, cudaStream_t s);
 // A := (A + A^H)/2
 void hermitize(double2* A, int n, cudaStream_t s);
 // C = opA(A) opB(B), n x n complex128 (row-major); flags: 1 conj(A), 2 B transposed, 4 conj(B).
@@ -154,7 +156,7 @@ void sd_matrix(const double2* C, const double* eig, double alpha, int n, double2
 void cholesky_inverse(double2* A, double2* M, int n, int* status, cudaStream_t s);
 // Same with an explicit relative pivot tolerance (pivot <= tol * S_jj fails).
 void cholesky_inverse_tol(double2* A, double2* M, int n, double tol, int* status, cudaStream_t s);
-// Mixed path (n <= 160): M = conj(L^{-1}) for S = L L^H from an FP32 Cholesky pass, refined
+// Mixed path (n <= 256): M = conj(L^{-1}) for S = L L^H from an FP32 Cholesky pass, refined
 // by FP64 triangular products when `refine` (cholqr_mixed.cu); work holds
 // cholesky_mixed_workspace(n) complex128.  M32, when given, receives an FP32 copy of M.
 // Same status convention as cholesky_inverse.
@@ -164,24 +166,22 @@ void cholesky_inverse_mixed(const double2* S, double2* M, int n, double tol, dou
 // Hermitian eigen-decomposition of A (destroyed) by cyclic Jacobi; eig ascending, rows of
 // Vt = eigenvectors (largest-magnitude component real positive).  `V` is n*n workspace.
 void jacobi_eigh(double2* A, double2* V, double* eig, double2* Vt, int n, cudaStream_t s);
-// Householder + bisection + twisted-factorization eigenvectors, FP32, one CTA (n <= 128):
-// V (n x n complex128, columns = eigenvectors, unsorted).
-void eigh_householder_f32(const double2* A, double2* V, int n, cudaStream_t s);
-// Mixed path (n <= 128): eigh_householder_f32 on the FP64 Hermitian A (kept), eigenvalues =
-// FP64 Rayleigh quotients of the FP32 vectors on A; same outputs as jacobi_eigh.
-// V is n*n workspace, lam n doubles of workspace.
-void eigh_mixed(const double2* A, double2* V, double* lam, double* eig, double2* Vt, int n, cudaStream_t s);
-// Mixed path for 128 < n <= 256: FP32 parallel Jacobi on a copy of A (one CTA, matrix in
-// global memory), eigenvalues = FP64 Rayleigh quotients of the FP32 vectors on A; same outputs
-// as eigh_mixed.  work: 2 n^2 complex64.
-void eigh_jacobi_mixed(const double2* A, double2* V, double* lam, double* eig, double2* Vt, float2* work, int n,
-                       cudaStream_t s);
-// Rayleigh-Ritz step of the mixed block iteration in one CTA (n <= 128), FP32 in and out:
-// H_sub = conj(M) Hraw M^T (Hermitian part, exported to Aout), its eigenpairs, C = Vt M and
+// Householder + bisection + twisted-factorisation eigenvectors, FP32 (n <= 256, eigh.cu): V (n x n
+// complex128, columns = eigenvectors, unsorted).  work: eigh_workspace(n) bytes, work2: 2 n^2 floats.
+size_t eigh_workspace(int n);
+void eigh_vectors_f32(const double2* A, double2* V, int n, void* work, void* work2, cudaStream_t s);
+// Mixed path (n <= 256): eigh_vectors_f32 on the FP64 Hermitian A (kept), eigenvalues = FP64 Rayleigh
+// quotients of the FP32 vectors on A; same outputs as jacobi_eigh.  V is n*n workspace, lam n doubles
+// of workspace, work eigh_workspace(n) bytes.
+void eigh_mixed(const double2* A, double2* V, double* lam, double* eig, double2* Vt, void* work, int n,
+                cudaStream_t s);
+// Rayleigh-Ritz step of the mixed block iteration (n <= 128), FP32 in and out: H_sub = conj(M) Hraw M^T
+// (exported to Aout; its Hermitian part is decomposed), its eigenpairs, C = Vt M and
 // Mcat = [(I + alpha Lambda) C | -alpha C] (n x 2n) with rows in ascending eigenvalue order;
-// Vout holds the eigenvectors as columns in solver order and perm their ranks.
+// Vout holds the eigenvectors as columns in solver order and perm their ranks.  work:
+// eigh_workspace(n) bytes.
 void rr_step_mixed(const float2* Hraw, const float2* M, double alpha, int n, float2* Mcat, float2* Aout,
-                   float2* Vout, int* perm, cudaStream_t s);
+                   float2* Vout, int* perm, void* work, cudaStream_t s);
 // eig[perm[j]] = FP64 Rayleigh quotient of column j of V on A (outputs of rr_step_mixed).
 void ritz_values(const float2* A, const float2* V, const int* perm, int n, double* eig, cudaStream_t s);
 
