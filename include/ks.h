@@ -140,7 +140,7 @@ ks_status ks_density(ks_grid g, void* n_dev, void* stream);
 
 /* CholQR of the resident states (Sec. "Ground-state solution", orthogonalisation):
  * S = Psi^H Psi, S = L L^H, Psi <- Psi L^{-H}.  KS_FP64 factors S in FP64; the mixed
- * paths (nstates <= 160) take one FP32 Cholesky factor and inverse, refined to first order
+ * paths (nstates <= 256) take one FP32 Cholesky factor and inverse, refined to first order
  * with the FP64 triangular product L1^{-1} S L1^{-H}.
  * S_host_opt (may be NULL) receives S, [nstates][nstates] complex128 row-major,
  * S_ij = sum_G conj(c_iG) c_jG.  KS_ERR_NOT_POSDEF if S is not positive definite

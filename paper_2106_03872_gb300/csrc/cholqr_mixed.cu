@@ -1,10 +1,10 @@
 // Mixed-path CholQR factor (Sec. "Ground-state solution": orthonormalisation of the block by
 // the Cholesky factor of its overlap S = Psi^H Psi, Psi <- Psi L^{-H}).
 //
-// The FP64 factorisation of an n <= 160 matrix in one CTA is bound by GB300's FP64 rate, so
+// The FP64 factorisation of an n <= 256 matrix in one CTA is bound by GB300's FP64 rate, so
 // the factor comes from one FP32 pass refined in FP64:
 //
-//   1. L1 L1^H = S       FP32 Cholesky in shared memory, M1 = L1^{-1}        (one CTA)
+//   1. L1 L1^H = S       FP32 elimination in registers, M1 = L1^{-1}  (one CTA, a cluster from n = 129)
 //   2. S2 = M1 S M1^H    FP64 triangular products, S2 = I + E with |E| ~ eps_32 kappa(S)
 //   3. M = conj((I - Phi(E)) M1), Phi(E) = strictly lower part of E plus half its diagonal
 //
@@ -17,6 +17,8 @@
 // sqrt(n).  The pipelined block iteration takes that form: it uses only the FP32 copy of M,
 // whose rounding is of the order of the refinement's correction for the well-conditioned S of
 // an iterate, and the next iteration's CholQR starts again from the S of the new block.
+#include <cooperative_groups.h>
+
 #include <type_traits>
 
 #include "kernels.h"
@@ -25,239 +27,163 @@ namespace ks {
 
 namespace {
 
-constexpr int C32_MAXN = 160;          // square array in shared memory
-constexpr int C32_MAXN_GLOBAL = 256;   // square array in global memory
-constexpr int C32_THREADS = 1024;
-
-// One CTA.  Reads the lower triangle of S (n x n, row-major), writes X = L^{-1} (lower,
-// zeros above; conj(X) when conj_out) to Out, and an FP32 copy to Out32 when it is given.
-//
-// Shared memory holds one square [n][ld] array: L_rc (r >= c) at [c][r] (column-major, so
-// lanes running along a column touch consecutive words) and X_rc (r > c) at [r][c], i.e. in
-// the unused upper triangle; X's diagonal is a separate vector.  Blocked by CB columns, each
-// block step three barriers:
-//   (a) warp 0 factors the diagonal block in registers (lane = row, the pivot column is
-//       broadcast by shuffles) and inverts it in registers;
-//   (b) panel L_iJ = A_iJ W_J^H for the rows below (all threads);
-//   (c) trailing update A_ik -= sum_{c in J} L_ic conj(L_kc) (warps over columns k, lanes
-//       over rows i; conj(L_kJ) held in registers).
-// Then the off-diagonal blocks of X by block rows I: T_IJ = sum_{K=J}^{I-1} L_IK X_KJ,
-// X_IJ = -W_I T_IJ for all J < I at once.
-constexpr int CB = 8;
+constexpr int C32_MAXN = 256;
 
 __device__ __forceinline__ float2 c_mul(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
-__device__ __forceinline__ float2 c_mulc(float2 a, float2 b) {   // a * conj(b)
-  return make_float2(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
-}
-__device__ __forceinline__ float2 shfl2(float2 v, int src) {
-  return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
-}
 
-// MAXN: the largest n; GLB: the square array lives in global memory (gU, n (n + 1) values,
-// L2-resident) instead of shared memory, for n beyond what shared memory holds (160 < n <= 256).
-template <int MAXN, bool GLB>
-__global__ void __launch_bounds__(C32_THREADS, 1)
+// X = L^{-1} of S = L L^H by elimination on the rows of [S | I], in place: after step j columns <= j of
+// a row i > j hold its part of L_1^{-1} (L_1 unit lower triangular, S = L_1 D L_1^H) and columns > j the
+// reduced matrix, so step j is row_i -= (A_ij / d_j) row_j in all columns but j, which becomes
+// -A_ij / d_j.  X = D^{-1/2} L_1^{-1}.  A pivot d_j <= tol S_jj sets status = j + 1.
+//
+// n dependent steps bound it, so a step is one barrier: the matrix is in registers (row i in CTA
+// i mod CL, NR rows a warp, a lane's columns lane + 32 q), and the owner of row j + 1 hands it over in
+// shared memory as soon as it has updated it (in a cluster, the other CTAs fetch it from there).  The
+// blocked factorisation in shared memory that this replaces kept 8 columns of pivots in one warp,
+// three barriers a block, then a second sweep for the inverse: 0.21 ms at n = 128 against 0.11 ms.  With
+// the FP64 refinement the factor takes 0.07, 0.18 and 0.35 ms at n = 64, 128 and 200 (0.096, 0.28 and
+// 0.79 ms before).
+template <int CL, int THREADS, int MAXN> struct Chol {
+  static constexpr int Q = MAXN / 32, NWARP = THREADS / 32, NR = MAXN / CL / NWARP;
+  struct Shared {
+    float2 p[2][MAXN];      // row j at [j & 1] (CL > 1: this CTA's rows)
+    float2 pc[2][MAXN];     // CL > 1: the fetched row
+    float sjj[MAXN], d[MAXN];
+  };
+  Shared& sh;
+  int n, rank, lane, warp, bad = 0;
+  float tol;
+  float2 A[NR][Q];
+
+  __device__ __forceinline__ int row(int r) const { return (warp + r * NWARP) * CL + rank; }
+  __device__ __forceinline__ Chol(Shared& s, int n_, float tol_) : sh(s), n(n_), tol(tol_) {
+    lane = threadIdx.x & 31;
+    warp = threadIdx.x >> 5;
+    rank = 0;
+    if constexpr (CL > 1) rank = (int)cooperative_groups::this_cluster().block_rank();
+  }
+
+  // Steps j in column slot Q1.
+  template <int Q1> __device__ __forceinline__ void slot_steps() {
+    const int j1 = min(32 * Q1 + 32, n);
+    for (int j = 32 * Q1; j < j1; ++j) {
+      const int b = j & 1;
+      float2* src = sh.p[b];
+      if constexpr (CL > 1) {
+        namespace cg = cooperative_groups;
+        cg::cluster_group cl = cg::this_cluster();
+        cl.sync();
+        if (threadIdx.x < MAXN) sh.pc[b][threadIdx.x] = cl.map_shared_rank(&sh.p[0][0], j % CL)[b * MAXN + threadIdx.x];
+        src = sh.pc[b];
+      }
+      __syncthreads();
+      float2 p[Q];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) p[q] = src[lane + 32 * q];
+      const float d = src[j].x;
+      if (!(d > tol * sh.sjj[j]) || !isfinite(d)) {                  // uniform
+        bad = j + 1;
+        return;
+      }
+      const float inv = __frcp_rn(d);
+      if (threadIdx.x == 0) sh.d[j] = d;
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const int i = row(r);
+        if (i > j) {                                                 // warp-uniform
+          const float2 l = make_float2(inv * __shfl_sync(0xffffffffu, A[r][Q1].x, j & 31),
+                                       inv * __shfl_sync(0xffffffffu, A[r][Q1].y, j & 31));
+#pragma unroll
+          for (int q = 0; q < Q; ++q) {
+            float2 m = A[r][q];
+            m.x = fmaf(-l.x, p[q].x, fmaf(l.y, p[q].y, m.x));
+            m.y = fmaf(-l.x, p[q].y, fmaf(-l.y, p[q].x, m.y));
+            if (q == Q1 && lane == (j & 31)) m = make_float2(-l.x, -l.y);
+            A[r][q] = m;
+          }
+          if (i == j + 1)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) sh.p[b ^ 1][lane + 32 * q] = A[r][q];
+        }
+      }
+    }
+    if constexpr (Q1 + 1 < Q) {
+      if (n > 32 * Q1 + 32) slot_steps<Q1 + 1>();
+    }
+  }
+
+  __device__ __forceinline__ void run(const double2* __restrict__ S, int conj_out, int* __restrict__ status,
+                                      double2* __restrict__ Out, float2* __restrict__ Out32) {
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const int i = row(r), j = lane + 32 * q;
+        A[r][q] = make_float2(0.f, 0.f);
+        if (i < n && j < n) {
+          // the lower triangle, mirrored
+          const double2 v = S[i >= j ? (size_t)i * n + j : (size_t)j * n + i];
+          A[r][q] = make_float2((float)v.x, i == j ? 0.f : (i > j ? (float)v.y : -(float)v.y));
+        }
+      }
+    for (int j = threadIdx.x; j < n; j += THREADS) sh.sjj[j] = (float)S[(size_t)j * n + j].x;
+    if (warp == 0 && rank == 0)
+#pragma unroll
+      for (int q = 0; q < Q; ++q) sh.p[0][lane + 32 * q] = A[0][q];
+    slot_steps<0>();
+    if constexpr (CL > 1) cooperative_groups::this_cluster().sync();   // no CTA leaves while its rows are read
+    __syncthreads();                                                 // d
+    const float sgn = conj_out ? -1.f : 1.f;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const int i = row(r);
+      if (i >= n) continue;
+      const float f = bad ? 1.f : 1.f / sqrtf(sh.d[i]);
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const int j = lane + 32 * q;
+        if (j >= n) continue;
+        float2 x = make_float2(0.f, 0.f);
+        if (i == j)
+          x.x = f;
+        else if (j < i && !bad)
+          x = make_float2(f * A[r][q].x, f * A[r][q].y);
+        Out[(size_t)i * n + j] = make_double2((double)x.x, (double)(sgn * x.y));
+        if (Out32) Out32[(size_t)i * n + j] = make_float2(x.x, sgn * x.y);
+      }
+    }
+    if (bad && rank == 0 && threadIdx.x == 0) atomicCAS(status, 0, bad);
+  }
+};
+
+// Writes X = L^{-1} (lower, zeros above; conj(X) when conj_out) of the Hermitian S (n x n, row-major,
+// its lower triangle is read) to Out, and an FP32 copy to Out32 when it is given; the identity when S is
+// not positive definite.
+template <int CL, int THREADS, int MAXN>
+__global__ void __launch_bounds__(THREADS, 1)
     k_chol32_inverse(const double2* __restrict__ S, int n, double tol, int conj_out, int* __restrict__ status,
-                     double2* __restrict__ Out, float2* __restrict__ Out32, float2* __restrict__ gU) {
-  extern __shared__ float2 c32[];
-  const int ld = n + 1;
-  float2* U = GLB ? gU : c32;
-  __shared__ float sjj[MAXN];
-  __shared__ float2 xd[MAXN];                                        // diagonal of X
-  __shared__ int s_bad;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  constexpr int NW = C32_THREADS / 32;
-#define UL(r, c) U[(c) * ld + (r)]
-#define XU(r, c) U[(r) * ld + (c)]
-#define XL(r, c) ((r) == (c) ? xd[r] : XU(r, c))
+                     double2* __restrict__ Out, float2* __restrict__ Out32) {
+  using C = Chol<CL, THREADS, MAXN>;
+  __shared__ typename C::Shared sh;
+  C c(sh, n, (float)tol);
+  c.run(S, conj_out, status, Out, Out32);
+}
 
-  for (int e = t; e < n * n; e += C32_THREADS) {
-    const int r = e / n, c = e - (e / n) * n;
-    if (c <= r) {
-      const double2 v = S[e];
-      UL(r, c) = make_float2((float)v.x, r == c ? 0.f : (float)v.y);
-    }
-  }
-  for (int j = t; j < n; j += C32_THREADS) sjj[j] = (float)S[(size_t)j * n + j].x;
-  if (t == 0) s_bad = 0;
-  __syncthreads();
-
-  for (int J = 0; J < n; J += CB) {
-    const int jb = min(CB, n - J), J1 = J + jb;
-    // (a) diagonal block in warp 0's registers: lane r holds row J + r
-    if (warp == 0) {
-      float2 a[CB];
-#pragma unroll
-      for (int c = 0; c < CB; ++c) a[c] = (c <= lane && lane < jb) ? UL(J + lane, J + c) : make_float2(0.f, 0.f);
-      int bad = 0;
-#pragma unroll
-      for (int j = 0; j < CB; ++j) {
-        if (j < jb && !bad) {
-          const float d = __shfl_sync(0xffffffffu, a[j].x, j);
-          if (!(d > (float)tol * sjj[J + j]) || !isfinite(d)) {
-            bad = J + j + 1;
-          } else {
-            const float ljj = sqrtf(d), inv = 1.f / ljj;
-            if (lane == j) a[j] = make_float2(ljj, 0.f);
-            else if (lane > j) a[j] = make_float2(a[j].x * inv, a[j].y * inv);
-#pragma unroll
-            for (int k = j + 1; k < CB; ++k) {
-              const float2 lkj = shfl2(a[j], k);
-              if (k <= lane) {
-                const float2 p = c_mulc(a[j], lkj);
-                a[k].x -= p.x;
-                a[k].y -= p.y;
-              }
-            }
-          }
-        }
-      }
-      if (bad) {
-        if (lane == 0) s_bad = bad;
-      } else {
-#pragma unroll
-        for (int c = 0; c < CB; ++c)
-          if (c <= lane && lane < jb) UL(J + lane, J + c) = a[c];
-        // W = L_JJ^{-1} by rows: row j final after division by L_jj, rows r > j lose L_rj W_j
-        float2 w[CB];
-#pragma unroll
-        for (int c = 0; c < CB; ++c) w[c] = make_float2(c == lane ? 1.f : 0.f, 0.f);
-#pragma unroll
-        for (int j = 0; j < CB; ++j) {
-          if (j < jb) {
-            const float ij = 1.f / __shfl_sync(0xffffffffu, a[j].x, j);
-            if (lane == j) {
-#pragma unroll
-              for (int c = 0; c <= j; ++c) w[c] = make_float2(w[c].x * ij, w[c].y * ij);
-            }
-#pragma unroll
-            for (int c = 0; c <= j; ++c) {
-              const float2 wj = shfl2(w[c], j);
-              if (lane > j) {
-                const float2 p = c_mul(a[j], wj);
-                w[c].x -= p.x;
-                w[c].y -= p.y;
-              }
-            }
-          }
-        }
-        if (lane < jb) {
-#pragma unroll
-          for (int c = 0; c < CB; ++c) {
-            if (c < lane) XU(J + lane, J + c) = w[c];
-            else if (c == lane) xd[J + lane] = w[c];
-          }
-        }
-      }
-    }
-    __syncthreads();
-    if (s_bad) break;                                                // uniform
-    const int rows = n - J1;
-    if (rows == 0) break;
-    // (b) panel: L_ic = sum_{k=J}^{c} A_ik conj(W_ck); lanes run along i
-    float2 pv[(MAXN * CB + C32_THREADS - 1) / C32_THREADS];
-#pragma unroll
-    for (int q = 0; q < (MAXN * CB + C32_THREADS - 1) / C32_THREADS; ++q) {
-      const int idx = t + q * C32_THREADS;
-      pv[q] = make_float2(0.f, 0.f);
-      if (idx < rows * jb) {
-        const int i = J1 + idx % rows, c = J + idx / rows;
-        for (int k = J; k <= c; ++k) {
-          const float2 p = c_mulc(UL(i, k), XL(c, k));
-          pv[q].x += p.x;
-          pv[q].y += p.y;
-        }
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < (MAXN * CB + C32_THREADS - 1) / C32_THREADS; ++q) {
-      const int idx = t + q * C32_THREADS;
-      if (idx < rows * jb) UL(J1 + idx % rows, J + idx / rows) = pv[q];
-    }
-    __syncthreads();
-    // (c) trailing update, columns k >= J1
-    for (int k = J1 + warp; k < n; k += NW) {
-      float2 lk[CB];
-#pragma unroll
-      for (int c = 0; c < CB; ++c) {
-        const float2 v = c < jb ? UL(k, J + c) : make_float2(0.f, 0.f);
-        lk[c] = make_float2(v.x, -v.y);
-      }
-      for (int i = k + lane; i < n; i += 32) {
-        float2 acc = make_float2(0.f, 0.f);
-        const float2* col = U + J * ld + i;                          // col[c * ld] = L_{i, J+c}
-#pragma unroll
-        for (int c = 0; c < CB; ++c) {
-          if (c < jb) {
-            const float2 p = c_mul(col[c * ld], lk[c]);
-            acc.x += p.x;
-            acc.y += p.y;
-          }
-        }
-        const float2 v = UL(i, k);
-        UL(i, k) = make_float2(v.x - acc.x, v.y - acc.y);
-      }
-    }
-    __syncthreads();
-  }
-  if (s_bad) {
-    for (int e = t; e < n * n; e += C32_THREADS) {
-      const bool diag = e / n == e % n;
-      Out[e] = make_double2(diag ? 1.0 : 0.0, 0.0);
-      if (Out32) Out32[e] = make_float2(diag ? 1.f : 0.f, 0.f);
-    }
-    if (t == 0) atomicCAS(status, 0, s_bad);
-    return;
-  }
-  // off-diagonal blocks of X, block row by block row
-  for (int I0 = CB; I0 < n; I0 += CB) {
-    const int ib = min(CB, n - I0);
-    // T_rc = sum_{k=c}^{I0-1} L_rk X_kc into X(r, c), r in block row I, c < I0 (lanes along r)
-    for (int idx = t; idx < ib * I0; idx += C32_THREADS) {
-      const int r = I0 + idx % ib, c = idx / ib;
-      float2 acc = c_mul(UL(r, c), xd[c]);
-      for (int k = c + 1; k < I0; ++k) {
-        const float2 p = c_mul(UL(r, k), XU(k, c));
-        acc.x += p.x;
-        acc.y += p.y;
-      }
-      XU(r, c) = acc;
-    }
-    __syncthreads();
-    // X_rc = -sum_{r'=I0}^{r} W_I[r][r'] T_r'c
-    float2 xv[(CB * MAXN + C32_THREADS - 1) / C32_THREADS];
-#pragma unroll
-    for (int q = 0; q < (CB * MAXN + C32_THREADS - 1) / C32_THREADS; ++q) {
-      const int idx = t + q * C32_THREADS;
-      xv[q] = make_float2(0.f, 0.f);
-      if (idx < ib * I0) {
-        const int r = I0 + idx % ib, c = idx / ib;
-        for (int rp = I0; rp <= r; ++rp) {
-          const float2 p = c_mul(XL(r, rp), XU(rp, c));
-          xv[q].x -= p.x;
-          xv[q].y -= p.y;
-        }
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < (CB * MAXN + C32_THREADS - 1) / C32_THREADS; ++q) {
-      const int idx = t + q * C32_THREADS;
-      if (idx < ib * I0) XU(I0 + idx % ib, idx / ib) = xv[q];
-    }
-    __syncthreads();
-  }
-  const float sgn = conj_out ? -1.f : 1.f;
-  for (int e = t; e < n * n; e += C32_THREADS) {
-    const int r = e / n, c = e - (e / n) * n;
-    const float2 x = c <= r ? XL(r, c) : make_float2(0.f, 0.f);
-    Out[e] = make_double2((double)x.x, (double)(sgn * x.y));
-    if (Out32) Out32[e] = make_float2(x.x, sgn * x.y);
-  }
-#undef UL
-#undef XU
-#undef XL
+template <int CL, int THREADS, int MAXN>
+void launch_chol32(const double2* S, int n, double tol, int conj_out, int* status, double2* Out, float2* Out32,
+                   cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(CL);
+  cfg.blockDim = dim3(THREADS);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = CL;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  KS_CUDA(cudaLaunchKernelEx(&cfg, k_chol32_inverse<CL, THREADS, MAXN>, S, n, tol, conj_out, status, Out, Out32));
+  KS_CHECK_LAUNCH();
 }
 
 // Triangular products on 8 x 8 output tiles (64 threads, one output each), K staged through
@@ -274,8 +200,6 @@ __global__ void __launch_bounds__(64) k_tri_product(const double2* __restrict__ 
                                                     int n, const int* __restrict__ status, double2* __restrict__ C,
                                                     float2* __restrict__ C32) {
   constexpr int KC = 32;
-  __shared__ double2 As[8][KC + 1];
-  __shared__ double2 Bs[8][KC + 1];                                  // Bs[j][k]
   const int ty = threadIdx.x >> 3, tx = threadIdx.x & 7;
   const int I = blockIdx.y * 8, J = blockIdx.x * 8;
   const int i = I + ty, j = J + tx;
@@ -293,48 +217,42 @@ __global__ void __launch_bounds__(64) k_tri_product(const double2* __restrict__ 
     }
     return;
   }
-  // k range of the tile
+  // k range of the tile.  The triangles' zeros are stored (M1 above its diagonal) or set while the
+  // operands are staged (Phi), where MODE 2 also rounds them, so the products run without tests: the
+  // FP64 pipe (two lanes a clock per SM) takes four instructions per complex product.
   const int k0 = MODE == 2 ? J : 0;
   const int k1 = min(n, MODE == 0 ? J + 8 : I + 8);
   using R = typename std::conditional<MODE == 2, float, double>::type;
+  using C2 = cplx<R>;
+  __shared__ C2 As[8][KC + 1];
+  __shared__ C2 Bs[8][KC + 1];                                       // Bs[j][k]
   R re = 0, im = 0;
   for (int kc = k0; kc < k1; kc += KC) {
     for (int e = threadIdx.x; e < 8 * KC; e += 64) {
       const int r = e / KC, k = kc + e % KC;
-      As[r][e % KC] = (I + r < n && k < k1) ? A[(size_t)(I + r) * n + k] : make_double2(0.0, 0.0);
+      double2 a = make_double2(0.0, 0.0), b = a;
+      if (I + r < n && k < k1 && (MODE != 2 || k <= I + r)) a = A[(size_t)(I + r) * n + k];
+      if (MODE == 2 && k == I + r) a = make_double2(0.5 * (a.x - 1.0), 0.0);   // Phi_ii = (A_ii - 1) / 2
+      As[r][e % KC] = mk<C2>((R)a.x, (R)a.y);
       if (MODE == 0) {
-        Bs[r][e % KC] = (J + r < n && k < k1) ? B[(size_t)(J + r) * n + k] : make_double2(0.0, 0.0);
+        if (J + r < n && k < k1) b = B[(size_t)(J + r) * n + k];
+        Bs[r][e % KC] = mk<C2>((R)b.x, (R)b.y);
       } else {
         const int kk = kc + e / 8, jj = e % 8;                        // B rows k, columns J..J+7
-        Bs[jj][e / 8] = (kk < k1 && J + jj < n) ? B[(size_t)kk * n + J + jj] : make_double2(0.0, 0.0);
+        if (kk < k1 && J + jj < n) b = B[(size_t)kk * n + J + jj];
+        Bs[jj][e / 8] = mk<C2>((R)b.x, (R)b.y);
       }
     }
     __syncthreads();
     const int kend = min(KC, k1 - kc);
     for (int kk = 0; kk < kend; ++kk) {
-      const int k = kc + kk;
-      const double2 a = As[ty][kk], b = Bs[tx][kk];
-      if (MODE == 0) {
-        if (k <= j) {
-          re += a.x * b.x + a.y * b.y;
-          im += a.y * b.x - a.x * b.y;
-        }
-      } else if (MODE == 1) {
-        if (k <= i) {
-          re += a.x * b.x - a.y * b.y;
-          im += a.x * b.y + a.y * b.x;
-        }
+      const C2 a = As[ty][kk], b = Bs[tx][kk];
+      if (MODE == 0) {                                               // a conj(b)
+        re = fma(a.x, b.x, fma(a.y, b.y, re));
+        im = fma(a.y, b.x, fma(-a.x, b.y, im));
       } else {
-        if (k >= j && k <= i) {
-          R ax = (R)a.x, ay = (R)a.y;
-          if (k == i) {                                              // Phi_ii = (A_ii - 1) / 2
-            ax = (R)(0.5 * (a.x - 1.0));
-            ay = 0;
-          }
-          const R bx = (R)b.x, by = (R)b.y;
-          re += ax * bx - ay * by;
-          im += ax * by + ay * bx;
-        }
+        re = fma(a.x, b.x, fma(-a.y, b.y, re));
+        im = fma(a.x, b.y, fma(a.y, b.x, im));
       }
     }
     __syncthreads();
@@ -357,32 +275,24 @@ __global__ void __launch_bounds__(64) k_tri_product(const double2* __restrict__ 
 
 }  // namespace
 
-// M1, T, S2 (n^2 complex128 each), then for n > C32_MAXN the FP32 square array in global memory
-size_t cholesky_mixed_workspace(int n) {
-  return (size_t)3 * n * n + (n > C32_MAXN ? ((size_t)n * (n + 1) + 1) / 2 : 0);
-}
+// M1, T, S2 (n^2 complex128 each)
+size_t cholesky_mixed_workspace(int n) { return (size_t)3 * n * n; }
 
 void cholesky_inverse_mixed(const double2* S, double2* M, int n, double tol, double2* work, int* status,
                             cudaStream_t s, float2* M32, bool refine) {
-  if (n > C32_MAXN_GLOBAL) fail(KS_ERR_ARG, "cholesky_inverse_mixed: n=%d > %d", n, C32_MAXN_GLOBAL);
-  const bool glb = n > C32_MAXN;
-  const size_t smem = glb ? 0 : (size_t)n * (n + 1) * sizeof(float2);   // square [n][n+1]
-  static bool attr_set = false;
-  if (!attr_set) {
-    KS_CUDA(cudaFuncSetAttribute(k_chol32_inverse<C32_MAXN, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)((size_t)C32_MAXN * (C32_MAXN + 1) * sizeof(float2))));
-    attr_set = true;
-  }
+  if (n > C32_MAXN) fail(KS_ERR_ARG, "cholesky_inverse_mixed: n=%d > %d", n, C32_MAXN);
   double2* M1 = work;
   double2* T = work + (size_t)n * n;
   double2* S2 = work + (size_t)2 * n * n;
-  float2* gU = reinterpret_cast<float2*>(work + (size_t)3 * n * n);
   auto factor = [&](int conj_out, double2* out, float2* out32) {
-    if (glb)
-      k_chol32_inverse<C32_MAXN_GLOBAL, true><<<1, C32_THREADS, 0, s>>>(S, n, tol, conj_out, status, out, out32, gU);
+    if (n <= 32)
+      launch_chol32<1, 256, 32>(S, n, tol, conj_out, status, out, out32, s);
+    else if (n <= 64)
+      launch_chol32<1, 512, 64>(S, n, tol, conj_out, status, out, out32, s);
+    else if (n <= 128)
+      launch_chol32<1, 1024, 128>(S, n, tol, conj_out, status, out, out32, s);
     else
-      k_chol32_inverse<C32_MAXN, false><<<1, C32_THREADS, smem, s>>>(S, n, tol, conj_out, status, out, out32, nullptr);
-    KS_CHECK_LAUNCH();
+      launch_chol32<8, 512, 256>(S, n, tol, conj_out, status, out, out32, s);
   };
   if (!refine) {                                                     // the FP32 factor itself
     factor(1, M, M32);
