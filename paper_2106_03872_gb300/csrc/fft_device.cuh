@@ -275,8 +275,24 @@ __device__ __forceinline__ void fft_lines_grouped(C* s, int lines, int lstride, 
 // ---------------------------------------------------------------------------------------------
 namespace ks {
 
-// cos(2 pi m / N) for the composite in-register DFTs (N = 12, 16).
+// cos(2 pi m / N) for the composite in-register DFTs (N = 6, 9, 12, 16, 18).
 __host__ __device__ constexpr double cos_frac(int m, int N) {
+  if (N == 6) return cos_frac(2 * m, 12);
+  if (N == 9) return cos_frac(2 * m, 18);
+  if (N == 18) {
+    switch (((m % 18) + 18) % 18) {
+      case 0: return 1.0;
+      case 1: case 17: return 0.93969262078590838405;
+      case 2: case 16: return 0.76604444311897803520;
+      case 3: case 15: return 0.5;
+      case 4: case 14: return 0.17364817766693034885;
+      case 5: case 13: return -0.17364817766693034885;
+      case 6: case 12: return -0.5;
+      case 7: case 11: return -0.76604444311897803520;
+      case 8: case 10: return -0.93969262078590838405;
+      default: return -1.0;
+    }
+  }
   if (N == 16) {
     switch (((m % 16) + 16) % 16) {
       case 0: return 1.0;
@@ -299,6 +315,24 @@ __host__ __device__ constexpr double cos_frac(int m, int N) {
     case 5: case 7: return -0.86602540378443864676;
     default: return -1.0;
   }
+}
+
+// sin(2 pi m / N), the same sizes.
+__host__ __device__ constexpr double sin_frac(int m, int N) {
+  if (N == 6) return cos_frac(2 * m - 3, 12);
+  if (N == 9) return sin_frac(2 * m, 18);
+  if (N == 18) {
+    const int q = ((m % 18) + 18) % 18;
+    const double sg = q > 9 ? -1.0 : 1.0;
+    switch (q > 9 ? 18 - q : q) {
+      case 1: case 8: return sg * 0.34202014332566873304;
+      case 2: case 7: return sg * 0.64278760968653932632;
+      case 3: case 6: return sg * 0.86602540378443864676;
+      case 4: case 5: return sg * 0.98480775301220805937;
+      default: return 0.0;
+    }
+  }
+  return cos_frac(m - N / 4, N);
 }
 
 // In-register DFT of size R1*R2 by one Cooley-Tukey split: n = R2 n1 + n2, k = k1 + R1 k2:
@@ -330,7 +364,7 @@ template <int R1, int R2, typename C> __device__ __forceinline__ void dft_compos
         else
           y[n2][k1] = mk<C>(a.y, -a.x);                              // times -i
       } else {
-        const C w = mk<C>(T(cos_frac(m, N)), T(sign) * T(cos_frac(m - N / 4, N)));
+        const C w = mk<C>(T(cos_frac(m, N)), T(sign) * T(sin_frac(m, N)));
         y[n2][k1] = cmul(t[k1], w);
       }
     }
@@ -349,15 +383,27 @@ template <int R1, int R2, typename C> __device__ __forceinline__ void dft_compos
 template <typename C> struct SmallDft<16, C> {
   static __device__ __forceinline__ void run(C* v, int sign) { dft_composite<4, 4, C>(v, sign); }
 };
+template <typename C> struct SmallDft<6, C> {
+  static __device__ __forceinline__ void run(C* v, int sign) { dft_composite<2, 3, C>(v, sign); }
+};
+template <typename C> struct SmallDft<9, C> {
+  static __device__ __forceinline__ void run(C* v, int sign) { dft_composite<3, 3, C>(v, sign); }
+};
+template <typename C> struct SmallDft<18, C> {
+  static __device__ __forceinline__ void run(C* v, int sign) { dft_composite<3, 6, C>(v, sign); }
+};
 template <typename C> struct SmallDft<12, C> {
   static __device__ __forceinline__ void run(C* v, int sign) { dft_composite<4, 3, C>(v, sign); }
 };
 
 // Radix sequence: a final 12- or 16-point stage where it fits (96 = 8 x 12, 128 = 8 x 16,
-// 48 = 4 x 12, 36 = 12 x 3), else 8, 4, 2, 3.
+// 48 = 4 x 12, 36 = 12 x 3), 54 = 6 x 9, 72 = 8 x 9, 108 = 12 x 9, else 8, 4, 2, 3.
 template <int N, int Ns> struct RadixOf {
   static constexpr int rem = N / Ns;
-  static constexpr int R = (rem == 12 || rem == 16) ? rem
+  static constexpr int first = N == 54 ? 6 : N == 72 ? 8 : N == 108 ? 12 : 0;   // then 9
+  static constexpr int R = (first && Ns == 1)         ? first
+                           : first                    ? rem
+                           : (rem == 12 || rem == 16) ? rem
                            : (rem == 48)            ? 4
                            : (rem == 36)            ? 12
                            : (rem % 8 == 0)         ? 8

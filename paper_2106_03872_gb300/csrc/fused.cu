@@ -56,7 +56,7 @@ template <int N> struct FCfg {
   static constexpr int PMIN = N >= 128 ? 1 : (N >= 64 ? 2 : 4);
   // lines per call: at most 8 complex per thread per stage; 96 takes 32 so that three calls
   // cover the 96 x-lines exactly and no warp straddles two lines' radix jobs
-  static constexpr int LPC = N == 96 ? 32 : ((8 * PT / N) < N ? (8 * PT / N) : N);
+  static constexpr int LPC = N == 96 ? 32 : (N == 72 || N == 108) ? 36 : ((8 * PT / N) < N ? (8 * PT / N) : N);
   static constexpr int ZT = 512;
   static constexpr int CT = (4096 / N) < 32 ? (4096 / N) : 32;
 };
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(FCfg<N>::PT, FCfg<N>::PMIN)
 }
 
 // ---------------------------------------------------------------------------------------------
-// Team plane kernel (N = 32, 48, 64, 96, 128): the same H application per (state, z-plane) as k_plane,
+// Team plane kernel (N = 32, 48, 54, 64, 72, 96, 108, 128): the same H application per (state, z-plane) as k_plane,
 // with the line transforms owned by teams of W warps.  A team owns 32 lines, one per lane, so
 // a warp's 32 lanes always touch 32 consecutive lines at one element: with the odd row pitch
 // N + 1 every shared-memory access is free of bank conflicts along x and along y.  A team's
@@ -413,6 +413,9 @@ template <int N> struct TPlan {
 };
 template <> struct TPlan<32> { static constexpr bool ok = true; static constexpr int R1 = 8, R2 = 4, W = 4; };
 template <> struct TPlan<48> { static constexpr bool ok = true; static constexpr int R1 = 4, R2 = 12, W = 4; };
+template <> struct TPlan<54> { static constexpr bool ok = true; static constexpr int R1 = 6, R2 = 9, W = 3; };
+template <> struct TPlan<72> { static constexpr bool ok = true; static constexpr int R1 = 6, R2 = 12, W = 6; };
+template <> struct TPlan<108> { static constexpr bool ok = true; static constexpr int R1 = 6, R2 = 18, W = 6; };
 template <> struct TPlan<64> { static constexpr bool ok = true; static constexpr int R1 = 8, R2 = 8, W = 4; };
 template <> struct TPlan<96> { static constexpr bool ok = true; static constexpr int R1 = 8, R2 = 12, W = 4; };
 template <> struct TPlan<128> { static constexpr bool ok = true; static constexpr int R1 = 8, R2 = 16, W = 8; };
@@ -432,7 +435,7 @@ template <int N> struct PlaneForm {
 template <int N> struct TCfg {
   static constexpr int TEAMS = (N + 31) / 32;
   static constexpr int PT = 32 * TPlan<N>::W * TEAMS;
-  static constexpr int PMIN = N >= 128 ? 1 : 2;
+  static constexpr int PMIN = N >= 108 ? 1 : 2;
   static constexpr int NW = (N + 31) / 32;                // bitmap words per line
 };
 
@@ -604,10 +607,8 @@ __device__ __forceinline__ void team_x_roundtrip(float2* P, int xr, const float*
   // inverse stage B (radix R2, natural order out), pointwise u, forward stage A' (radix R2 on the
   // same elements e = j + r R1)
   {
-    // element e = j + R1 r (j < R1, R1 dividing 32) lies in bitmap word (R1 r) / 32 at bit
-    // (R1 r mod 32) + j: the word index is a compile-time constant; pre[k] counts the line's points
-    // in words < k
-    static_assert(32 % R1 == 0, "bitmap word of e = j + R1 r");
+    // element e = j + R1 r (j < R1): where R1 divides 32 it lies in bitmap word (R1 r) / 32 at bit
+    // (R1 r mod 32) + j, the word index a compile-time constant
     uint32_t wbits[NW];
     int lo = 0;
     if (act) {
@@ -638,12 +639,20 @@ __device__ __forceinline__ void team_x_roundtrip(float2* P, int xr, const float*
 #pragma unroll
         for (int r = 0; r < R2; ++r) {
           float2 u = make_float2(v[q][r].x * vv[r], v[q][r].y * vv[r]);
-          const uint32_t word = wbits[(R1 * r) >> 5];
-          const int bit = ((R1 * r) & 31) + j;
+          uint32_t word = wbits[(R1 * r) >> 5];
+          int bit = ((R1 * r) & 31) + j, nw = (R1 * r) >> 5;
+          if constexpr (32 % R1 != 0) {
+            if (bit >= 32) {                                  // the element spills into the next word
+              word = wbits[min((R1 * r) / 32 + 1, NW - 1)];
+              bit -= 32;
+              ++nw;
+            }
+          }
           if ((word >> bit) & 1u) {
             int before = lo;                                  // points of this line in earlier words
 #pragma unroll
-            for (int k = 0; k < (R1 * r) >> 5; ++k) before += __popc(wbits[k]);
+            for (int k = 0; k < NW; ++k)
+              if (k < nw) before += __popc(wbits[k]);
             const float2 a = nlv[before + __popc(word & ((1u << bit) - 1u))];
             u.x += a.x;
             u.y += a.y;
@@ -882,7 +891,7 @@ __global__ void __launch_bounds__(FCfg<N>::ZT, 2) k_zfwd_group(const __grid_cons
   zfwd_body<N>(M.cb2, M.psi, M.hpsi, nG, col_off, col_half, g2half, ncols, scale, twg, M.te, blockIdx.y - M.s0);
 }
 
-// Density partial sums with the team transforms (N = 32, 48, 64, 96, 128): one (z-plane, chunk of
+// Density partial sums with the team transforms (TPlan<N>::ok): one (z-plane, chunk of
 // states) per CTA, states in order.  Per state: the band rows are zeroed, the columns scattered,
 // the inverse y transform of the band rows, then the inverse x transform whose stage B leaves
 // each thread the elements e = j + r R1 of its x-line in registers; f |u|^2 is added to
@@ -1234,7 +1243,7 @@ class FusedImpl final : public FusedOps {
  public:
   static bool supported(int N) {
     switch (N) {
-      case 18: case 24: case 32: case 36: case 48: case 64: case 96: case 128: return true;
+      case 18: case 24: case 32: case 36: case 48: case 54: case 64: case 72: case 96: case 108: case 128: return true;
       default: return false;
     }
   }
@@ -1458,8 +1467,11 @@ class FusedImpl final : public FusedOps {
       case 32: f(IntTag<32>{}); break;
       case 36: f(IntTag<36>{}); break;
       case 48: f(IntTag<48>{}); break;
+      case 54: f(IntTag<54>{}); break;
       case 64: f(IntTag<64>{}); break;
+      case 72: f(IntTag<72>{}); break;
       case 96: f(IntTag<96>{}); break;
+      case 108: f(IntTag<108>{}); break;
       case 128: f(IntTag<128>{}); break;
       default: fail(KS_ERR_ARG, "fused path: unsupported grid %d", N_);
     }
@@ -1580,7 +1592,7 @@ class FusedImpl final : public FusedOps {
   // at N = 128
   bool team_density() const {
     switch (N_) {
-      case 32: case 48: case 64: case 96: case 128: return true;
+      case 32: case 48: case 54: case 64: case 72: case 96: case 108: case 128: return true;
       default: return false;
     }
   }
