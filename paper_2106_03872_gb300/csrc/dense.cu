@@ -63,8 +63,7 @@ __global__ void __launch_bounds__(256) k_gemm_cn(const cplx<T>* __restrict__ A, 
     }
 }
 
-__global__ void k_reduce_parts(const double2* __restrict__ part, int nks, size_t mn, double2* __restrict__ out,
-                               float2* __restrict__ out32) {
+__global__ void k_reduce_parts(const double2* __restrict__ part, int nks, size_t mn, double2* __restrict__ out) {
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < mn; e += (size_t)gridDim.x * blockDim.x) {
     double2 s = make_double2(0.0, 0.0);
     for (int k = 0; k < nks; ++k) {
@@ -73,13 +72,12 @@ __global__ void k_reduce_parts(const double2* __restrict__ part, int nks, size_t
       s.y += p.y;
     }
     out[e] = s;
-    if (out32) out32[e] = make_float2((float)s.x, (float)s.y);
   }
 }
 
 // Y[i][k] = sum_j M[i][j] X[j][k]; tile 32 rows x 64 columns, each thread 2 x 4 outputs.
-template <typename T, typename MC>
-__global__ void __launch_bounds__(256) k_rotate(const MC* __restrict__ M, int nin, const cplx<T>* __restrict__ X,
+template <typename T>
+__global__ void __launch_bounds__(256) k_rotate(const double2* __restrict__ M, int nin, const cplx<T>* __restrict__ X,
                                                 const cplx<T>* __restrict__ X2, int nin1, int ldx, cplx<T>* __restrict__ Y,
                                                 int ldy, int m, int K) {
   using C = cplx<T>;
@@ -91,12 +89,8 @@ __global__ void __launch_bounds__(256) k_rotate(const MC* __restrict__ M, int ni
   for (int j0 = 0; j0 < nin; j0 += KT) {
     for (int e = threadIdx.x; e < 32 * KT; e += 256) {
       const int r = e / KT, jj = e % KT;
-      C v = mk<C>(T(0), T(0));
-      if (i0 + r < m && j0 + jj < nin) {
-        const MC q = M[(size_t)(i0 + r) * nin + j0 + jj];
-        v = mk<C>(T(q.x), T(q.y));
-      }
-      Ms[r][jj] = v;
+      const double2 v = (i0 + r < m && j0 + jj < nin) ? M[(size_t)(i0 + r) * nin + j0 + jj] : make_double2(0.0, 0.0);
+      Ms[r][jj] = mk<C>(T(v.x), T(v.y));
     }
     for (int e = threadIdx.x; e < KT * 64; e += 256) {
       const int jj = e / 64, c = e % 64;
@@ -496,7 +490,7 @@ __global__ void __launch_bounds__(SV_THREADS) k_sort_vectors(const double* __res
 
 template <typename T>
 void gemm_cn(const cplx<T>* A, int lda, const cplx<T>* B, int ldb, int m, int n, int K, double2* part,
-             size_t part_elems, double2* out, cudaStream_t s, float2* out32) {
+             size_t part_elems, double2* out, cudaStream_t s) {
   const int tm = (m + GT - 1) / GT, tn = (n + GT - 1) / GT;
   int ks = std::max(1, 304 / (tm * tn));
   ks = std::min(ks, std::max(1, K / 256));
@@ -509,16 +503,16 @@ void gemm_cn(const cplx<T>* A, int lda, const cplx<T>* B, int ldb, int m, int n,
   k_gemm_cn<T><<<g, 256, 0, s>>>(A, lda, B, ldb, m, n, K, kchunk, part);
   KS_CHECK_LAUNCH();
   const size_t mn = (size_t)m * n;
-  k_reduce_parts<<<(unsigned)std::min<size_t>((mn + 255) / 256, 1024), 256, 0, s>>>(part, ks, mn, out, out32);
+  k_reduce_parts<<<(unsigned)std::min<size_t>((mn + 255) / 256, 1024), 256, 0, s>>>(part, ks, mn, out);
   KS_CHECK_LAUNCH();
 }
 
-template <typename T, typename MC>
-void rotate(const MC* M, int nin, const cplx<T>* X, const cplx<T>* X2, int nin1, int ldx, cplx<T>* Y, int ldy,
+template <typename T>
+void rotate(const double2* M, int nin, const cplx<T>* X, const cplx<T>* X2, int nin1, int ldx, cplx<T>* Y, int ldy,
             int m, int K, cudaStream_t s) {
   if (!X2) nin1 = nin;
   dim3 g((K + 63) / 64, (m + 31) / 32);
-  k_rotate<T, MC><<<g, 256, 0, s>>>(M, nin, X, X2, nin1, ldx, Y, ldy, m, K);
+  k_rotate<T><<<g, 256, 0, s>>>(M, nin, X, X2, nin1, ldx, Y, ldy, m, K);
   KS_CHECK_LAUNCH();
 }
 
@@ -540,7 +534,10 @@ void cholesky_inverse_tol(double2* A, double2* M, int n, double tol, int* status
 
 void eigh_mixed(const double2* A, double2* V, double* lam, double* eig, double2* Vt, void* work, int n,
                 cudaStream_t s) {
-  eigh_vectors_f32(A, V, n, work, Vt, s);                              // Vt is scratch until the sort
+  if (n <= SMALL_SUBSPACE)
+    eigh_small(A, V, n, s);
+  else
+    eigh_vectors_f32(A, V, n, work, Vt, s);                            // Vt is scratch until the sort
   k_rayleigh_quotients<<<n, 256, 0, s>>>(A, V, n, lam);
   KS_CHECK_LAUNCH();
   k_sort_vectors<<<n, SV_THREADS, 0, s>>>(lam, V, n, eig, Vt);
@@ -568,14 +565,12 @@ void jacobi_eigh(double2* A, double2* V, double* eig, double2* Vt, int n, cudaSt
 }
 
 template void gemm_cn<float>(const float2*, int, const float2*, int, int, int, int, double2*, size_t, double2*,
-                             cudaStream_t, float2*);
+                             cudaStream_t);
 template void gemm_cn<double>(const double2*, int, const double2*, int, int, int, int, double2*, size_t, double2*,
-                              cudaStream_t, float2*);
-template void rotate<float, double2>(const double2*, int, const float2*, const float2*, int, int, float2*, int, int,
-                                     int, cudaStream_t);
-template void rotate<float, float2>(const float2*, int, const float2*, const float2*, int, int, float2*, int, int,
-                                    int, cudaStream_t);
-template void rotate<double, double2>(const double2*, int, const double2*, const double2*, int, int, double2*, int,
-                                      int, int, cudaStream_t);
+                              cudaStream_t);
+template void rotate<float>(const double2*, int, const float2*, const float2*, int, int, float2*, int, int, int,
+                            cudaStream_t);
+template void rotate<double>(const double2*, int, const double2*, const double2*, int, int, double2*, int, int, int,
+                             cudaStream_t);
 
 }  // namespace ks

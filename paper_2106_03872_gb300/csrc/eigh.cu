@@ -693,6 +693,10 @@ void eigh_vectors_f32(const double2* A, double2* V, int n, void* work, void* wor
 void rr_step_mixed(const float2* Hraw, const float2* M, double alpha, int n, float2* Mcat, float2* Aout,
                    float2* Vout, int* perm, void* work, cudaStream_t s) {
   if (n > RR_MAXN || n < 1) fail(KS_ERR_ARG, "rr_step_mixed: n=%d not in [1, %d]", n, RR_MAXN);
+  if (n <= SMALL_SUBSPACE) {
+    rr_step_small(Hraw, M, alpha, n, Mcat, Aout, Vout, perm, s);
+    return;
+  }
   float *lam, *G;
   const Tri T = lay_out(work, n, lam, G);
   float* zt = reinterpret_cast<float*>(Mcat);                        // [n][n] floats, read before Mcat is written

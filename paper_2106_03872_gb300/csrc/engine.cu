@@ -303,7 +303,7 @@ template <typename T> class Engine final : public EngineBase {
     }
     // ---- dense LA
     const size_t nn = (size_t)ns_ * ns_;
-    part_elems_ = std::max<size_t>(nn * (small_block() ? 304 : 8), 4096);
+    part_elems_ = std::max<size_t>(nn * 8, 4096);
     if (use_tc()) {
       part_elems_ = std::max(part_elems_, tc_overlap_part_elems(ns_, ns_));
       rotws_bytes_ = tc_rotation_workspace_bytes(ns_, 2 * ns_);
@@ -640,7 +640,7 @@ template <typename T> class Engine final : public EngineBase {
           ProfScope p(prof, "rr_step", aux_);
           rr_step_mixed(hraw32_, m32_, alpha, n, mcat32_, aexp_, vexp_, perm_, ehw_, aux_);
         }
-        if (use_tc()) {
+        {
           ProfScope p(prof, "rot_prep", aux_);
           tc_rotate_prepare(mcat32_, n, 2 * n, rotws_, rotws_bytes_, aux_);
         }
@@ -1426,13 +1426,7 @@ template <typename T> class Engine final : public EngineBase {
       if (buf_[i] != a && buf_[i] != b) return buf_[i];
     fail(KS_ERR_STATE, "internal: no spare state buffer");
   }
-  // Blocks of at most 16 states take the CUDA-core FP32 overlap and rotation instead of the
-  // tensor-core kernels: an eighth of a 128-row operand tile would be states, and the unsplit FP32
-  // products are exact to 24 bits where the split ones carry 16 (an orthonormalised block of 7 states
-  // is off by 5e-6 with them).
-  static constexpr int SMALL_BLOCK = 16;
-  bool small_block() const { return sizeof(T) == 4 && ns_ <= SMALL_BLOCK; }
-  bool use_tc() const { return sizeof(T) == 4 && prec_ == KS_MIXED_BF16X3 && !small_block(); }
+  bool use_tc() const { return sizeof(T) == 4 && prec_ == KS_MIXED_BF16X3; }
   bool mixed_cholesky() const { return sizeof(T) == 4 && ns_ <= 256; }
   bool mixed_eigh() const { return sizeof(T) == 4 && ns_ <= 256; }
   // the mixed path's FP32 Householder eigensolver up to 256 states (finished by FP64 Rayleigh
@@ -1447,7 +1441,7 @@ template <typename T> class Engine final : public EngineBase {
   // the Rayleigh-Ritz eigensolver in FP64 (as on the FP64 path), the states and their GEMMs mixed
   bool fp64_subspace_ = false;
   // the block iteration's Rayleigh-Ritz step runs in FP32 (rr_step_mixed)
-  bool fused_rr() const { return sizeof(T) == 4 && ns_ <= 128; }
+  bool fused_rr() const { return use_tc() && ns_ <= 128; }
 
   // out = A^H B over the sphere (n x n), tensor cores on the bf16x3 mixed path
   void overlap(const C* A, const C* B, int n, double2* out, cudaStream_t s, float2* out32 = nullptr) {
@@ -1457,7 +1451,7 @@ template <typename T> class Engine final : public EngineBase {
         return;
       }
     }
-    gemm_cn<T>(A, g_.nG, B, g_.nG, n, n, g_.nG, part_, part_elems_, out, s, out32);
+    gemm_cn<T>(A, g_.nG, B, g_.nG, n, n, g_.nG, part_, part_elems_, out, s);
   }
 
   // Y = M X (rows of states); with X2, M is n x 2n and X = [X; X2]
@@ -1469,18 +1463,14 @@ template <typename T> class Engine final : public EngineBase {
         return;
       }
     }
-    rotate<T, double2>(M, nin, X, X2, ns_, g_.nG, Y, g_.nG, ns_, g_.nG, s);
+    rotate<T>(M, nin, X, X2, ns_, g_.nG, Y, g_.nG, ns_, g_.nG, s);
   }
 
-  // Y = Mcat [X; X2] from the split image of mcat32_ that tc_rotate_prepare left in rotws_ (small
-  // blocks: from mcat32_ itself)
+  // Y = Mcat [X; X2] from the split image of mcat32_ that tc_rotate_prepare left in rotws_
   void rot_prepared(const C* X, const C* X2, C* Y, cudaStream_t s) {
-    if constexpr (std::is_same<T, float>::value) {
-      if (use_tc())
-        tc_rotate_prepared(rotws_, 2 * ns_, X, X2, ns_, g_.nG, Y, g_.nG, ns_, g_.nG, status_ + 1, s);
-      else
-        rotate<float, float2>(mcat32_, 2 * ns_, X, X2, ns_, g_.nG, Y, g_.nG, ns_, g_.nG, s);
-    } else
+    if constexpr (std::is_same<T, float>::value)
+      tc_rotate_prepared(rotws_, 2 * ns_, X, X2, ns_, g_.nG, Y, g_.nG, ns_, g_.nG, status_ + 1, s);
+    else
       fail(KS_ERR_STATE, "internal: prepared rotation on the FP64 path");
   }
 

@@ -134,15 +134,13 @@ template <typename T> void real_to_double(const T* in, double* out, size_t n, cu
 
 // ---- dense linear algebra (dense.cu) ----------------------------------------------------------
 // out[i][j] = sum_k conj(A[i][k]) B[j][k] for i < m, j < n (row-major, FP64 out); split-K with
-// deterministic reduction through `part` (>= gemm_cn_parts(...) double2 elements); out32, when given,
-// receives an FP32 copy.
+// deterministic reduction through `part` (>= gemm_cn_parts(...) double2 elements).
 template <typename T> void gemm_cn(const cplx<T>* A, int lda, const cplx<T>* B, int ldb, int m, int n, int K,
-                                   double2* part, size_t part_elems, double2* out, cudaStream_t s,
-                                   float2* out32 = nullptr);
+                                   double2* part, size_t part_elems, double2* out, cudaStream_t s);
 // Y[i][k] = sum_j M[i][j] X[j][k], i < m, j < nin, k < K; rows j >= nin1 of X come from X2
 // (row j - nin1) when X2 is non-NULL.  Y must not overlap X or X2.
-template <typename T, typename MC> void rotate(const MC* M, int nin, const cplx<T>* X, const cplx<T>* X2, int nin1,
-                                               int ldx, cplx<T>* Y, int ldy, int m, int K, cudaStream_t s);
+template <typename T> void rotate(const double2* M, int nin, const cplx<T>* X, const cplx<T>* X2, int nin1, int ldx,
+                                  cplx<T>* Y, int ldy, int m, int K, cudaStream_t s);
 // A := (A + A^H)/2
 void hermitize(double2* A, int n, cudaStream_t s);
 // C = opA(A) opB(B), n x n complex128 (row-major); flags: 1 conj(A), 2 B transposed, 4 conj(B).
@@ -182,6 +180,14 @@ void eigh_mixed(const double2* A, double2* V, double* lam, double* eig, double2*
 // eigh_workspace(n) bytes.
 void rr_step_mixed(const float2* Hraw, const float2* M, double alpha, int n, float2* Mcat, float2* Aout,
                    float2* Vout, int* perm, void* work, cudaStream_t s);
+// Blocks of at most SMALL_SUBSPACE states take one-CTA kernels instead (subspace_small.cu), through
+// cholesky_inverse_mixed, eigh_mixed and rr_step_mixed.
+constexpr int SMALL_SUBSPACE = 16;
+void cholesky_small(const double2* S, double2* M, int n, double tol, double2* work, int* status, cudaStream_t s,
+                    float2* M32, bool refine);
+void eigh_small(const double2* A, double2* V, int n, cudaStream_t s);
+void rr_step_small(const float2* Hraw, const float2* M, double alpha, int n, float2* Mcat, float2* Aout,
+                   float2* Vout, int* perm, cudaStream_t s);
 // eig[perm[j]] = FP64 Rayleigh quotient of column j of V on A (outputs of rr_step_mixed).
 void ritz_values(const float2* A, const float2* V, const int* perm, int n, double* eig, cudaStream_t s);
 
