@@ -392,8 +392,14 @@ template <typename T> class Engine final : public EngineBase {
   }
   void td_prepare(int hartree_xc, cudaStream_t s) {
     hpsi_valid_ = false;
-    if (!hartree_xc)
-      KS_CUDA(cudaMemcpyAsync(vtot_, vloc_, (size_t)g_.N * g_.N * g_.N * sizeof(T), cudaMemcpyDeviceToDevice, s));
+    if (!hartree_xc) reset_potential(s);
+  }
+  // V = V_loc
+  void reset_potential(cudaStream_t s) {
+    KS_CUDA(cudaMemcpyAsync(vtot_, vloc_, (size_t)g_.N * g_.N * g_.N * sizeof(T), cudaMemcpyDeviceToDevice, s));
+    if constexpr (sizeof(T) == 4) {
+      if (fused_) fused_->load_potential(vtot_, s);
+    }
   }
   void td_read_slot0(double* nrm, double* e, cudaStream_t s) {
     KS_CUDA(cudaMemcpyAsync(nrm, norms_dev_, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -431,7 +437,7 @@ template <typename T> class Engine final : public EngineBase {
     ProfScope scope(prof, "apply_h", s);
     if constexpr (std::is_same<T, float>::value) {
       if (fused_) {
-        fused_->apply_h(psi, hpsi, n, vtot_, s);
+        fused_->apply_h(psi, hpsi, n, s);
         return;
       }
     }
@@ -504,6 +510,14 @@ template <typename T> class Engine final : public EngineBase {
     ProfScope scope(prof, "hartree_xc", s);
     const int N = g_.N;
     const size_t N3 = (size_t)N * N * N;
+    if constexpr (std::is_same<T, float>::value) {
+      if (fused_) {
+        static_assert(HXC_BLOCKS >= 128, "a row of sums per x-plane");
+        fused_->hartree_exchange(n, vloc_, vtot_, pwork_, hxc_partials_, s);
+        hxc_finish(hxc_partials_, N, g_.dV, parts_, s);
+        return;
+      }
+    }
     real_to_complex<T>(n, pwork_, (int)N3, s);
     for (int ax = 2; ax >= 0; --ax) fft_axis<T>(pwork_, 1, N, ax, -1, t_.tw, s);
     poisson_multiply<T>(pwork_, N, g_.L, T(1.0 / double(N3)), s);
@@ -1005,7 +1019,7 @@ template <typename T> class Engine final : public EngineBase {
                 double* dipole_out, cudaStream_t s) override {
     hpsi_valid_ = false;
     if (nsteps < 0 || (propagator != 0 && propagator != 1)) fail(KS_ERR_ARG, "td: nsteps=%d propagator=%d", nsteps, propagator);
-    if (!hartree_xc) KS_CUDA(cudaMemcpyAsync(vtot_, vloc_, (size_t)g_.N * g_.N * g_.N * sizeof(T), cudaMemcpyDeviceToDevice, s));
+    if (!hartree_xc) reset_potential(s);
     double first_norm = 0;
     bool have_first = false;
     for (int c0 = 0; c0 < nsteps; c0 += MAX_STEPS_CHUNK) {
@@ -1086,8 +1100,7 @@ template <typename T> class Engine final : public EngineBase {
     for (int i = 0; i < 3 * na; ++i)
       if (!std::isfinite(vel[i])) fail(KS_ERR_ARG, "ehrenfest: velocity %d is not finite", i);
     hpsi_valid_ = false;
-    const size_t N3 = (size_t)g_.N * g_.N * g_.N;
-    if (!hartree_xc) KS_CUDA(cudaMemcpyAsync(vtot_, vloc_, N3 * sizeof(T), cudaMemcpyDeviceToDevice, s));
+    if (!hartree_xc) reset_potential(s);
     std::vector<double> F(3 * (size_t)na), F1(3 * (size_t)na), R1(3 * (size_t)na);
     if (na) forces(F.data(), s);
     double first_norm = 0.0;
@@ -1262,7 +1275,6 @@ template <typename T> class Engine final : public EngineBase {
           it.psi = kk == 1 ? x[i] : (*outs[kk - 2])[i];
           it.n = es[i]->ns_;
           it.cols_ready = kk == 1 && cols_ready;
-          it.v = es[i]->vtot_;
           if (kk < 4) {
             it.hpsi = (*outs[kk - 1])[i];
           } else {
@@ -1334,7 +1346,6 @@ template <typename T> class Engine final : public EngineBase {
           it.psi = w[i];
           it.hpsi = wn[i];
           it.n = es[i]->ns_;
-          it.v = es[i]->vtot_;
           it.te.acc1 = acc1[i];
           it.te.a1 = make_float2((float)a1.x, (float)a1.y);
           it.te.acc2 = acc2[i];
@@ -1367,7 +1378,7 @@ template <typename T> class Engine final : public EngineBase {
     const size_t N3 = (size_t)N * N * N;
     build_axis_tables(s);
     vloc_from_axes<T>(fxyz_, g_.natoms, N, g_.vloc_depth, vloc_, vloc64_, s);
-    KS_CUDA(cudaMemcpyAsync(vtot_, vloc_, N3 * sizeof(T), cudaMemcpyDeviceToDevice, s));
+    reset_potential(s);
     minmax(vloc64_, N3, hxc_partials_, HXC_BLOCKS, vmm_, s);
     double mm[2];
     KS_CUDA(cudaMemcpyAsync(mm, vmm_, sizeof(mm), cudaMemcpyDeviceToHost, s));

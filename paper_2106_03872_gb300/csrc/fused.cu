@@ -156,6 +156,7 @@ template <int N>
 __global__ void __launch_bounds__(FCfg<N>::ZT, 2) k_zinv(const float2* __restrict__ psi, int nG, const int* __restrict__ col_off,
                                                       const int* __restrict__ col_half, int ncols, int nstates,
                                                       float2* __restrict__ colbuf, const float2* __restrict__ twg) {
+  chain_begin();
   zinv_body<N>(psi, nG, col_off, col_half, ncols, nstates, colbuf, twg, blockIdx.y);
 }
 
@@ -261,6 +262,7 @@ __global__ void __launch_bounds__(FCfg<N>::ZT, 2) k_zfwd(const float2* __restric
                                                       const int* __restrict__ col_half, const float* __restrict__ g2half,
                                                       int ncols, float scale, const float2* __restrict__ twg,
                                                       TaylorEpi te) {
+  chain_begin();
   zfwd_body<N>(colbuf, psi, hpsi, nG, col_off, col_half, g2half, ncols, scale, twg, te, blockIdx.y);
 }
 
@@ -335,6 +337,7 @@ __global__ void __launch_bounds__(FCfg<N>::PT, FCfg<N>::PMIN)
     k_plane(const float2* __restrict__ colbuf1, float2* __restrict__ colbuf2, int ncols, const int* __restrict__ col_xy,
             int xr, const float* __restrict__ vplane, PlaneNL nl, const float2* __restrict__ pf, int nprojtot,
             int pf_smem, const float2* __restrict__ twg) {
+  chain_begin();
   constexpr int ld = N + 1, PT = FCfg<N>::PT;
   extern __shared__ __align__(16) float2 psm[];
   float2* tw = psm;
@@ -776,6 +779,7 @@ constexpr int NLB = 8;
 template <bool P4>
 __global__ void __launch_bounds__(256) k_nl_values(const float2* __restrict__ pf, int nprojtot, int n, PlaneNL nl,
                                                    int npts, float2* __restrict__ nlval) {
+  chain_begin();
   const int pt = blockIdx.x * blockDim.x + threadIdx.x;
   if (pt >= npts) return;
   const int b0 = blockIdx.y * NLB, nb = min(NLB, n - b0);
@@ -827,6 +831,7 @@ __global__ void __launch_bounds__(TCfg<N>::PT, TCfg<N>::PMIN)
     k_plane_team(const float2* __restrict__ colbuf1, float2* __restrict__ colbuf2, int ncols,
                  const int* __restrict__ col_xy, int xr, const int* __restrict__ rowym,
                  const float* __restrict__ vplane, TeamNL nl, int cap, const float2* __restrict__ twg) {
+  chain_begin();
   plane_team_body<N>(colbuf1, colbuf2, ncols, col_xy, xr, rowym, vplane, nl, cap, twg, blockIdx.x, blockIdx.y);
 }
 
@@ -868,6 +873,7 @@ __global__ void __launch_bounds__(FCfg<N>::ZT, 2) k_zinv_group(const __grid_cons
                                                             const int* __restrict__ col_off,
                                                             const int* __restrict__ col_half, int ncols,
                                                             const float2* __restrict__ twg) {
+  chain_begin();
   const GMember& M = gd.m[member_by_zblock(gd, blockIdx.y)];
   zinv_body<N>(M.psi, nG, col_off, col_half, ncols, M.n, M.cb1, twg, blockIdx.y - M.z0);
 }
@@ -876,6 +882,7 @@ template <int N>
 __global__ void __launch_bounds__(TCfg<N>::PT, TCfg<N>::PMIN)
     k_plane_team_group(const __grid_constant__ GDesc gd, int ncols, const int* __restrict__ col_xy, int xr,
                        const int* __restrict__ rowym, const float2* __restrict__ twg) {
+  chain_begin();
   const GMember& M = gd.m[member_by_state(gd, blockIdx.y)];
   plane_team_body<N>(M.cb1, M.cb2, ncols, col_xy, xr, rowym, M.vplane, M.nl, M.cap, twg, blockIdx.x,
                      blockIdx.y - M.s0);
@@ -887,6 +894,7 @@ __global__ void __launch_bounds__(FCfg<N>::ZT, 2) k_zfwd_group(const __grid_cons
                                                             const int* __restrict__ col_half,
                                                             const float* __restrict__ g2half, int ncols, float scale,
                                                             const float2* __restrict__ twg) {
+  chain_begin();
   const GMember& M = gd.m[member_by_state(gd, blockIdx.y)];
   zfwd_body<N>(M.cb2, M.psi, M.hpsi, nG, col_off, col_half, g2half, ncols, scale, twg, M.te, blockIdx.y - M.s0);
 }
@@ -903,6 +911,7 @@ __global__ void __launch_bounds__(TCfg<N>::PT, TCfg<N>::PMIN)
                          const int* __restrict__ rowym, int nstates, int chunk, const double* __restrict__ occ,
                          float scale,
                          float* __restrict__ partial, const float2* __restrict__ twg) {
+  chain_begin();
   using TP = TPlan<N>;
   constexpr int R1 = TP::R1, R2 = TP::R2, W = TP::W, QA = R2 / W, QB = R1 / W;
   constexpr int ld = N + 1, KS = N + 1, PT = TCfg<N>::PT;
@@ -1094,6 +1103,7 @@ __global__ void __launch_bounds__(FCfg<N>::PT, FCfg<N>::PMIN)
     k_plane_density_chunk(const float2* __restrict__ colbuf1, int ncols, const int* __restrict__ col_xy, int xr,
                           int nstates, int chunk, const double* __restrict__ occ, float scale,
                           float* __restrict__ partial, const float2* __restrict__ twg) {
+  chain_begin();
   constexpr int ld = N + 1, PT = FCfg<N>::PT;
   extern __shared__ __align__(16) float2 psm[];
   float2* tw = psm;
@@ -1114,6 +1124,7 @@ __global__ void __launch_bounds__(FCfg<N>::PT, FCfg<N>::PMIN)
 
 // n[(jx*N + jy)*N + z] = sum_ch partial[ch][z][jx*N + jy]
 __global__ void k_density_reduce(const float* __restrict__ partial, int nch, int N, float* __restrict__ n) {
+  chain_begin();
   const size_t N3 = (size_t)N * N * N;
   for (size_t j = blockIdx.x * (size_t)blockDim.x + threadIdx.x; j < N3; j += (size_t)gridDim.x * blockDim.x) {
     const int z = (int)(j % N);
@@ -1126,6 +1137,7 @@ __global__ void k_density_reduce(const float* __restrict__ partial, int nch, int
 
 // vplane[z][jx*N + jy] = v[(jx*N + jy)*N + z]
 __global__ void k_to_planes(const float* __restrict__ v, int N, float* __restrict__ vplane) {
+  chain_begin();
   const size_t N3 = (size_t)N * N * N;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < N3; e += (size_t)gridDim.x * blockDim.x) {
     const size_t z = e / ((size_t)N * N), xy = e % ((size_t)N * N);
@@ -1133,13 +1145,116 @@ __global__ void k_to_planes(const float* __restrict__ v, int N, float* __restric
   }
 }
 
-// pf[b][ip] = scale * (float) pout[ip][b]
-__global__ void k_proj_to_states(const double2* __restrict__ pout, int nprojtot, int nst, float scale,
-                                 float2* __restrict__ pf) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nprojtot * nst; e += gridDim.x * blockDim.x) {
-    const int b = e / nprojtot, ip = e - b * nprojtot;
-    const double2 v = pout[(size_t)ip * nst + b];
-    pf[e] = make_float2((float)(v.x * scale), (float)(v.y * scale));
+// ---------------------------------------------------------------------------------------------
+// V = V_loc + v_H[n] + v_x[n] on the grid in three passes of whole (y, z) planes and x lines:
+//   k_hx_fwd   one x-plane per CTA: n to shared memory, forward z and y transforms
+//   k_hx_x     32 x lines per CTA (one y, 32 consecutive z): forward x transform, 4 pi / |G|^2 N^-3 from a
+//              table over |m|^2, inverse x transform
+//   k_hx_inv   one x-plane per CTA: inverse y and z transforms, then v_x, V, the energy sums, and V in
+//              the H application's per-plane layout
+// Six line passes through HBM with a kernel each for the copy in, the Poisson factor (an FP64 division
+// per point) and the sums took 116, 132 and 339 us a call at N = 32, 64 and 128 (with a one-thread final
+// sum); these take 20, 31 and 80 us.
+// ---------------------------------------------------------------------------------------------
+template <int N>
+__global__ void __launch_bounds__(FCfg<N>::PT, FCfg<N>::PMIN)
+    k_hx_fwd(const float* __restrict__ n, float2* __restrict__ w, const float2* __restrict__ twg) {
+  constexpr int ld = N + 1, PT = FCfg<N>::PT;
+  extern __shared__ __align__(16) float2 psm[];
+  chain_begin();
+  float2* tw = psm;
+  float2* P = psm + N;                                               // [y][z]
+  const size_t plane = (size_t)blockIdx.x * N * N;
+  for (int t = threadIdx.x; t < N; t += PT) tw[t] = twg[t];
+  for (int e = threadIdx.x; e < N * N; e += PT) P[(e / N) * ld + e % N] = make_float2(n[plane + e], 0.f);
+  __syncthreads();
+  cfft_lines<N, PT, FCfg<N>::LPC, true, -1>(P, N, ld, 1, tw);        // z lines
+  x_pass<N, -1>(P, tw);                                              // y lines (stride N + 1)
+  for (int e = threadIdx.x; e < N * N; e += PT) w[plane + e] = P[(e / N) * ld + e % N];
+}
+
+__device__ __forceinline__ int grid_freq(int j, int N) { return 2 * j < N ? j : j - N; }
+
+template <int N>
+__global__ void __launch_bounds__(FCfg<N>::ZT, 2)
+    k_hx_x(float2* __restrict__ w, const float* __restrict__ pois, const float2* __restrict__ twg) {
+  constexpr int ld = N + 1, ZT = FCfg<N>::ZT, LB = 32;
+  __shared__ float2 tw[N];
+  __shared__ float2 s[LB * ld];
+  chain_begin();
+  const int z0 = blockIdx.x * LB, y = blockIdx.y, nl = min(LB, N - z0);
+  for (int t = threadIdx.x; t < N; t += ZT) tw[t] = twg[t];
+  for (int e = threadIdx.x; e < N * LB; e += ZT) {
+    const int x = e / LB, l = e % LB;
+    if (l < nl) s[l * ld + x] = w[((size_t)x * N + y) * N + z0 + l];
+  }
+  __syncthreads();
+  cfft_lines<N, ZT, LB, true, -1>(s, nl, ld, 1, tw);
+  const int my = grid_freq(y, N);
+  for (int e = threadIdx.x; e < N * LB; e += ZT) {
+    const int x = e / LB, l = e % LB;
+    if (l < nl) {
+      const int mx = grid_freq(x, N), mz = grid_freq(z0 + l, N);
+      const float f = pois[mx * mx + my * my + mz * mz];
+      const float2 v = s[l * ld + x];
+      s[l * ld + x] = make_float2(v.x * f, v.y * f);
+    }
+  }
+  __syncthreads();
+  cfft_lines<N, ZT, LB, true, +1>(s, nl, ld, 1, tw);
+  for (int e = threadIdx.x; e < N * LB; e += ZT) {
+    const int x = e / LB, l = e % LB;
+    if (l < nl) w[((size_t)x * N + y) * N + z0 + l] = s[l * ld + x];
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(FCfg<N>::PT, FCfg<N>::PMIN)
+    k_hx_inv(const float2* __restrict__ w, const float* __restrict__ n, const float* __restrict__ vloc,
+             float* __restrict__ vtot, float* __restrict__ vplane, double* __restrict__ partials,
+             const float2* __restrict__ twg) {
+  constexpr int ld = N + 1, PT = FCfg<N>::PT;
+  extern __shared__ __align__(16) float2 psm[];
+  __shared__ double red[2][PT / 32];
+  chain_begin();
+  float2* tw = psm;
+  float2* P = psm + N;                                               // [y][z]
+  const size_t plane = (size_t)blockIdx.x * N * N;
+  for (int t = threadIdx.x; t < N; t += PT) tw[t] = twg[t];
+  for (int e = threadIdx.x; e < N * N; e += PT) P[(e / N) * ld + e % N] = w[plane + e];
+  __syncthreads();
+  x_pass<N, +1>(P, tw);                                              // y lines
+  cfft_lines<N, PT, FCfg<N>::LPC, true, +1>(P, N, ld, 1, tw);        // z lines
+  double acc[2] = {0.0, 0.0};                                        // n v_H, n v_x (FP64, as before)
+  for (int e = threadIdx.x; e < N * N; e += PT) {
+    const float nj = n[plane + e], vh = P[(e / N) * ld + e % N].x;
+    const float vx = -cbrtf(float(3.0 / M_PI) * (nj > 0.f ? nj : 0.f));
+    const float v = vloc[plane + e] + vh + vx;
+    vtot[plane + e] = v;
+    P[(e / N) * ld + e % N].x = v;
+    const double nd = (double)nj;
+    acc[0] = fma(nd, (double)vh, acc[0]);
+    acc[1] = fma(nd, (double)vx, acc[1]);
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    for (int o = 16; o > 0; o >>= 1) acc[i] += __shfl_down_sync(0xffffffffu, acc[i], o);
+    if ((threadIdx.x & 31) == 0) red[i][threadIdx.x >> 5] = acc[i];
+  }
+  __syncthreads();                                                   // the plane of V, and the sums
+  for (int e = threadIdx.x; e < N * N; e += PT) {
+    const int z = e / N, y = e % N;
+    vplane[((size_t)z * N + blockIdx.x) * N + y] = P[y * ld + z].x;
+  }
+  if (threadIdx.x == 0) {
+    double a = 0.0, b = 0.0;
+    for (int q = 0; q < PT / 32; ++q) {
+      a += red[0][q];
+      b += red[1][q];
+    }
+    partials[3 * blockIdx.x] = a;
+    partials[3 * blockIdx.x + 1] = 0.75 * b;
+    partials[3 * blockIdx.x + 2] = b;
   }
 }
 
@@ -1261,10 +1376,15 @@ class FusedImpl final : public FusedOps {
     colbuf1_ = alloc<float2>((size_t)ns_ * N_ * ncols_);
     colbuf2_ = alloc<float2>((size_t)ns_ * N_ * ncols_);
     vplane_ = alloc<float>(N3);
+    // 4 pi / |G|^2 / N^3 by |m|^2 (0 at G = 0)
+    std::vector<float> pois(3 * (N_ / 2) * (N_ / 2) + 1, 0.f);
+    const double kf = 2.0 * M_PI / g.L;
+    for (size_t m2 = 1; m2 < pois.size(); ++m2)
+      pois[m2] = (float)(4.0 * M_PI / (kf * kf * (double)m2)) * (float)(1.0 / (double)N3);
+    pois_ = upload(pois);
     if (nprojtot_ > 0) {
       B_ = alloc<float2>((size_t)nprojtot_ * g.nG);
       Bimg_ = arena_.alloc(tc_overlap_image_bytes(nprojtot_, g.nG));
-      pout_ = alloc<double2>((size_t)nprojtot_ * ns_);
       pf_ = alloc<float2>((size_t)nprojtot_ * ns_);
       part_elems_ = std::max<size_t>(tc_overlap_part_elems(nprojtot_, ns_, true), 4096);
       part_ = alloc<double2>(part_elems_);
@@ -1275,28 +1395,43 @@ class FusedImpl final : public FusedOps {
     KS_CUDA(cudaStreamSynchronize(setup_));                           // the uploaded tables have landed
   }
 
-  // The per-cell part of an H application: V re-laid per z-plane and the projections
-  // p_Il = sum_G conj(b_Il(G)) c_G of the block (tensor cores), scaled for the plane kernel.
-  void pre_h(const float2* psi, int n, const float* v, cudaStream_t s) {
-    const size_t N3 = (size_t)N_ * N_ * N_;
-    k_to_planes<<<nblk(N3, 256), 256, 0, s>>>(v, N_, vplane_);
-    KS_CHECK_LAUNCH();
+  void load_potential(const float* v, cudaStream_t s) override {
+    launch_chain(points(1), k_to_planes, dim3(nblk((size_t)N_ * N_ * N_, 256)), dim3(256), 0, s, v, N_, vplane_);
+  }
+
+  void hartree_exchange(const float* n, const float* vloc, float* vtot, float2* work, double* partials,
+                        cudaStream_t s) override {
+    dispatch([&](auto tag) {
+      constexpr int N = decltype(tag)::value;
+      static bool attr = false;
+      if (!attr) {
+        KS_CUDA(cudaFuncSetAttribute(k_hx_fwd<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plane_smem<N>()));
+        KS_CUDA(cudaFuncSetAttribute(k_hx_inv<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plane_smem<N>()));
+        attr = true;
+      }
+      launch_chain(points(1), k_hx_fwd<N>, dim3(N), dim3(FCfg<N>::PT), plane_smem<N>(), s, n, work, t_.tw);
+      launch_chain(points(1), k_hx_x<N>, dim3((N + 31) / 32, N), dim3(FCfg<N>::ZT), 0, s, work, pois_, t_.tw);
+      launch_chain(points(1), k_hx_inv<N>, dim3(N), dim3(FCfg<N>::PT), plane_smem<N>(), s, work, n, vloc, vtot, vplane_,
+                   partials, t_.tw);
+    });
+  }
+
+  // The per-cell part of an H application: the projections p_Il = sum_G conj(b_Il(G)) c_G of the
+  // block (tensor cores), scaled for the plane kernel, and the projector values they give.
+  void pre_h(const float2* psi, int n, cudaStream_t s) {
     if (nprojtot_ > 0) {
       {
         ProfScope ps(prof_, "proj_gemm", s);
-        tc_overlap(B_, g_.nG, psi, g_.nG, nprojtot_, n, g_.nG, part_, part_elems_, pout_, err_, s, nullptr, Bimg_);
-        const float scale = (float)(g_.D * std::sqrt(g_.omega));
-        k_proj_to_states<<<nblk((size_t)nprojtot_ * n, 256), 256, 0, s>>>(pout_, nprojtot_, n, scale, pf_);
-        KS_CHECK_LAUNCH();
+        tc_overlap(B_, g_.nG, psi, g_.nG, nprojtot_, n, g_.nG, part_, part_elems_, nullptr, err_, s, nullptr, Bimg_, pf_,
+                   (float)(g_.D * std::sqrt(g_.omega)));
       }
       if (npts_ > 0 && nlval_) {
         ProfScope ps(prof_, "nl_values", s);
         const dim3 grid((npts_ + 255) / 256, (n + NLB - 1) / NLB);
         if (g_.nproj == 4)
-          k_nl_values<true><<<grid, 256, 0, s>>>(pf_, nprojtot_, n, nl_, npts_, nlval_);
+          launch_chain(points(n), k_nl_values<true>, grid, dim3(256), 0, s, pf_, nprojtot_, n, nl_, npts_, nlval_);
         else
-          k_nl_values<false><<<grid, 256, 0, s>>>(pf_, nprojtot_, n, nl_, npts_, nlval_);
-        KS_CHECK_LAUNCH();
+          launch_chain(points(n), k_nl_values<false>, grid, dim3(256), 0, s, pf_, nprojtot_, n, nl_, npts_, nlval_);
       }
     }
   }
@@ -1315,7 +1450,7 @@ class FusedImpl final : public FusedOps {
       FusedImpl* f = static_cast<FusedImpl*>(it.ops);
       if (!same_geometry(f0, f)) fail(KS_ERR_ARG, "packed H application: the members' grids differ");
       if (it.n < 1 || it.n > f->ns_) fail(KS_ERR_ARG, "packed H application: member with %d states", it.n);
-      f->pre_h(it.psi, it.n, it.v, s);
+      f->pre_h(it.psi, it.n, s);
     }
     f0->dispatch([&](auto tag) { group_launch<decltype(tag)::value>(items, s); });
   }
@@ -1366,9 +1501,8 @@ class FusedImpl final : public FusedOps {
         for (size_t k = a; k < std::min(items.size(), a + GMAX); ++k) cols_ready = cols_ready && items[k].cols_ready;
         if (!cols_ready) {
           ProfScope ps(f0->prof_, "zinv", s);
-          k_zinv_group<N><<<dim3(ncb, z0), FCfg<N>::ZT, zsmem<N>(), s>>>(gd, f0->g_.nG, f0->t_.col_off,
-                                                                         f0->t_.col_half, f0->ncols_, f0->t_.tw);
-          KS_CHECK_LAUNCH();
+          launch_chain(f0->points(s0), k_zinv_group<N>, dim3(ncb, z0), dim3(FCfg<N>::ZT), zsmem<N>(), s, gd, f0->g_.nG, f0->t_.col_off,
+                       f0->t_.col_half, f0->ncols_, f0->t_.tw);
         }
         {
           ProfScope ps(f0->prof_, "plane", s);
@@ -1378,25 +1512,21 @@ class FusedImpl final : public FusedOps {
               f->template launch_plane_team_single<N>(items[k].n, s);
             }
           } else {
-            k_plane_team_group<N><<<dim3(N, s0), TCfg<N>::PT, smem, s>>>(gd, f0->ncols_, f0->t_.col_xy, f0->g_.xr,
-                                                                         f0->rowym_, f0->t_.tw);
-            KS_CHECK_LAUNCH();
+            launch_chain(f0->points(s0), k_plane_team_group<N>, dim3(N, s0), dim3(TCfg<N>::PT), smem, s, gd, f0->ncols_, f0->t_.col_xy,
+                         f0->g_.xr, f0->rowym_, f0->t_.tw);
           }
         }
         {
           ProfScope ps(f0->prof_, "zfwd", s);
-          k_zfwd_group<N><<<dim3(ncb, s0), FCfg<N>::ZT, 0, s>>>(gd, f0->g_.nG, f0->t_.col_off, f0->t_.col_half,
-                                                                f0->t_.g2half, f0->ncols_,
-                                                                (float)(1.0 / ((double)N * N * N)), f0->t_.tw);
-          KS_CHECK_LAUNCH();
+          launch_chain(f0->points(s0), k_zfwd_group<N>, dim3(ncb, s0), dim3(FCfg<N>::ZT), 0, s, gd, f0->g_.nG, f0->t_.col_off,
+                       f0->t_.col_half, f0->t_.g2half, f0->ncols_, (float)(1.0 / ((double)N * N * N)), f0->t_.tw);
         }
       }
     }
   }
 
-  void apply_h(const float2* psi, float2* hpsi, int n, const float* v, cudaStream_t s,
-               const TaylorEpi* te) override {
-    pre_h(psi, n, v, s);
+  void apply_h(const float2* psi, float2* hpsi, int n, cudaStream_t s, const TaylorEpi* te) override {
+    pre_h(psi, n, s);
     zinv(psi, n, s);
     {
       ProfScope ps(prof_, "plane", s);
@@ -1452,8 +1582,7 @@ class FusedImpl final : public FusedOps {
     }
     dispatch([&](auto tag) { launch_density<decltype(tag)::value>(n, occ, s, variant); });
     const int nch = (n + density_chunk(variant) - 1) / density_chunk(variant);
-    k_density_reduce<<<nblk((size_t)N_ * N_ * N_, 256), 256, 0, s>>>(dpartial_, nch, N_, nout);
-    KS_CHECK_LAUNCH();
+    launch_chain(points(n), k_density_reduce, dim3(nblk((size_t)N_ * N_ * N_, 256)), dim3(256), 0, s, dpartial_, nch, N_, nout);
   }
 
  private:
@@ -1477,6 +1606,8 @@ class FusedImpl final : public FusedOps {
     }
   }
 
+  size_t points(int n) const { return (size_t)n * N_ * N_ * N_; }   // grid points of n states
+
   void zinv(const float2* psi, int n, cudaStream_t s) {
     ProfScope ps(prof_, "zinv", s);
     dispatch([&](auto tag) { launch_zinv<decltype(tag)::value>(psi, n, s); });
@@ -1489,14 +1620,13 @@ class FusedImpl final : public FusedOps {
       attr = true;
     }
     dim3 grid((ncols_ + FCfg<N>::CT - 1) / FCfg<N>::CT, (n + ZSB - 1) / ZSB);
-    k_zinv<N><<<grid, FCfg<N>::ZT, zsmem<N>(), s>>>(psi, g_.nG, t_.col_off, t_.col_half, ncols_, n, colbuf1_, t_.tw);
-    KS_CHECK_LAUNCH();
+    launch_chain(points(n), k_zinv<N>, grid, dim3(FCfg<N>::ZT), zsmem<N>(), s, psi, g_.nG, t_.col_off, t_.col_half, ncols_, n,
+                 colbuf1_, t_.tw);
   }
   template <int N> void launch_zfwd(const float2* psi, float2* hpsi, int n, const TaylorEpi& te, cudaStream_t s) {
     dim3 grid((ncols_ + FCfg<N>::CT - 1) / FCfg<N>::CT, n);
-    k_zfwd<N><<<grid, FCfg<N>::ZT, 0, s>>>(colbuf2_, psi, hpsi, g_.nG, t_.col_off, t_.col_half, t_.g2half, ncols_,
-                                           (float)(1.0 / ((double)N * N * N)), t_.tw, te);
-    KS_CHECK_LAUNCH();
+    launch_chain(points(n), k_zfwd<N>, grid, dim3(FCfg<N>::ZT), 0, s, colbuf2_, psi, hpsi, g_.nG, t_.col_off, t_.col_half,
+                 t_.g2half, ncols_, (float)(1.0 / ((double)N * N * N)), t_.tw, te);
   }
   template <int N> static size_t plane_smem() { return (size_t)(N + N * (N + 1)) * sizeof(float2); }
   static constexpr size_t SMEM_MAX = 227 * 1024;
@@ -1539,8 +1669,8 @@ class FusedImpl final : public FusedOps {
           m.nl = team_nl();
           m.cap = team_cap();
           m.n = n;
-          k_plane_team_group<N><<<dim3(N, n), TCfg<N>::PT, smem, s>>>(gd, ncols_, t_.col_xy, g_.xr, rowym_, t_.tw);
-          KS_CHECK_LAUNCH();
+          launch_chain(points(n), k_plane_team_group<N>, dim3(N, n), dim3(TCfg<N>::PT), smem, s, gd, ncols_, t_.col_xy, g_.xr,
+                       rowym_, t_.tw);
           return;
         }
         if (cb1 != colbuf1_) fail(KS_ERR_ARG, "plane kernel: column buffer");
@@ -1558,9 +1688,8 @@ class FusedImpl final : public FusedOps {
     const int pf_smem = with_pf <= SMEM_MAX;
     if (base > SMEM_MAX) fail(KS_ERR_ARG, "plane kernel: %zu bytes of shared memory for N=%d", base, N);
     dim3 grid(N, n);
-    k_plane<N><<<grid, FCfg<N>::PT, pf_smem ? with_pf : base, s>>>(cb1, colbuf2_, ncols_, t_.col_xy, g_.xr,
-                                                                   vplane_, nl_, pf, nprojtot_, pf_smem, t_.tw);
-    KS_CHECK_LAUNCH();
+    launch_chain(points(n), k_plane<N>, grid, dim3(FCfg<N>::PT), pf_smem ? with_pf : base, s, cb1, colbuf2_, ncols_, t_.col_xy,
+                 g_.xr, vplane_, nl_, pf, nprojtot_, pf_smem, t_.tw);
   }
   // The single-cell team plane kernel over n states of this cell's column buffers.
   template <int N> void launch_plane_team_single(int n, cudaStream_t s) {
@@ -1572,9 +1701,8 @@ class FusedImpl final : public FusedOps {
       }
       const size_t smem = team_smem<N>(team_cap());
       if (smem > SMEM_MAX) fail(KS_ERR_ARG, "plane kernel: %zu bytes of shared memory for N=%d", smem, N);
-      k_plane_team<N><<<dim3(N, n), TCfg<N>::PT, smem, s>>>(colbuf1_, colbuf2_, ncols_, t_.col_xy, g_.xr, rowym_,
-                                                            vplane_, team_nl(), team_cap(), t_.tw);
-      KS_CHECK_LAUNCH();
+      launch_chain(points(n), k_plane_team<N>, dim3(N, n), dim3(TCfg<N>::PT), smem, s, colbuf1_, colbuf2_, ncols_, t_.col_xy,
+                   g_.xr, rowym_, vplane_, team_nl(), team_cap(), t_.tw);
     }
   }
   template <int N> void launch_plane_inverse(int n, float2* out, cudaStream_t s) {
@@ -1615,10 +1743,8 @@ class FusedImpl final : public FusedOps {
           attr = true;
         }
         const size_t tsmem = plane_smem<N>() + (N == 96 ? (size_t)N * N * sizeof(float) : 0) + N * sizeof(int);
-        k_plane_density_team<N><<<dim3(N, nch), TCfg<N>::PT, tsmem, s>>>(colbuf1_, ncols_, t_.col_xy, g_.xr, rowym_, n,
-                                                                         density_chunk(0), occ,
-                                                                         (float)(1.0 / g_.omega), dpartial_, t_.tw);
-        KS_CHECK_LAUNCH();
+        launch_chain(points(n), k_plane_density_team<N>, dim3(N, nch), dim3(TCfg<N>::PT), tsmem, s, colbuf1_, ncols_, t_.col_xy,
+                     g_.xr, rowym_, n, density_chunk(0), occ, (float)(1.0 / g_.omega), dpartial_, t_.tw);
         return;
       }
     }
@@ -1829,9 +1955,9 @@ class FusedImpl final : public FusedOps {
   float2* colbuf1_ = nullptr;
   float2* colbuf2_ = nullptr;
   float* vplane_ = nullptr;
+  const float* pois_ = nullptr;      // Poisson factor by |m|^2
   float2* B_ = nullptr;
   void* Bimg_ = nullptr;             // B_ split into bf16 hi/lo operand tiles
-  double2* pout_ = nullptr;
   float2* pf_ = nullptr;
   const int* rowym_ = nullptr;       // [2 xr + 1] column range of each band row
   const uint32_t* nlbits_ = nullptr; // [N][N][NW] covered points of each plane

@@ -39,10 +39,17 @@ struct TaylorEpi {
 class FusedOps {
  public:
   virtual ~FusedOps() = default;
-  // hpsi = H psi for n states with potential v (grid order); te (may be null): the Taylor
-  // accumulators updated by the same pass.
-  virtual void apply_h(const float2* psi, float2* hpsi, int n, const float* v, cudaStream_t s,
-                       const TaylorEpi* te = nullptr) = 0;
+  // hpsi = H psi for n states with the loaded potential; te (may be null): the Taylor accumulators
+  // updated by the same pass.
+  virtual void apply_h(const float2* psi, float2* hpsi, int n, cudaStream_t s, const TaylorEpi* te = nullptr) = 0;
+  // The potential v (grid order) of the H applications that follow, copied to the per-plane layout;
+  // called wherever the engine's potential changes, so that an H application need not.
+  virtual void load_potential(const float* v, cudaStream_t s) = 0;
+  // vtot = vloc + v_H[n] + v_x[n] (grid order; periodic Poisson, Slater exchange), loaded as
+  // load_potential does; work [N^3].  partials receives N rows of the sums over an x-plane of n v_H,
+  // n 0.75 v_x and n v_x.
+  virtual void hartree_exchange(const float* n, const float* vloc, float* vtot, float2* work, double* partials,
+                                cudaStream_t s) = 0;
   // nout = sum_k occ[k] |psi_k(r)|^2 (grid order).
   virtual void density(const float2* psi, int n, const double* occ, float* nout, cudaStream_t s) = 0;
   // out[b][z][x][y] = Omega^{1/2} psi_b(r) on the grid (plane-major: z slowest), the unscaled
@@ -57,14 +64,13 @@ class FusedOps {
   virtual void set_atoms(const DevTables<float>& t) = 0;
 };
 
-// One member of a packed H application: a block of states of one cell, its output and its
-// potential (grid order), with the Taylor accumulators of the same pass.
+// One member of a packed H application: a block of states of one cell and its output (with the cell's
+// loaded potential), and the Taylor accumulators of the same pass.
 struct FusedGroupItem {
   FusedOps* ops = nullptr;
   const float2* psi = nullptr;
   float2* hpsi = nullptr;
   int n = 0;
-  const float* v = nullptr;
   TaylorEpi te{};
   // the cell's first column buffer already holds the z transform of these n states (a density
   // of the same block was the cell's last use of it): the z-transform launch is skipped when

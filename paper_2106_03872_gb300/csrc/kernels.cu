@@ -245,6 +245,7 @@ __global__ void k_vloc_from_axes(const double* __restrict__ xyz, int natoms, int
 // Block partials of sum_j n_j (r_j - L/2) (three components), r_j = h (jx, jy, jz)
 template <typename T>
 __global__ void k_dipole_partials(const T* __restrict__ n, int N, double h, double L, double* __restrict__ partials) {
+  chain_begin();
   const size_t N3 = (size_t)N * N * N;
   double acc[3] = {0.0, 0.0, 0.0};
   for (size_t j = blockIdx.x * (size_t)blockDim.x + threadIdx.x; j < N3; j += (size_t)gridDim.x * blockDim.x) {
@@ -259,13 +260,29 @@ __global__ void k_dipole_partials(const T* __restrict__ n, int N, double h, doub
     for (int i = 0; i < 3; ++i) partials[blockIdx.x * 3 + i] = acc[i];
 }
 
-__global__ void k_dipole_finish(const double* __restrict__ partials, int nblocks, double dV, double* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s[3] = {0, 0, 0};
-    for (int b = 0; b < nblocks; ++b)
-      for (int i = 0; i < 3; ++i) s[i] += partials[b * 3 + i];
-    for (int i = 0; i < 3; ++i) out[i] = dV * s[i];
-  }
+// The sums of the block partials, one block of RED_THREADS (one thread adding 296 rows of them took
+// 40 us, as long as the passes that made them): out[i] = scale[i] sum_b partials[b NV + i].
+template <int NV> struct FinishScale {
+  double v[NV];
+};
+template <int NV>
+__global__ void __launch_bounds__(RED_THREADS)
+    k_finish_sums(const double* __restrict__ partials, int nblocks, FinishScale<NV> scale, double* __restrict__ out) {
+  chain_begin();
+  double acc[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) acc[i] = 0.0;
+  for (int b = threadIdx.x; b < nblocks; b += RED_THREADS)
+#pragma unroll
+    for (int i = 0; i < NV; ++i) acc[i] += partials[b * NV + i];
+  block_sum<NV>(acc);
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int i = 0; i < NV; ++i) out[i] = scale.v[i] * acc[i];
+}
+template <int NV>
+void finish_sums(const double* partials, int nblocks, const FinishScale<NV>& scale, double* out, cudaStream_t s) {
+  launch_chain(1, k_finish_sums<NV>, dim3(1), dim3(RED_THREADS), 0, s, partials, nblocks, scale, out);
 }
 
 template <typename T, int NP>
@@ -380,17 +397,6 @@ __global__ void k_hxc_combine(const T* __restrict__ n, const cplx<T>* __restrict
     for (int i = 0; i < 3; ++i) partials[blockIdx.x * 3 + i] = acc[i];
 }
 
-__global__ void k_hxc_finish(const double* __restrict__ partials, int nblocks, double dV, double* __restrict__ parts) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s[3] = {0, 0, 0};
-    for (int b = 0; b < nblocks; ++b)
-      for (int i = 0; i < 3; ++i) s[i] += partials[b * 3 + i];
-    parts[0] = 0.5 * dV * s[0];
-    parts[1] = dV * s[1];
-    parts[2] = dV * s[2];
-  }
-}
-
 // Linear density mixing (Sec. Ground-state solution): nin <- nin + mix (nout - nin); the
 // block partials of sum |nout - nin| (before the update) give the self-consistency residual.
 template <typename T>
@@ -429,15 +435,6 @@ __global__ void k_pulay_store(const T* __restrict__ nout, const T* __restrict__ 
   block_sum<2 + PULAY_MAX>(acc);
   if (threadIdx.x == 0)
     for (int i = 0; i < 2 + PULAY_MAX; ++i) partials[blockIdx.x * (2 + PULAY_MAX) + i] = acc[i];
-}
-
-__global__ void k_pulay_finish(const double* __restrict__ partials, int nblocks, double dV, double* __restrict__ out) {
-  const int i = threadIdx.x;
-  if (blockIdx.x == 0 && i < 2 + PULAY_MAX) {
-    double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += partials[b * (2 + PULAY_MAX) + i];
-    out[i] = dV * s;
-  }
 }
 
 // nin = sum_i a_i (n_i + mix r_i) over the history pairs
@@ -495,17 +492,10 @@ __global__ void k_teter_update(cplx<T>* __restrict__ psi, const cplx<T>* __restr
   }
 }
 
-__global__ void k_sum_partials(const double* __restrict__ partials, int nblocks, double scale, double* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += partials[b];
-    *out = scale * s;
-  }
-}
-
 template <typename T>
 __global__ void k_state_dots(const cplx<T>* __restrict__ a, const cplx<T>* __restrict__ bb, int nG,
                              double2* __restrict__ dots) {
+  chain_begin();
   const int b = blockIdx.x;
   double acc[2] = {0.0, 0.0};
   if constexpr (std::is_same<T, float>::value) {
@@ -540,14 +530,14 @@ __global__ void k_state_dots(const cplx<T>* __restrict__ a, const cplx<T>* __res
   if (threadIdx.x == 0) dots[b] = make_double2(acc[0], acc[1]);
 }
 
-__global__ void k_weighted_energy(const double2* __restrict__ dots, const double* __restrict__ occ, int nb,
-                                  const double* __restrict__ parts, double* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double e = 0;
-    for (int b = 0; b < nb; ++b) e += occ[b] * dots[b].x;
-    if (parts) e += -parts[0] + parts[1] - parts[2];
-    out[0] = e;
-  }
+__global__ void __launch_bounds__(RED_THREADS)
+    k_weighted_energy(const double2* __restrict__ dots, const double* __restrict__ occ, int nb,
+                      const double* __restrict__ parts, double* __restrict__ out) {
+  chain_begin();
+  double e[1] = {0.0};
+  for (int b = threadIdx.x; b < nb; b += RED_THREADS) e[0] += occ[b] * dots[b].x;
+  block_sum<1>(e);
+  if (threadIdx.x == 0) out[0] = parts ? e[0] - parts[0] + parts[1] - parts[2] : e[0];
 }
 
 template <typename T>
@@ -727,10 +717,9 @@ void vloc_from_axes(const double* xyz, int natoms, int N, double depth, T* v, do
 
 template <typename T>
 void dipole(const T* n, int N, double L, double* partials, int nblocks, double* out, cudaStream_t s) {
-  k_dipole_partials<T><<<nblocks, RED_THREADS, 0, s>>>(n, N, L / N, L, partials);
-  KS_CHECK_LAUNCH();
-  k_dipole_finish<<<1, 32, 0, s>>>(partials, nblocks, (L / N) * (L / N) * (L / N), out);
-  KS_CHECK_LAUNCH();
+  launch_chain((size_t)N * N * N, k_dipole_partials<T>, dim3(nblocks), dim3(RED_THREADS), 0, s, n, N, L / N, L, partials);
+  const double dV = (L / N) * (L / N) * (L / N);
+  finish_sums<3>(partials, nblocks, FinishScale<3>{{dV, dV, dV}}, out, s);
 }
 
 template <typename T>
@@ -791,8 +780,7 @@ void hxc_combine(const T* n, const cplx<T>* work, const T* vloc, T* vtot, double
 }
 
 void hxc_finish(const double* partials, int nblocks, double dV, double* parts, cudaStream_t s) {
-  k_hxc_finish<<<1, 32, 0, s>>>(partials, nblocks, dV, parts);
-  KS_CHECK_LAUNCH();
+  finish_sums<3>(partials, nblocks, FinishScale<3>{{0.5 * dV, dV, dV}}, parts, s);
 }
 
 template <typename T>
@@ -806,8 +794,9 @@ void pulay_store(const T* nout, const T* nin, T* hn, T* hr, int N3, const PulayR
                  int nblocks, double dV, double* out, cudaStream_t s) {
   k_pulay_store<T><<<nblocks, RED_THREADS, 0, s>>>(nout, nin, hn, hr, (size_t)N3, refs, partials);
   KS_CHECK_LAUNCH();
-  k_pulay_finish<<<1, 32, 0, s>>>(partials, nblocks, dV, out);
-  KS_CHECK_LAUNCH();
+  FinishScale<2 + PULAY_MAX> sc;
+  for (double& v : sc.v) v = dV;
+  finish_sums<2 + PULAY_MAX>(partials, nblocks, sc, out, s);
 }
 
 template <typename T>
@@ -868,19 +857,16 @@ void minmax(const double* v, size_t n, double* partials, int nblocks, double* ou
 }
 
 void sum_partials(const double* partials, int nblocks, double scale, double* out, cudaStream_t s) {
-  k_sum_partials<<<1, 32, 0, s>>>(partials, nblocks, scale, out);
-  KS_CHECK_LAUNCH();
+  finish_sums<1>(partials, nblocks, FinishScale<1>{{scale}}, out, s);
 }
 
 template <typename T>
 void state_dots(const cplx<T>* a, const cplx<T>* b, int nG, int nb, double2* dots, cudaStream_t s) {
-  k_state_dots<T><<<nb, RED_THREADS, 0, s>>>(a, b, nG, dots);
-  KS_CHECK_LAUNCH();
+  launch_chain(8 * (size_t)nb * nG, k_state_dots<T>, dim3(nb), dim3(RED_THREADS), 0, s, a, b, nG, dots);
 }
 
 void weighted_energy(const double2* dots, const double* occ, int nb, const double* parts, double* out, cudaStream_t s) {
-  k_weighted_energy<<<1, 32, 0, s>>>(dots, occ, nb, parts, out);
-  KS_CHECK_LAUNCH();
+  launch_chain(1, k_weighted_energy, dim3(1), dim3(RED_THREADS), 0, s, dots, occ, nb, parts, out);
 }
 
 template <typename T>

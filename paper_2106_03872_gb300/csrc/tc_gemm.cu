@@ -226,6 +226,7 @@ __global__ void __launch_bounds__(PREP ? O_THREADS_PREP : O_THREADS, PREP ? 2 : 
                  int nchunks = 0) {
   constexpr int NOP = PREP ? O_NOP_PREP : O_NOP, RING = NOP * O_OP_STAGE;
   extern __shared__ __align__(1024) unsigned char tsm[];
+  chain_begin();
   const uint32_t op0 = smem_u32(tsm);
   uint64_t* bars = reinterpret_cast<uint64_t*>(tsm + RING);
   uint32_t* slot = reinterpret_cast<uint32_t*>(tsm + RING + 128);
@@ -437,6 +438,7 @@ __global__ void __launch_bounds__(OTCfg<SAME, PREP>::THREADS, 1)
   using CF = OTCfg<SAME, PREP>;
   constexpr int NOP = OT_NOP, NRAW = CF::NRAW, NOPER = CF::NOPER;
   extern __shared__ __align__(1024) unsigned char tsm[];
+  chain_begin();
   const uint32_t op0 = smem_u32(tsm), raw0 = op0 + CF::OP_RING;
   uint64_t* bars = reinterpret_cast<uint64_t*>(tsm + CF::RING);
   uint32_t* slot = reinterpret_cast<uint32_t*>(tsm + CF::RING + 256);
@@ -850,7 +852,9 @@ __device__ __forceinline__ void two_sum_acc(float& s, float& c, float x) {
 // warp w takes partials w, w + 8, ...; the eight (sum, error) pairs are combined in a fixed
 // order, so the result is deterministic.
 __global__ void __launch_bounds__(256) k_reduce_parts_tc(const float2* __restrict__ part, int nks, int m, size_t mn,
-                                                         int n, double2* __restrict__ out, float2* __restrict__ out32) {
+                                                         int n, double2* __restrict__ out, float2* __restrict__ out32,
+                                                         float2* __restrict__ cols, float cscale) {
+  chain_begin();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const size_t e = (size_t)blockIdx.x * 32 + lane;
   __shared__ float4 red[8][32];
@@ -874,6 +878,10 @@ __global__ void __launch_bounds__(256) k_reduce_parts_tc(const float2* __restric
       ly += r.w;
     }
     const double x = (double)hx + (double)lx, y = (double)hy + (double)ly;
+    if (cols) {                                                       // cols[j][i] = cscale out[i][j], FP32
+      cols[e] = make_float2((float)(x * cscale), (float)(y * cscale));
+      return;
+    }
     const size_t o = (e % (size_t)m) * n + e / (size_t)m;             // row-major out[i][j]
     out[o] = make_double2(x, y);
     if (out32) out32[o] = make_float2((float)x, (float)y);
@@ -1035,7 +1043,8 @@ size_t tc_rotation_workspace_bytes(int m, int nin) {
 }
 
 void tc_overlap(const float2* A, int lda, const float2* B, int ldb, int m, int n, int K, double2* part,
-                size_t part_elems, double2* out, int* err, cudaStream_t s, float2* out32, const void* Aimg) {
+                size_t part_elems, double2* out, int* err, cudaStream_t s, float2* out32, const void* Aimg, float2* cols,
+                float cscale) {
   set_attrs();
   const int tm = (m + TC_M - 1) / TC_M, tn = (n + TC_N / 2 - 1) / (TC_N / 2);
   const bool same = A == B && lda == ldb && m == n && tm == 1 && tn == 1;
@@ -1060,28 +1069,29 @@ void tc_overlap(const float2* A, int lda, const float2* B, int ldb, int m, int n
   dim3 g(tn, tm, ks);
   float2* p32 = reinterpret_cast<float2*>(part);                      // FP32 partials
   // one output tile of A^H A: both operands are the same rows
+  const uint4* img = static_cast<const uint4*>(Aimg);
+  const int nchunks = Aimg ? (K + O_KC - 1) / O_KC : 0;
+  const size_t work = 8 * (size_t)n * K;                             // grid points of the states: ~8 a plane wave
   if (tma) {
     if (Aimg)
-      k_tc_overlap_tma<false, true><<<g, OTCfg<false, true>::THREADS, OTCfg<false, true>::SMEM, s>>>(
-          mp, m, n, K, kchunk, p32, err, static_cast<const uint4*>(Aimg), (K + O_KC - 1) / O_KC);
+      launch_chain(work, k_tc_overlap_tma<false, true>, g, dim3(OTCfg<false, true>::THREADS), OTCfg<false, true>::SMEM, s, mp,
+                   m, n, K, kchunk, p32, err, img, nchunks);
     else if (same)
-      k_tc_overlap_tma<true><<<g, OTCfg<true, false>::THREADS, OTCfg<true, false>::SMEM, s>>>(mp, m, n, K, kchunk, p32,
-                                                                                           err, nullptr, 0);
+      launch_chain(work, k_tc_overlap_tma<true>, g, dim3(OTCfg<true, false>::THREADS), OTCfg<true, false>::SMEM, s, mp, m, n,
+                   K, kchunk, p32, err, img, 0);
     else
-      k_tc_overlap_tma<false><<<g, OTCfg<false, false>::THREADS, OTCfg<false, false>::SMEM, s>>>(
-          mp, m, n, K, kchunk, p32, err, nullptr, 0);
+      launch_chain(work, k_tc_overlap_tma<false>, g, dim3(OTCfg<false, false>::THREADS), OTCfg<false, false>::SMEM, s, mp, m,
+                   n, K, kchunk, p32, err, img, 0);
   } else if (Aimg)
-    k_tc_overlap<false, true><<<g, O_THREADS_PREP, O_SMEM_PREP, s>>>(A, lda, B, ldb, m, n, K, kchunk, p32, err,
-                                                                static_cast<const uint4*>(Aimg),
-                                                                (K + O_KC - 1) / O_KC);
+    launch_chain(work, k_tc_overlap<false, true>, g, dim3(O_THREADS_PREP), O_SMEM_PREP, s, A, lda, B, ldb, m, n, K, kchunk,
+                 p32, err, img, nchunks);
   else if (same)
-    k_tc_overlap<true><<<g, O_THREADS, O_SMEM, s>>>(A, lda, B, ldb, m, n, K, kchunk, p32, err);
+    launch_chain(work, k_tc_overlap<true>, g, dim3(O_THREADS), O_SMEM, s, A, lda, B, ldb, m, n, K, kchunk, p32, err, img, 0);
   else
-    k_tc_overlap<false><<<g, O_THREADS, O_SMEM, s>>>(A, lda, B, ldb, m, n, K, kchunk, p32, err);
-  KS_CHECK_LAUNCH();
+    launch_chain(work, k_tc_overlap<false>, g, dim3(O_THREADS), O_SMEM, s, A, lda, B, ldb, m, n, K, kchunk, p32, err, img, 0);
   const size_t mn = (size_t)m * n;
-  k_reduce_parts_tc<<<(unsigned)((mn + 31) / 32), 256, 0, s>>>(p32, ks, m, mn, n, out, out32);
-  KS_CHECK_LAUNCH();
+  launch_chain(work, k_reduce_parts_tc, dim3((unsigned)((mn + 31) / 32)), dim3(256), 0, s, p32, ks, m, mn, n, out, out32, cols,
+               cscale);
 }
 
 namespace {
