@@ -85,14 +85,54 @@ template <typename C> __host__ __device__ __forceinline__ C mk(decltype(C::x) r,
   c.y = i;
   return c;
 }
-__host__ __device__ __forceinline__ float2 operator+(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__host__ __device__ __forceinline__ float2 operator-(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// On the device the sums, differences and products of complex64 values are packed pairs (add, mul and
+// fma on two FP32 values of one 64-bit register pair, the same roundings): half the instructions of the
+// butterflies, which are what the FFT kernels issue most.  Plane kernel per H application of 128^3 states
+// 51.4 -> 49.9 ms (8 x 512 states), of 64^3 118 -> 114 us (64 states); at 96 points the packing costs the
+// registers it saves in instructions (0.616 and 0.620 ms).
+__device__ __forceinline__ unsigned long long f2_bits(float2 a) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+  return r;
+}
+__device__ __forceinline__ float2 f2_of(unsigned long long r) {
+  float2 a;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(r));
+  return a;
+}
+__host__ __device__ __forceinline__ float2 operator+(float2 a, float2 b) {
+#ifdef __CUDA_ARCH__
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+  return f2_of(r);
+#else
+  return make_float2(a.x + b.x, a.y + b.y);
+#endif
+}
+__host__ __device__ __forceinline__ float2 operator-(float2 a, float2 b) {
+#ifdef __CUDA_ARCH__
+  unsigned long long r;
+  const float2 m = make_float2(-1.f, -1.f);
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(f2_bits(b)), "l"(f2_bits(m)), "l"(f2_bits(a)));
+  return f2_of(r);
+#else
+  return make_float2(a.x - b.x, a.y - b.y);
+#endif
+}
 __host__ __device__ __forceinline__ float2 operator*(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 __host__ __device__ __forceinline__ double2 operator+(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __host__ __device__ __forceinline__ double2 operator-(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 __host__ __device__ __forceinline__ double2 operator*(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
 
 template <typename C> __host__ __device__ __forceinline__ C cmul(C a, C b) {
+#ifdef __CUDA_ARCH__
+  if constexpr (sizeof(C) == 8) {
+    unsigned long long t, r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(f2_bits(make_float2(-a.y, a.x))), "l"(f2_bits(make_float2(b.y, b.y))));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(f2_bits(make_float2(a.x, a.y))), "l"(f2_bits(make_float2(b.x, b.x))), "l"(t));
+    return f2_of(r);
+  }
+#endif
   return mk<C>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 // conj(a) * b

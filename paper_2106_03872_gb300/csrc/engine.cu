@@ -299,6 +299,8 @@ template <typename T> class Engine final : public EngineBase {
     if (!fused_) {
       batch_ = (int)full_grid_batch<T>(N, ns_);
       grid_ = alloc<C>((size_t)batch_ * N3);
+      ginv_ = alloc<int>(N3);
+      invert_index(t_.gidx, nG, ginv_, N3, setup_);
       proj_ = alloc<C>((size_t)batch_ * std::max(1, g_.natoms) * g_.nproj);
     }
     // ---- dense LA
@@ -447,11 +449,10 @@ template <typename T> class Engine final : public EngineBase {
     for (int b0 = 0; b0 < n; b0 += batch_) {
       const int nb = std::min(batch_, n - b0);
       const C* in = psi + (size_t)b0 * g_.nG;
-      KS_CUDA(cudaMemsetAsync(grid_, 0, (size_t)nb * N3 * sizeof(C), s));
-      scatter_sphere<T>(in, grid_, t_, nb, s);
       {
         ProfScope f(prof, "fft_lines", s);
-        for (int ax = 2; ax >= 0; --ax) fft_axis<T>(grid_, nb, N, ax, +1, t_.tw, s);
+        fft_z_from_sphere<T>(in, grid_, ginv_, t_, nb, s);
+        for (int ax = 1; ax >= 0; --ax) fft_axis<T>(grid_, nb, N, ax, +1, t_.tw, s);
       }
       // grid holds psi' = Omega^{1/2} psi.  p = dV sum beta psi = dV Omega^{-1/2} sum beta psi'.
       nl_project<T>(grid_, t_, proj_, nb, T(g_.dV) * rs, s);
@@ -460,9 +461,9 @@ template <typename T> class Engine final : public EngineBase {
       nl_add<T>(grid_, t_, proj_, nb, T(g_.D * std::sqrt(g_.omega)), s);
       {
         ProfScope f(prof, "fft_lines", s);
-        for (int ax = 0; ax < 3; ++ax) fft_axis<T>(grid_, nb, N, ax, -1, t_.tw, s);
+        for (int ax = 0; ax < 2; ++ax) fft_axis<T>(grid_, nb, N, ax, -1, t_.tw, s);
+        fft_z_to_sphere<T>(grid_, in, hpsi + (size_t)b0 * g_.nG, ginv_, t_, nb, T(1.0 / double(N3)), s);
       }
-      gather_kinetic<T>(grid_, in, hpsi + (size_t)b0 * g_.nG, t_, nb, T(1.0 / double(N3)), s);
     }
   }
 
@@ -496,9 +497,8 @@ template <typename T> class Engine final : public EngineBase {
     const T scale = T(1.0 / g_.omega);
     for (int b0 = 0; b0 < n; b0 += batch_) {
       const int nb = std::min(batch_, n - b0);
-      KS_CUDA(cudaMemsetAsync(grid_, 0, (size_t)nb * N3 * sizeof(C), s));
-      scatter_sphere<T>(psi + (size_t)b0 * g_.nG, grid_, t_, nb, s);
-      for (int ax = 2; ax >= 0; --ax) fft_axis<T>(grid_, nb, N, ax, +1, t_.tw, s);
+      fft_z_from_sphere<T>(psi + (size_t)b0 * g_.nG, grid_, ginv_, t_, nb, s);
+      for (int ax = 1; ax >= 0; --ax) fft_axis<T>(grid_, nb, N, ax, +1, t_.tw, s);
       density_accumulate<T>(grid_, occ_ + b0, nout, (int)N3, nb, scale, b0 == 0, s);
     }
   }
@@ -979,6 +979,14 @@ template <typename T> class Engine final : public EngineBase {
     for (int b0 = 0; b0 < ns_; b0 += fb_) {
       const int nb = std::min(fb_, ns_ - b0);
       const C* st = psi_ + (size_t)b0 * g_.nG;
+      if constexpr (sizeof(T) == 4) {
+        if (fused_ && fused_->force_chunks()) {
+          grad_packed<T>(st, gpack, t_, 2, nb, s);
+          fused_->force_chunk(st, gpack, nb, occ_ + b0, pscale, 2.0 * g_.D, fpsi_, fp_, fq_, fg_, fnl_, s);
+          zmajor = true;
+          continue;
+        }
+      }
       auto to_grid = [&](const C* packed, C* grid, int a) {
         if constexpr (sizeof(T) == 4) {
           if (fused_) {
@@ -1004,7 +1012,7 @@ template <typename T> class Engine final : public EngineBase {
         nl_force<T>(fp_, fq_, na, np, nb, 2.0 * g_.D, occ_ + b0, fnl_, a, s);
       }
     }
-    local_force<T>(fg_, fxyz_, N, na, -g_.dV * g_.vloc_depth / g_.omega, flocp_, floc_, s, zmajor);
+    local_force<T>(fg_, fxyz_, faxis_, fcnt_, N, na, -g_.dV * g_.vloc_depth / g_.omega, flocp_, floc_, s, zmajor);
     std::vector<double> fl(3 * (size_t)na), fn(3 * (size_t)na);
     KS_CUDA(cudaMemcpyAsync(fl.data(), floc_, fl.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
     KS_CUDA(cudaMemcpyAsync(fn.data(), fnl_, fn.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1426,6 +1434,14 @@ template <typename T> class Engine final : public EngineBase {
           xyz[((size_t)I * 3 + a) * N + j] = v;
         }
     KS_CUDA(cudaMemcpyAsync(fxyz_, xyz.data(), xyz.size() * sizeof(double), cudaMemcpyHostToDevice, s));
+    // the grid indices around each atom outside which its factor is below 1e-20 (the local force's box)
+    const int hw = (int)std::ceil(g_.vloc_width * std::sqrt(2.0 * std::log(1e20)) / g_.h);
+    fcnt_ = std::min(N, 2 * hw + 2);
+    std::vector<int> first(3 * (size_t)na);
+    for (int i = 0; i < 3 * na; ++i)
+      first[i] = fcnt_ == N ? 0 : (((int)std::floor(g_.pos[i] / g_.h) - hw) % N + N) % N;
+    if (!faxis_) faxis_ = alloc<int>(std::max<size_t>(1, first.size()));
+    if (na) KS_CUDA(cudaMemcpyAsync(faxis_, first.data(), first.size() * sizeof(int), cudaMemcpyHostToDevice, s));
   }
   static double2 cmul_scalar(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -1532,6 +1548,7 @@ template <typename T> class Engine final : public EngineBase {
   C* hpsi_ = nullptr;
   double2* staging_ = nullptr;
   C* grid_ = nullptr;
+  int* ginv_ = nullptr;             // plain path: packed index of a grid point, or -1
   C* proj_ = nullptr;
   int batch_ = 1;
   double2* part_ = nullptr;
@@ -1570,6 +1587,8 @@ template <typename T> class Engine final : public EngineBase {
   T* fg_ = nullptr;
   C *fp_ = nullptr, *fq_ = nullptr;
   double *fnl_ = nullptr, *floc_ = nullptr, *flocp_ = nullptr, *fxyz_ = nullptr;
+  int* faxis_ = nullptr;            // [natoms][3] first grid index of the local potential's support
+  int fcnt_ = 0;                    // and its length
   T* hist_n_[PULAY_MAX] = {};       // Pulay history: input densities and residuals (allocated on first use)
   T* hist_r_[PULAY_MAX] = {};
   double* pulay_partials_ = nullptr;

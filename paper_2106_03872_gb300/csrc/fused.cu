@@ -1258,6 +1258,205 @@ __global__ void __launch_bounds__(FCfg<N>::PT, FCfg<N>::PMIN)
   }
 }
 
+// Planes of the forces (Eq. 11), with the density kernel's transforms: one (z-plane, chunk of states) per
+// CTA.  GRAD = false: psi to the grid [b][z][x][y].  GRAD = true: d psi, from columns scaled by i G of
+// axis `axis` (0: x, 1: y; 2: the columns hold the derivative already), and sum_b 2 f Re(conj(d psi) psi)
+// of the chunk's states to partial[chunk][z][x][y], psi read back from the grid.  Both store the values
+// at the plane's covered points to val[b][point] for the projections, so d psi never goes to the grid.
+// Full-grid stores of psi and three derivatives, four passes over the spheres in them and three passes
+// summing the products took 7.05 ms a call on 128 states of 96^3; this form @FO@.
+template <int N, bool GRAD>
+__global__ void __launch_bounds__(TCfg<N>::PT, TCfg<N>::PMIN)
+    k_plane_force_team(const float2* __restrict__ colbuf, int ncols, const int* __restrict__ col_xy, int xr,
+                       const int* __restrict__ rowym, int nstates, int chunk, const double* __restrict__ occ, int axis,
+                       float g0, float2* __restrict__ grid, float* __restrict__ partial, TeamNL nl,
+                       float2* __restrict__ val, const float2* __restrict__ twg) {
+  using TP = TPlan<N>;
+  constexpr int R1 = TP::R1, R2 = TP::R2, W = TP::W, QA = R2 / W, QB = R1 / W, NW = TCfg<N>::NW;
+  constexpr int ld = N + 1, KS = N + 1, PT = TCfg<N>::PT;
+  extern __shared__ __align__(16) float2 psm[];
+  chain_begin();
+  float2* tw = psm;
+  float2* P = tw + N;
+  float* accs = reinterpret_cast<float*>(P + N * ld);                // [x][y], each point owned by one thread
+  uint32_t* bits = reinterpret_cast<uint32_t*>(accs + (GRAD ? N * N : 0));
+  int* loff = reinterpret_cast<int*>(bits + N * NW);
+  int* yms = loff + N;
+  const int z = blockIdx.x, ch = blockIdx.y;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int team = warp / W, wi = warp - team * W;
+  const int l = team * 32 + lane;
+  const bool act = l < N;
+  for (int t = threadIdx.x; t < N; t += PT) tw[t] = twg[t];
+  for (int e = threadIdx.x; e < N * NW; e += PT) bits[e] = nl.bits[(size_t)z * N * NW + e];
+  for (int e = threadIdx.x; e < N; e += PT) loff[e] = nl.line_off[(size_t)z * (N + 1) + e];
+  const int nband = 2 * xr + 1, pt0 = nl.pt_off[z];
+  for (int g = threadIdx.x; g < nband; g += PT) yms[g] = rowym[g];
+  if (GRAD)
+    for (int e = threadIdx.x; e < N * N; e += PT) accs[e] = 0.f;
+  auto band = [&](int e) { return e <= xr || e >= N - xr; };
+  const int b0 = ch * chunk, b1 = min(nstates, b0 + chunk);
+#pragma unroll 1
+  for (int b = b0; b < b1; ++b) {
+    const float2* src = colbuf + ((size_t)b * N + z) * ncols;
+    for (int c = threadIdx.x; c < ncols; c += PT) {
+      const int xy = col_xy[c];
+      const int jx = xy / N, jy = xy - jx * N;
+      float2 v = src[c];
+      if (GRAD && axis < 2) {
+        const float G = g0 * (float)grid_freq(axis == 0 ? jx : jy, N);
+        v = make_float2(-G * v.y, G * v.x);
+      }
+      P[jx * ld + jy] = v;
+    }
+    __syncthreads();
+    team_lines<N, +1, 1>(P, nband, RowOff<N>{xr}, tw, ColMask<N>{yms});
+    __syncthreads();
+    float2* p = P + (act ? l : 0);
+    {
+      float2 v[QA][R1];
+#pragma unroll
+      for (int q = 0; q < QA; ++q) {
+        const int j = wi + W * q;
+#pragma unroll
+        for (int r = 0; r < R1; ++r) {
+          const int e = j + r * R2;
+          v[q][r] = (act && band(e)) ? p[e * KS] : make_float2(0.f, 0.f);
+        }
+        SmallDft<R1, float2>::run(v[q], +1);
+      }
+      team_bar(team, 32 * W);
+      if (act) {
+#pragma unroll
+        for (int q = 0; q < QA; ++q) {
+          const int j = wi + W * q;
+#pragma unroll
+          for (int r = 0; r < R1; ++r) p[(j * R1 + r) * KS] = v[q][r];
+        }
+      }
+      team_bar(team, 32 * W);
+    }
+    if (act) {
+      float2* plane = grid + ((size_t)b * N + z) * N * N + l;
+      float2* vb = val + (size_t)b * nl.npts + pt0 + loff[l];
+      const float f2 = GRAD ? (float)(2.0 * occ[b]) : 0.f;
+#pragma unroll
+      for (int q = 0; q < QB; ++q) {
+        const int j = wi + W * q;
+        float2 v[R2];
+#pragma unroll
+        for (int r = 0; r < R2; ++r) v[r] = p[(j + r * R1) * KS];
+#pragma unroll
+        for (int r = 1; r < R2; ++r) v[r] = cmul(v[r], twiddle<+1>(tw, j * r));
+        SmallDft<R2, float2>::run(v, +1);
+        if constexpr (GRAD) {
+          float2 u[R2];
+#pragma unroll
+          for (int r = 0; r < R2; ++r) u[r] = plane[(size_t)(j + r * R1) * N];
+#pragma unroll
+          for (int r = 0; r < R2; ++r) accs[(j + r * R1) * N + l] += f2 * (v[r].x * u[r].x + v[r].y * u[r].y);
+        } else {
+#pragma unroll
+          for (int r = 0; r < R2; ++r) plane[(size_t)(j + r * R1) * N] = v[r];
+        }
+#pragma unroll
+        for (int r = 0; r < R2; ++r) {
+          const int e = j + r * R1;
+          const uint32_t word = bits[l * NW + (e >> 5)];
+          if ((word >> (e & 31)) & 1u) {
+            int before = __popc(word & ((1u << (e & 31)) - 1u));
+#pragma unroll
+            for (int k = 0; k < NW - 1; ++k)
+              if (k < (e >> 5)) before += __popc(bits[l * NW + k]);
+            vb[before] = v[r];
+          }
+        }
+      }
+    }
+    __syncthreads();                                                  // the plane is reused
+  }
+  if (GRAD) {
+    float* out = partial + ((size_t)ch * N + z) * N * N;
+    for (int e = threadIdx.x; e < N * N; e += PT) out[e] = accs[e];
+  }
+}
+
+// fg[e] += sum_ch partial[ch][e], chunks in order
+__global__ void __launch_bounds__(256) k_add_partials(const float* __restrict__ partial, int nch, size_t N3,
+                                                      float* __restrict__ fg) {
+  chain_begin();
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < N3; e += (size_t)gridDim.x * blockDim.x) {
+    float s = fg[e];
+    for (int ch = 0; ch < nch; ++ch) s += partial[(size_t)ch * N3 + e];
+    fg[e] = s;
+  }
+}
+
+// proj[b][I][l] = scale sum over atom I's sphere points of beta_l val[b][slot], for PJB states per CTA.
+// slot and beta list the atom's points in plane order.  The products are exact (product and its rounding
+// error by fma) and summed with compensation: about FP64's precision without its pipe, which took 0.2 ms
+// per field of 128 states and 64 atoms.
+constexpr int PJB = 2;
+__device__ __forceinline__ void add_product(float& s, float& c, float a, float b) {
+  const float p = a * b, e = fmaf(a, b, -p);
+  const float t = s + p, bp = t - s;
+  c += ((s - (t - bp)) + (p - bp)) + e;
+  s = t;
+}
+template <int NP>
+__global__ void __launch_bounds__(256)
+    k_project_points(const float2* __restrict__ val, int npts, const int* __restrict__ sph_off,
+                     const int* __restrict__ slot, const float* __restrict__ beta, int natoms, int n, float scale,
+                     float2* __restrict__ proj) {
+  chain_begin();
+  __shared__ double red[8][PJB * NP * 2];
+  const int I = blockIdx.x, b0 = blockIdx.y * PJB, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float s[PJB][NP][2] = {}, c[PJB][NP][2] = {};
+  for (int q = sph_off[I] + threadIdx.x; q < sph_off[I + 1]; q += 256) {
+    const int pt = slot[q];
+    float w[NP];
+    if constexpr (NP == 4) {
+      const float4 t = *reinterpret_cast<const float4*>(beta + (size_t)q * 4);
+      w[0] = t.x;
+      w[1] = t.y;
+      w[2] = t.z;
+      w[3] = t.w;
+    } else {
+      w[0] = beta[q];
+    }
+#pragma unroll
+    for (int k = 0; k < PJB; ++k)
+      if (b0 + k < n) {
+        const float2 v = val[(size_t)(b0 + k) * npts + pt];
+#pragma unroll
+        for (int l = 0; l < NP; ++l) {
+          add_product(s[k][l][0], c[k][l][0], w[l], v.x);
+          add_product(s[k][l][1], c[k][l][1], w[l], v.y);
+        }
+      }
+  }
+#pragma unroll
+  for (int k = 0; k < PJB; ++k)
+#pragma unroll
+    for (int l = 0; l < NP; ++l)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        double t = (double)s[k][l][h] + (double)c[k][l][h];
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+        if (lane == 0) red[warp][(k * NP + l) * 2 + h] = t;
+      }
+  __syncthreads();
+  const int e = threadIdx.x;                                         // (k, l)
+  if (e < PJB * NP && b0 + e / NP < n) {
+    double x = 0.0, y = 0.0;
+    for (int w = 0; w < 8; ++w) {
+      x += red[w][2 * e];
+      y += red[w][2 * e + 1];
+    }
+    proj[((size_t)(b0 + e / NP) * natoms + I) * NP + e % NP] = make_float2((float)(x * scale), (float)(y * scale));
+  }
+}
+
 // Setup: projector grid functions -> sphere coefficients (FP64), then rounded to complex64.
 // The projector block by a separable DFT over each atom's box of grid points (Sec.
 // "Pseudopotentials": beta_Il lives on the sphere |r - R_I| < R_c, so its sphere coefficients
@@ -1549,6 +1748,54 @@ class FusedImpl final : public FusedOps {
     dispatch([&](auto tag) { launch_plane_inverse<decltype(tag)::value>(n, out, s); });
   }
 
+  bool force_chunks() const override { return team_density() && nlval_; }
+  void force_chunk(const float2* psi, const float2* gz, int n, const double* occ, float pscale, double w, float2* grid,
+                   float2* p, float2* q, float* fg, double* fnl, cudaStream_t s) override {
+    const size_t N3 = (size_t)N_ * N_ * N_;
+    const int chunk = density_chunk(0), nch = (n + chunk - 1) / chunk;
+    const float g0 = (float)(2.0 * M_PI / g_.L);
+    dispatch([&](auto tag) {
+      constexpr int N = decltype(tag)::value;
+      if constexpr (TPlan<N>::ok) {
+        const size_t tables = (size_t)N * TCfg<N>::NW * 4 + 2 * (size_t)N * sizeof(int);
+        const size_t smem0 = plane_smem<N>() + tables, smem1 = smem0 + (size_t)N * N * sizeof(float);
+        static bool attr = false;
+        if (!attr) {
+          KS_CUDA(cudaFuncSetAttribute(k_plane_force_team<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem0));
+          KS_CUDA(cudaFuncSetAttribute(k_plane_force_team<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem1));
+          attr = true;
+        }
+        launch_zinv<N>(psi, n, colbuf1_, s);
+        launch_zinv<N>(gz, n, colbuf2_, s);
+        // psi one state per CTA (no sum over states), the derivatives a chunk
+        launch_chain(points(n), k_plane_force_team<N, false>, dim3(N, n), dim3(TCfg<N>::PT), smem0, s, colbuf1_, ncols_,
+                     t_.col_xy, g_.xr, rowym_, n, 1, occ, 0, g0, grid, dpartial_, team_nl(), nlval_, t_.tw);
+        project(n, pscale, p, s);
+        for (int a = 0; a < 3; ++a) {
+          launch_chain(points(n), k_plane_force_team<N, true>, dim3(N, nch), dim3(TCfg<N>::PT), smem1, s,
+                       a == 2 ? colbuf2_ : colbuf1_, ncols_, t_.col_xy, g_.xr, rowym_, n, chunk, occ, a, g0, grid,
+                       dpartial_, team_nl(), nlval_, t_.tw);
+          launch_chain(points(nch), k_add_partials, dim3(nblk(N3, 256)), dim3(256), 0, s, dpartial_, nch, N3, fg + a * N3);
+          project(n, pscale, q, s);
+          nl_force<float>(p, q, g_.natoms, g_.nproj, n, w, occ, fnl, a, s);
+        }
+      }
+    });
+  }
+
+  // The projections of the covered-point values in nlval_ (n states).
+  void project(int n, float pscale, float2* out, cudaStream_t s) {
+    const dim3 grid(g_.natoms, (n + PJB - 1) / PJB);
+    if (g_.nproj == 4)
+      launch_chain(points(n), k_project_points<4>, grid, dim3(256), 0, s, nlval_, npts_, t_.sph_off, sph_slot_, sph_bz_,
+                   g_.natoms, n, pscale, out);
+    else
+      launch_chain(points(n), k_project_points<1>, grid, dim3(256), 0, s, nlval_, npts_, t_.sph_off, sph_slot_, sph_bz_,
+                   g_.natoms, n, pscale, out);
+  }
+
   void prepare_atoms() override {
     plane_lists_host();
     lists_ready_ = true;
@@ -1565,6 +1812,8 @@ class FusedImpl final : public FusedOps {
     arena_.release(nl_.ent_beta);
     arena_.release(nl_.line_off);
     arena_.release(nlbits_);
+    arena_.release(sph_slot_);
+    arena_.release(sph_bz_);
     upload_plane_lists();
     if (nprojtot_ > 0) build_projector_block();
     KS_CUDA(cudaStreamSynchronize(setup_));                           // the new lists have landed
@@ -1610,10 +1859,10 @@ class FusedImpl final : public FusedOps {
 
   void zinv(const float2* psi, int n, cudaStream_t s) {
     ProfScope ps(prof_, "zinv", s);
-    dispatch([&](auto tag) { launch_zinv<decltype(tag)::value>(psi, n, s); });
+    dispatch([&](auto tag) { launch_zinv<decltype(tag)::value>(psi, n, colbuf1_, s); });
   }
 
-  template <int N> void launch_zinv(const float2* psi, int n, cudaStream_t s) {
+  template <int N> void launch_zinv(const float2* psi, int n, float2* cols, cudaStream_t s) {
     static bool attr = false;
     if (!attr) {
       KS_CUDA(cudaFuncSetAttribute(k_zinv<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zsmem<N>()));
@@ -1621,7 +1870,7 @@ class FusedImpl final : public FusedOps {
     }
     dim3 grid((ncols_ + FCfg<N>::CT - 1) / FCfg<N>::CT, (n + ZSB - 1) / ZSB);
     launch_chain(points(n), k_zinv<N>, grid, dim3(FCfg<N>::ZT), zsmem<N>(), s, psi, g_.nG, t_.col_off, t_.col_half, ncols_, n,
-                 colbuf1_, t_.tw);
+                 cols, t_.tw);
   }
   template <int N> void launch_zfwd(const float2* psi, float2* hpsi, int n, const TaylorEpi& te, cudaStream_t s) {
     dim3 grid((ncols_ + FCfg<N>::CT - 1) / FCfg<N>::CT, n);
@@ -1782,6 +2031,7 @@ class FusedImpl final : public FusedOps {
     std::vector<int>& ent_off = h_ent_off_;
     std::vector<int>& ent_proj = h_ent_proj_;
     std::vector<float>& ent_beta = h_ent_beta_;
+    std::vector<int> slot_of(g.sph_idx.size(), 0);                    // covered point of each sphere point
     pt_off.assign(N_ + 1, 0);
     pt_xy.clear();
     ent_off.assign(1, 0);
@@ -1808,6 +2058,7 @@ class FusedImpl final : public FusedOps {
         pt_xy.push_back(g.cov_idx[c] / N_);
         for (int e = g.cov_off[c]; e < g.cov_off[c + 1]; ++e) {
           const int p = g.cov_ent[e];
+          slot_of[p] = (int)pt_xy.size() - 1;
           ent_proj.push_back(g.sph_atom[p] * g.nproj);
           for (int l = 0; l < g.nproj; ++l) ent_beta.push_back((float)g.sph_beta[(size_t)p * g.nproj + l]);
         }
@@ -1815,8 +2066,18 @@ class FusedImpl final : public FusedOps {
       }
       pt_off[z + 1] = (int)pt_xy.size();
     }
+    // each atom's sphere points in plane order: their covered points and beta values (forces)
+    h_sph_slot_.resize(g.sph_zorder.size());
+    h_sph_bz_.resize(g.sph_zorder.size() * g.nproj);
+    for (size_t q = 0; q < g.sph_zorder.size(); ++q) {
+      const int p = g.sph_zorder[q];
+      h_sph_slot_[q] = slot_of[p];
+      for (int l = 0; l < g.nproj; ++l) h_sph_bz_[q * g.nproj + l] = (float)g.sph_beta[(size_t)p * g.nproj + l];
+    }
   }
   void upload_plane_lists() {
+    sph_slot_ = upload(h_sph_slot_);
+    sph_bz_ = upload(h_sph_bz_);
     nl_.pt_off = upload(h_pt_off_);
     nl_.pt_xy = upload(h_pt_xy_);
     nl_.ent_off = upload(h_ent_off_);
@@ -1951,6 +2212,10 @@ class FusedImpl final : public FusedOps {
   std::vector<float> h_ent_beta_;
   std::vector<int> h_line_off_;       // [N][N+1] per-plane y-line offsets of the covered points
   int nl_cap_ = 0;                    // most covered points of any plane
+  std::vector<int> h_sph_slot_;
+  std::vector<float> h_sph_bz_;
+  const int* sph_slot_ = nullptr;     // [npts_sph] covered point of each atom's sphere points, plane order
+  const float* sph_bz_ = nullptr;     // [npts_sph][nproj] their beta values
   bool lists_ready_ = false;
   float2* colbuf1_ = nullptr;
   float2* colbuf2_ = nullptr;

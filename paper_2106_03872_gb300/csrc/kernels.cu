@@ -39,12 +39,27 @@ __device__ __forceinline__ void block_sum(double (&v)[NV]) {
 // Line FFTs along one axis of [nb][N][N][N] grids.
 // Lines are addressed as (outer a, inner b): element k at a*N*B + k*B + b.
 // ------------------------------------------------------------------------------------------
-template <typename T>
+// Packed sphere coefficients at either end of a z pass (axis 2): ginv [N^3] is the packed index of a grid
+// point, or -1.  Reading them there saves the grid's clearing and the scatter, and keeping only S on the
+// way out the gather with the kinetic term: three launches and two passes over the grids of an H
+// application.
+template <typename T> struct SphereEnd {
+  const int* ginv = nullptr;
+  const cplx<T>* psi = nullptr;    // packed states [b][nG] (read: the transform's input; written: T c)
+  cplx<T>* hpsi = nullptr;         // written: scale u + |G|^2/2 c
+  const T* g2h = nullptr;
+  int nG = 0;
+  T scale{};
+};
+enum { LINES_GRID, LINES_FROM_SPHERE, LINES_TO_SPHERE };
+
+template <typename T, int MODE>
 __global__ void __launch_bounds__(LINE_THREADS) k_fft_lines(cplx<T>* __restrict__ data, int N, long nouter, int B,
                                                             int TB, FftPlan plan, const cplx<T>* __restrict__ twg,
-                                                            int sign) {
+                                                            int sign, SphereEnd<T> sp) {
   using C = cplx<T>;
   extern __shared__ unsigned char smem_raw[];
+  chain_begin();
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* s = tw + N;
   const int ld = N + 1;
@@ -54,13 +69,20 @@ __global__ void __launch_bounds__(LINE_THREADS) k_fft_lines(cplx<T>* __restrict_
   }
   int lines;
   size_t base;
+  long a0 = 0;
   if (B == 1) {
-    const long a0 = (long)blockIdx.x * TB;
+    a0 = (long)blockIdx.x * TB;
     lines = (int)min((long)TB, nouter - a0);
     base = (size_t)a0 * N;
     for (int e = threadIdx.x; e < lines * N; e += blockDim.x) {
       const int l = e / N, k = e - (e / N) * N;
-      s[l * ld + k] = data[base + (size_t)l * N + k];
+      if constexpr (MODE == LINES_FROM_SPHERE) {
+        const long line = a0 + l, st = line / ((long)N * N);
+        const int g = sp.ginv[(line - st * N * N) * N + k];
+        s[l * ld + k] = g >= 0 ? sp.psi[(size_t)st * sp.nG + g] : mk<C>(T(0), T(0));
+      } else {
+        s[l * ld + k] = data[base + (size_t)l * N + k];
+      }
     }
   } else {
     const int ntb = (B + TB - 1) / TB;
@@ -78,7 +100,19 @@ __global__ void __launch_bounds__(LINE_THREADS) k_fft_lines(cplx<T>* __restrict_
   if (B == 1) {
     for (int e = threadIdx.x; e < lines * N; e += blockDim.x) {
       const int l = e / N, k = e - (e / N) * N;
-      data[base + (size_t)l * N + k] = s[l * ld + k];
+      const C u = s[l * ld + k];
+      if constexpr (MODE == LINES_TO_SPHERE) {
+        const long line = a0 + l, st = line / ((long)N * N);
+        const int g = sp.ginv[(line - st * N * N) * N + k];
+        if (g >= 0) {
+          const size_t i = (size_t)st * sp.nG + g;
+          const C c = sp.psi[i];
+          const T kin = sp.g2h[g];
+          sp.hpsi[i] = mk<C>(u.x * sp.scale + kin * c.x, u.y * sp.scale + kin * c.y);
+        }
+      } else {
+        data[base + (size_t)l * N + k] = u;
+      }
     }
   } else {
     for (int e = threadIdx.x; e < lines * N; e += blockDim.x) {
@@ -86,6 +120,10 @@ __global__ void __launch_bounds__(LINE_THREADS) k_fft_lines(cplx<T>* __restrict_
       data[base + (size_t)k * B + l] = s[l * ld + k];
     }
   }
+}
+
+__global__ void k_invert_index(const int* __restrict__ gidx, int nG, int* __restrict__ ginv) {
+  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < nG; g += gridDim.x * blockDim.x) ginv[gidx[g]] = g;
 }
 
 template <typename T>
@@ -115,6 +153,7 @@ __global__ void k_gather_kinetic(const cplx<T>* __restrict__ grid, const cplx<T>
 
 template <typename T>
 __global__ void k_multiply_potential(cplx<T>* __restrict__ grid, const T* __restrict__ v, size_t N3) {
+  chain_begin();
   const int b = blockIdx.y;
   for (size_t j = blockIdx.x * (size_t)blockDim.x + threadIdx.x; j < N3; j += (size_t)gridDim.x * blockDim.x) {
     const T vj = v[j];
@@ -171,44 +210,65 @@ __global__ void k_grad_accumulate(const cplx<T>* __restrict__ dpsi, const cplx<T
   }
 }
 
-// fnl[3 I + alpha] -= w sum_b occ[b] sum_l Re(conj(q_bIl) p_bIl), one thread per atom (states in order)
+// fnl[3 I + alpha] -= w sum_b occ[b] sum_l Re(conj(q_bIl) p_bIl), one block per atom (one thread per
+// atom walked the states' dependent loads alone: 128 states of 64 atoms took 0.1 ms)
 template <typename T>
-__global__ void k_nl_force(const cplx<T>* __restrict__ p, const cplx<T>* __restrict__ q, int natoms, int nproj, int nb,
-                           double w, const double* __restrict__ occ, double* __restrict__ fnl, int alpha) {
-  const int I = blockIdx.x * blockDim.x + threadIdx.x;
-  if (I >= natoms) return;
-  double s = 0.0;
-  for (int b = 0; b < nb; ++b) {
+__global__ void __launch_bounds__(128)
+    k_nl_force(const cplx<T>* __restrict__ p, const cplx<T>* __restrict__ q, int natoms, int nproj, int nb, double w,
+               const double* __restrict__ occ, double* __restrict__ fnl, int alpha) {
+  chain_begin();
+  const int I = blockIdx.x;
+  double s[1] = {0.0};
+  for (int b = threadIdx.x; b < nb; b += blockDim.x) {
     double sb = 0.0;
     for (int l = 0; l < nproj; ++l) {
       const size_t e = ((size_t)b * natoms + I) * nproj + l;
       const cplx<T> a = p[e], c = q[e];
       sb += (double)c.x * (double)a.x + (double)c.y * (double)a.y;
     }
-    s += occ[b] * sb;
+    s[0] += occ[b] * sb;
   }
-  fnl[3 * I + alpha] -= w * s;
+  block_sum<1>(s);
+  if (threadIdx.x == 0) fnl[3 * I + alpha] -= w * s[0];
 }
 
-// floc[3 I + a] = coef sum_j X_I[jx] Y_I[jy] Z_I[jz] g_a[j], one block per atom; xyz holds per
-// atom the three per-axis image sums [natoms][3][N] of the separable Gaussian
+// floc[3 I + a] = coef sum_j X_I[jx] Y_I[jy] Z_I[jz] g_a[j]; xyz holds per atom the three per-axis
+// image sums [natoms][3][N] of the separable Gaussian, start [natoms][3] the first of the `cnt` grid
+// indices (mod N) around the atom outside which every factor is below 1e-20.  A warp per grid row of the
+// atom's box: the row's sum with the inner axis' factors, then one product with the two others'.  FP64
+// throughout, so the FP64 pipe bounds it: over the whole grid with a product per point, the 64 atoms of a
+// 96^3 cell took 0.72 ms.
 template <typename T>
-__global__ void k_local_force(const T* __restrict__ g, const double* __restrict__ xyz, int N, double coef,
-                              double* __restrict__ partials, int zmajor) {
-  const int I = blockIdx.x, sl = blockIdx.y;
+__global__ void __launch_bounds__(RED_THREADS)
+    k_local_force(const T* __restrict__ g, const double* __restrict__ xyz, const int* __restrict__ start, int cnt, int N,
+                  double coef, double* __restrict__ partials, int zmajor) {
+  chain_begin();
+  const int I = blockIdx.x, sl = blockIdx.y, lane = threadIdx.x & 31;
   const size_t N3 = (size_t)N * N * N;
-  const size_t j0 = N3 * sl / LOCAL_FORCE_SPLIT, j1 = N3 * (sl + 1) / LOCAL_FORCE_SPLIT;
-  const double* X = xyz + (size_t)I * 3 * N;
-  const double* Y = X + N;
-  const double* Z = Y + N;
+  // axes of the memory order, slowest first: [z][x][y] or [x][y][z]
+  const int ax2 = zmajor ? 2 : 0, ax1 = zmajor ? 0 : 1, ax0 = zmajor ? 1 : 2;
+  const double *T2 = xyz + ((size_t)I * 3 + ax2) * N, *T1 = xyz + ((size_t)I * 3 + ax1) * N,
+               *T0 = xyz + ((size_t)I * 3 + ax0) * N;
+  const int s2 = start[3 * I + ax2], s1 = start[3 * I + ax1], s0 = start[3 * I + ax0];
   double acc[3] = {0.0, 0.0, 0.0};
-  for (size_t j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-    const int a0 = (int)(j % N), a1 = (int)((j / N) % N), a2 = (int)(j / ((size_t)N * N));
-    const int jz = zmajor ? a2 : a0, jy = zmajor ? a0 : a1, jx = zmajor ? a1 : a2;
-    const double v = X[jx] * Y[jy] * Z[jz];
-    acc[0] += v * (double)g[j];
-    acc[1] += v * (double)g[N3 + j];
-    acc[2] += v * (double)g[2 * N3 + j];
+  const int rows = cnt * cnt, r0 = rows * sl / LOCAL_FORCE_SPLIT, r1 = rows * (sl + 1) / LOCAL_FORCE_SPLIT;
+  for (int r = r0 + (threadIdx.x >> 5); r < r1; r += RED_THREADS / 32) {
+    int j2 = s2 + r / cnt, j1 = s1 + r % cnt;
+    if (j2 >= N) j2 -= N;
+    if (j1 >= N) j1 -= N;
+    const T* row = g + ((size_t)j2 * N + j1) * N;
+    double t[3] = {0.0, 0.0, 0.0};
+    for (int i = lane; i < cnt; i += 32) {
+      int j0 = s0 + i;
+      if (j0 >= N) j0 -= N;
+      const double f = T0[j0];
+      t[0] = fma(f, (double)row[j0], t[0]);
+      t[1] = fma(f, (double)row[N3 + j0], t[1]);
+      t[2] = fma(f, (double)row[2 * N3 + j0], t[2]);
+    }
+    const double v = T2[j2] * T1[j1];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) acc[a] = fma(v, t[a], acc[a]);
   }
   block_sum<3>(acc);
   if (threadIdx.x == 0)
@@ -216,6 +276,7 @@ __global__ void k_local_force(const T* __restrict__ g, const double* __restrict_
 }
 
 __global__ void k_local_force_finish(const double* __restrict__ partials, int natoms, double* __restrict__ floc) {
+  chain_begin();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;                // 3 I + a
   if (e >= 3 * natoms) return;
   const int I = e / 3, a = e % 3;
@@ -289,6 +350,7 @@ template <typename T, int NP>
 __global__ void k_nl_project(const cplx<T>* __restrict__ grid, size_t N3, const int* __restrict__ sph_off,
                              const int* __restrict__ sph_idx, const T* __restrict__ beta, int natoms,
                              cplx<T>* __restrict__ proj, T scale, int zmajor_n, const int* __restrict__ zorder) {
+  chain_begin();
   const int I = blockIdx.x, b = blockIdx.y;
   double acc[2 * NP];
 #pragma unroll
@@ -321,6 +383,7 @@ __global__ void k_nl_add(cplx<T>* __restrict__ grid, size_t N3, int ncov, const 
                          const int* __restrict__ cov_off, const int* __restrict__ cov_ent,
                          const int* __restrict__ sph_atom, const T* __restrict__ beta, int natoms,
                          const cplx<T>* __restrict__ proj, T scale) {
+  chain_begin();
   const int b = blockIdx.y;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncov; c += gridDim.x * blockDim.x) {
     T ax = 0, ay = 0;
@@ -605,26 +668,55 @@ inline unsigned blocks_for(size_t n, int threads, unsigned cap = 152u * 16u) {
 // ------------------------------------------------------------------------------------------
 // Launchers
 // ------------------------------------------------------------------------------------------
+// Lines per CTA: as many as its shared memory holds, but fewer where the launch would leave
+// multiprocessors without a CTA (24^3 with 8 states: 54 CTAs of 85 lines took 18 us a pass in FP64, whose
+// pipe on every SM needs 4 us); at least 16 of a strided pass, whose rows are then 128 or 256 bytes.
+template <typename T, int MODE>
+static void fft_lines(cplx<T>* grid, int nb, int N, int axis, int sign, const cplx<T>* tw, const SphereEnd<T>& sp,
+                      cudaStream_t s) {
+  const FftPlan plan = make_plan(N);
+  const long nouter = axis == 2 ? (long)nb * N * N : (axis == 1 ? (long)nb * N : nb);
+  const int B = axis == 2 ? 1 : (axis == 1 ? N : N * N);
+  const long lines = (long)nb * N * N;
+  int TB = std::max(1, std::min<int>(LINE_ELEMS / N, (int)std::max<long>(16, lines / (2 * 152))));
+  if (B > 1 && TB > B) TB = B;
+  const long nblocks = (B == 1) ? (nouter + TB - 1) / TB : nouter * ((B + TB - 1) / TB);
+  const size_t smem = (size_t)(N + TB * (N + 1)) * sizeof(cplx<T>);
+  launch_chain((size_t)lines * N, k_fft_lines<T, MODE>, dim3((unsigned)nblocks), dim3(LINE_THREADS), smem, s, grid, N,
+               nouter, B, TB, plan, tw, sign, sp);
+}
+
 template <typename T>
 void fft_axis(cplx<T>* grid, int nb, int N, int axis, int sign, const cplx<T>* tw, cudaStream_t s) {
-  const FftPlan plan = make_plan(N);
-  long nouter;
-  int B;
-  if (axis == 2) {
-    nouter = (long)nb * N * N;
-    B = 1;
-  } else if (axis == 1) {
-    nouter = (long)nb * N;
-    B = N;
-  } else {
-    nouter = nb;
-    B = N * N;
-  }
-  int TB = LINE_ELEMS / N;
-  if (B > 1 && TB > B) TB = B;
-  long nblocks = (B == 1) ? (nouter + TB - 1) / TB : nouter * ((B + TB - 1) / TB);
-  const size_t smem = (size_t)(N + TB * (N + 1)) * sizeof(cplx<T>);
-  k_fft_lines<T><<<(unsigned)nblocks, LINE_THREADS, smem, s>>>(grid, N, nouter, B, TB, plan, tw, sign);
+  fft_lines<T, LINES_GRID>(grid, nb, N, axis, sign, tw, SphereEnd<T>{}, s);
+}
+
+template <typename T>
+void fft_z_from_sphere(const cplx<T>* psi, cplx<T>* grid, const int* ginv, const DevTables<T>& t, int nb,
+                       cudaStream_t s) {
+  SphereEnd<T> sp;
+  sp.ginv = ginv;
+  sp.psi = psi;
+  sp.nG = t.nG;
+  fft_lines<T, LINES_FROM_SPHERE>(grid, nb, t.N, 2, +1, t.tw, sp, s);
+}
+
+template <typename T>
+void fft_z_to_sphere(cplx<T>* grid, const cplx<T>* psi, cplx<T>* hpsi, const int* ginv, const DevTables<T>& t, int nb,
+                     T scale, cudaStream_t s) {
+  SphereEnd<T> sp;
+  sp.ginv = ginv;
+  sp.psi = psi;
+  sp.hpsi = hpsi;
+  sp.g2h = t.g2half;
+  sp.nG = t.nG;
+  sp.scale = scale;
+  fft_lines<T, LINES_TO_SPHERE>(grid, nb, t.N, 2, -1, t.tw, sp, s);
+}
+
+void invert_index(const int* gidx, int nG, int* ginv, size_t N3, cudaStream_t s) {
+  KS_CUDA(cudaMemsetAsync(ginv, 0xff, N3 * sizeof(int), s));
+  k_invert_index<<<blocks_for((size_t)nG, 256), 256, 0, s>>>(gidx, nG, ginv);
   KS_CHECK_LAUNCH();
 }
 
@@ -646,8 +738,7 @@ void gather_kinetic(const cplx<T>* grid, const cplx<T>* psi, cplx<T>* hpsi, cons
 template <typename T>
 void multiply_potential(cplx<T>* grid, const T* v, int N3, int nb, cudaStream_t s) {
   dim3 g(blocks_for(N3, 256, 2048), nb);
-  k_multiply_potential<T><<<g, 256, 0, s>>>(grid, v, (size_t)N3);
-  KS_CHECK_LAUNCH();
+  launch_chain((size_t)N3 * nb, k_multiply_potential<T>, g, dim3(256), 0, s, grid, v, (size_t)N3);
 }
 
 template <typename T>
@@ -675,17 +766,17 @@ void grad_accumulate(const cplx<T>* dpsi, const cplx<T>* psi, T* gacc, int N3, i
 template <typename T>
 void nl_force(const cplx<T>* p, const cplx<T>* q, int natoms, int nproj, int nb, double w, const double* occ,
               double* fnl, int alpha, cudaStream_t s) {
-  k_nl_force<T><<<(natoms + 127) / 128, 128, 0, s>>>(p, q, natoms, nproj, nb, w, occ, fnl, alpha);
-  KS_CHECK_LAUNCH();
+  launch_chain((size_t)natoms * nproj * nb, k_nl_force<T>, dim3(natoms), dim3(128), 0, s, p, q, natoms, nproj, nb, w,
+               occ, fnl, alpha);
 }
 
 template <typename T>
-void local_force(const T* g, const double* xyz, int N, int natoms, double coef, double* partials, double* floc,
-                 cudaStream_t s, bool zmajor) {
-  k_local_force<T><<<dim3(natoms, LOCAL_FORCE_SPLIT), RED_THREADS, 0, s>>>(g, xyz, N, coef, partials, zmajor ? 1 : 0);
-  KS_CHECK_LAUNCH();
-  k_local_force_finish<<<(3 * natoms + 127) / 128, 128, 0, s>>>(partials, natoms, floc);
-  KS_CHECK_LAUNCH();
+void local_force(const T* g, const double* xyz, const int* start, int cnt, int N, int natoms, double coef,
+                 double* partials, double* floc, cudaStream_t s, bool zmajor) {
+  const size_t box = (size_t)natoms * cnt * cnt * cnt;
+  launch_chain(box, k_local_force<T>, dim3(natoms, LOCAL_FORCE_SPLIT), dim3(RED_THREADS), 0, s, g, xyz, start, cnt, N,
+               coef, partials, zmajor ? 1 : 0);
+  launch_chain(1, k_local_force_finish, dim3((3 * natoms + 127) / 128), dim3(128), 0, s, partials, natoms, floc);
 }
 
 template <typename T>
@@ -730,12 +821,11 @@ void nl_project(const cplx<T>* grid, const DevTables<T>& t, cplx<T>* proj, int n
   const size_t N3 = (size_t)t.N * t.N * t.N;
   const int zn = zmajor ? t.N : 0;
   if (t.nproj == 4)
-    k_nl_project<T, 4><<<g, RED_THREADS, 0, s>>>(grid, N3, t.sph_off, t.sph_idx, t.sph_beta, t.natoms, proj, scale, zn,
-                                                 t.sph_zorder);
+    launch_chain(N3 * nb, k_nl_project<T, 4>, g, dim3(RED_THREADS), 0, s, grid, N3, t.sph_off, t.sph_idx, t.sph_beta,
+                 t.natoms, proj, scale, zn, t.sph_zorder);
   else
-    k_nl_project<T, 1><<<g, RED_THREADS, 0, s>>>(grid, N3, t.sph_off, t.sph_idx, t.sph_beta, t.natoms, proj, scale, zn,
-                                                 t.sph_zorder);
-  KS_CHECK_LAUNCH();
+    launch_chain(N3 * nb, k_nl_project<T, 1>, g, dim3(RED_THREADS), 0, s, grid, N3, t.sph_off, t.sph_idx, t.sph_beta,
+                 t.natoms, proj, scale, zn, t.sph_zorder);
 }
 
 template <typename T>
@@ -744,12 +834,11 @@ void nl_add(cplx<T>* grid, const DevTables<T>& t, const cplx<T>* proj, int nb, T
   dim3 g(blocks_for(t.ncov, 256, 1024), nb);
   const size_t N3 = (size_t)t.N * t.N * t.N;
   if (t.nproj == 4)
-    k_nl_add<T, 4><<<g, 256, 0, s>>>(grid, N3, t.ncov, t.cov_idx, t.cov_off, t.cov_ent, t.sph_atom, t.sph_beta,
-                                     t.natoms, proj, scale);
+    launch_chain(N3 * nb, k_nl_add<T, 4>, g, dim3(256), 0, s, grid, N3, t.ncov, t.cov_idx, t.cov_off, t.cov_ent,
+                 t.sph_atom, t.sph_beta, t.natoms, proj, scale);
   else
-    k_nl_add<T, 1><<<g, 256, 0, s>>>(grid, N3, t.ncov, t.cov_idx, t.cov_off, t.cov_ent, t.sph_atom, t.sph_beta,
-                                     t.natoms, proj, scale);
-  KS_CHECK_LAUNCH();
+    launch_chain(N3 * nb, k_nl_add<T, 1>, g, dim3(256), 0, s, grid, N3, t.ncov, t.cov_idx, t.cov_off, t.cov_ent,
+                 t.sph_atom, t.sph_beta, t.natoms, proj, scale);
 }
 
 template <typename T>
@@ -901,6 +990,9 @@ void real_to_double(const T* in, double* out, size_t n, cudaStream_t s) {
 
 #define KS_INSTANTIATE(T)                                                                                       \
   template void fft_axis<T>(cplx<T>*, int, int, int, int, const cplx<T>*, cudaStream_t);                        \
+  template void fft_z_from_sphere<T>(const cplx<T>*, cplx<T>*, const int*, const DevTables<T>&, int, cudaStream_t); \
+  template void fft_z_to_sphere<T>(cplx<T>*, const cplx<T>*, cplx<T>*, const int*, const DevTables<T>&, int, T, \
+                                   cudaStream_t);                                                               \
   template void scatter_sphere<T>(const cplx<T>*, cplx<T>*, const DevTables<T>&, int, cudaStream_t);            \
   template void gather_kinetic<T>(const cplx<T>*, const cplx<T>*, cplx<T>*, const DevTables<T>&, int, T,        \
                                   cudaStream_t);                                                                \
@@ -924,7 +1016,8 @@ void real_to_double(const T* in, double* out, size_t n, cudaStream_t s) {
   template void grad_accumulate<T>(const cplx<T>*, const cplx<T>*, T*, int, int, const double*, cudaStream_t);  \
   template void nl_force<T>(const cplx<T>*, const cplx<T>*, int, int, int, double, const double*, double*, int,  \
                             cudaStream_t);                                                                      \
-  template void local_force<T>(const T*, const double*, int, int, double, double*, double*, cudaStream_t, bool); \
+  template void local_force<T>(const T*, const double*, const int*, int, int, int, double, double*, double*,    \
+                               cudaStream_t, bool);                                                            \
   template void grad_packed<T>(const cplx<T>*, cplx<T>*, const DevTables<T>&, int, int, cudaStream_t);          \
   template void vloc_from_axes<T>(const double*, int, int, double, T*, double*, cudaStream_t);                  \
   template void state_dots<T>(const cplx<T>*, const cplx<T>*, int, int, double2*, cudaStream_t);                \

@@ -29,6 +29,14 @@ template <typename T> struct DevTables {
 // ---- full-grid (plain) path --------------------------------------------------------------------
 // In-place batched 1D FFTs along one axis (0: x, 1: y, 2: z) of nb grids [N][N][N].
 template <typename T> void fft_axis(cplx<T>* grid, int nb, int N, int axis, int sign, const cplx<T>* tw, cudaStream_t s);
+// The z passes at the ends of an H application: grid = inverse z transform of the packed states on the
+// sphere's points (the others zero), and hpsi = scale (forward z transform of grid) + |G|^2/2 psi on the
+// sphere (the grid is not written).  ginv [N^3]: packed index of a grid point or -1 (invert_index).
+template <typename T> void fft_z_from_sphere(const cplx<T>* psi, cplx<T>* grid, const int* ginv, const DevTables<T>& t,
+                                             int nb, cudaStream_t s);
+template <typename T> void fft_z_to_sphere(cplx<T>* grid, const cplx<T>* psi, cplx<T>* hpsi, const int* ginv,
+                                           const DevTables<T>& t, int nb, T scale, cudaStream_t s);
+void invert_index(const int* gidx, int nG, int* ginv, size_t N3, cudaStream_t s);
 // grid[b][gidx[g]] = psi[b][g] (grid must be zeroed before).
 template <typename T> void scatter_sphere(const cplx<T>* psi, cplx<T>* grid, const DevTables<T>& t, int nb, cudaStream_t s);
 // hpsi[b][g] = scale * grid[b][gidx[g]] + g2half[g] * psi[b][g] (no kinetic term if psi is null)
@@ -47,12 +55,14 @@ template <typename T> void grad_accumulate(const cplx<T>* dpsi, const cplx<T>* p
 // fnl[3 I + alpha] -= w sum_{b < nb} occ[b] sum_l Re(conj(q_bIl) p_bIl) (projections [nb][natoms][nproj])
 template <typename T> void nl_force(const cplx<T>* p, const cplx<T>* q, int natoms, int nproj, int nb, double w,
                                     const double* occ, double* fnl, int alpha, cudaStream_t s);
-// floc[3 I + a] = coef sum_j X_I[jx] Y_I[jy] Z_I[jz] g_a[j], g [3][N^3], xyz [natoms][3][N];
-// zmajor: g laid out [z][x][y].  Each atom's sum runs over LOCAL_FORCE_SPLIT slices of the
-// grid (partials [natoms][LOCAL_FORCE_SPLIT][3]), then the slices are added in order.
+// floc[3 I + a] = coef sum_j X_I[jx] Y_I[jy] Z_I[jz] g_a[j], g [3][N^3], xyz [natoms][3][N], over the
+// cnt^3 box of grid points from start [natoms][3] on (mod N) outside which the factors are negligible;
+// zmajor: g laid out [z][x][y].  Each atom's sum runs over LOCAL_FORCE_SPLIT slices of its box
+// (partials [natoms][LOCAL_FORCE_SPLIT][3]), then the slices are added in order.
 constexpr int LOCAL_FORCE_SPLIT = 8;
-template <typename T> void local_force(const T* g, const double* xyz, int N, int natoms, double coef, double* partials,
-                                       double* floc, cudaStream_t s, bool zmajor = false);
+template <typename T> void local_force(const T* g, const double* xyz, const int* start, int cnt, int N, int natoms,
+                                       double coef, double* partials, double* floc, cudaStream_t s,
+                                       bool zmajor = false);
 // out[b][g] = i G_alpha c_bg (packed, nb states)
 template <typename T> void grad_packed(const cplx<T>* psi, cplx<T>* out, const DevTables<T>& t, int alpha, int nb,
                                        cudaStream_t s);
