@@ -339,7 +339,7 @@ template <typename T> class Engine final : public EngineBase {
     nin_ = alloc<T>(N3);
     resid_dev_ = alloc<double>(1);
     dip_partials_ = alloc<double>(HXC_BLOCKS * 3);
-    trr_ = alloc<double2>(ns_);
+    trr_ = alloc<double2>((size_t)ns_ * TETER_SPLIT);
     dipoles_dev_ = alloc<double>(3 * MAX_STEPS_CHUNK);
     parts_ = alloc<double>(4);
     dots_ = alloc<double2>(ns_);

@@ -414,21 +414,20 @@ template <int N, int Ns> struct RadixOf {
 
 // Identity epilogue of the last stage.
 struct NoEpi {
-  __device__ __forceinline__ float2 operator()(float2 v, int, int) const { return v; }
+  template <typename C> __device__ __forceinline__ C operator()(C v, int, int) const { return v; }
 };
 
 // One stage over `lines` lines (<= LPC lines; LPC = lines per call).  LINE_FAST: job =
 // j * LPC + l (consecutive threads on consecutive lines), else job = l * M + j.  The last
 // stage (Ns * R == N) passes every output through epi(value, element index, line index
 // within the call) before storing it.
-template <int N, int Ns, int R, int THREADS, int LPC, bool LINE_FAST, int SIGN, class Epi>
-__device__ __forceinline__ void cstage(float2* s, int lines, int lstride, int kstride, const float2* tw,
-                                       const Epi& epi) {
+template <int N, int Ns, int R, int THREADS, int LPC, bool LINE_FAST, int SIGN, class Epi, typename C>
+__device__ __forceinline__ void cstage(C* s, int lines, int lstride, int kstride, const C* tw, const Epi& epi) {
   constexpr int M = N / R;
   constexpr int step = N / (Ns * R);
   constexpr int JOBS = LPC * M;
   constexpr int Q = (JOBS + THREADS - 1) / THREADS;
-  float2 v[Q][R];
+  C v[Q][R];
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     const int job = threadIdx.x + q * THREADS;
@@ -442,18 +441,18 @@ __device__ __forceinline__ void cstage(float2* s, int lines, int lstride, int ks
     }
     if (job < JOBS && l < lines) {
       const int k = j % Ns;
-      const float2* line = s + l * lstride;
+      const C* line = s + l * lstride;
 #pragma unroll
       for (int r = 0; r < R; ++r) v[q][r] = line[(j + r * M) * kstride];
       if (Ns > 1) {
 #pragma unroll
         for (int r = 1; r < R; ++r) {
-          float2 w = tw[k * r * step];
+          C w = tw[k * r * step];
           if (SIGN < 0) w.y = -w.y;
           v[q][r] = cmul(v[q][r], w);
         }
       }
-      SmallDft<R, float2>::run(v[q], SIGN);
+      SmallDft<R, C>::run(v[q], SIGN);
     }
   }
   __syncthreads();
@@ -470,7 +469,7 @@ __device__ __forceinline__ void cstage(float2* s, int lines, int lstride, int ks
     }
     if (job < JOBS && l < lines) {
       const int k = j % Ns;
-      float2* line = s + l * lstride;
+      C* line = s + l * lstride;
       const int base = (j / Ns) * Ns * R + k;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
@@ -483,8 +482,8 @@ __device__ __forceinline__ void cstage(float2* s, int lines, int lstride, int ks
 }
 
 template <int N, int Ns, int THREADS, int LPC, bool LINE_FAST, int SIGN, class Epi> struct CFft {
-  static __device__ __forceinline__ void run(float2* s, int lines, int lstride, int kstride, const float2* tw,
-                                             const Epi& epi) {
+  template <typename C>
+  static __device__ __forceinline__ void run(C* s, int lines, int lstride, int kstride, const C* tw, const Epi& epi) {
     constexpr int R = RadixOf<N, Ns>::R;
     cstage<N, Ns, R, THREADS, LPC, LINE_FAST, SIGN, Epi>(s, lines, lstride, kstride, tw, epi);
     CFft<N, Ns * R, THREADS, LPC, LINE_FAST, SIGN, Epi>::run(s, lines, lstride, kstride, tw, epi);
@@ -492,19 +491,19 @@ template <int N, int Ns, int THREADS, int LPC, bool LINE_FAST, int SIGN, class E
 };
 template <int N, int THREADS, int LPC, bool LINE_FAST, int SIGN, class Epi>
 struct CFft<N, N, THREADS, LPC, LINE_FAST, SIGN, Epi> {
-  static __device__ __forceinline__ void run(float2*, int, int, int, const float2*, const Epi&) {}
+  template <typename C> static __device__ __forceinline__ void run(C*, int, int, int, const C*, const Epi&) {}
 };
 
 // Shifts the line index of an epilogue by the first line of a call.
 template <class Epi> struct EpiAt {
   const Epi& e;
   int l0;
-  __device__ __forceinline__ float2 operator()(float2 v, int x, int l) const { return e(v, x, l0 + l); }
+  template <typename C> __device__ __forceinline__ C operator()(C v, int x, int l) const { return e(v, x, l0 + l); }
 };
 
 // All `lines` lines, LPC at a time; epi(value, element, line) on the last stage's outputs.
-template <int N, int THREADS, int LPC, bool LINE_FAST, int SIGN, class Epi = NoEpi>
-__device__ __forceinline__ void cfft_lines(float2* s, int lines, int lstride, int kstride, const float2* tw,
+template <int N, int THREADS, int LPC, bool LINE_FAST, int SIGN, class Epi = NoEpi, typename C = float2>
+__device__ __forceinline__ void cfft_lines(C* s, int lines, int lstride, int kstride, const C* tw,
                                            const Epi& epi = Epi()) {
   for (int l0 = 0; l0 < lines; l0 += LPC)
     CFft<N, 1, THREADS, LPC, LINE_FAST, SIGN, EpiAt<Epi>>::run(s + l0 * lstride, min(LPC, lines - l0), lstride,

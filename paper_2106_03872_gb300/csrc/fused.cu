@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "exact_sum.cuh"
 #include "fft_device.cuh"
 #include "fused.h"
 #include "tuner.h"
@@ -1264,7 +1265,8 @@ __global__ void __launch_bounds__(FCfg<N>::PT, FCfg<N>::PMIN)
 // of the chunk's states to partial[chunk][z][x][y], psi read back from the grid.  Both store the values
 // at the plane's covered points to val[b][point] for the projections, so d psi never goes to the grid.
 // Full-grid stores of psi and three derivatives, four passes over the spheres in them and three passes
-// summing the products took 7.05 ms a call on 128 states of 96^3; this form @FO@.
+// summing the products took 7.05 ms a call on 128 states of 96^3; this form takes 2.46 ms (a derivative
+// 0.46 ms, of which the density kernel's transforms are 0.42).
 template <int N, bool GRAD>
 __global__ void __launch_bounds__(TCfg<N>::PT, TCfg<N>::PMIN)
     k_plane_force_team(const float2* __restrict__ colbuf, int ncols, const int* __restrict__ col_xy, int xr,
@@ -1299,6 +1301,11 @@ __global__ void __launch_bounds__(TCfg<N>::PT, TCfg<N>::PMIN)
 #pragma unroll 1
   for (int b = b0; b < b1; ++b) {
     const float2* src = colbuf + ((size_t)b * N + z) * ncols;
+    // psi's plane towards L2 while this state is transformed
+    if (GRAD && threadIdx.x == 0)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(grid + ((size_t)b * N + z) * N * N),
+                   "r"(N * N * (int)sizeof(float2))
+                   : "memory");
     for (int c = threadIdx.x; c < ncols; c += PT) {
       const int xy = col_xy[c];
       const int jx = xy / N, jy = xy - jx * N;
@@ -1392,69 +1399,56 @@ __global__ void __launch_bounds__(256) k_add_partials(const float* __restrict__ 
   }
 }
 
-// proj[b][I][l] = scale sum over atom I's sphere points of beta_l val[b][slot], for PJB states per CTA.
-// slot and beta list the atom's points in plane order.  The products are exact (product and its rounding
-// error by fma) and summed with compensation: about FP64's precision without its pipe, which took 0.2 ms
-// per field of 128 states and 64 atoms.
-constexpr int PJB = 2;
-__device__ __forceinline__ void add_product(float& s, float& c, float a, float b) {
-  const float p = a * b, e = fmaf(a, b, -p);
-  const float t = s + p, bp = t - s;
-  c += ((s - (t - bp)) + (p - bp)) + e;
-  s = t;
-}
+// proj[b][I][l] = scale sum over atom I's sphere points of beta_l val[b][slot], one warp per atom and
+// state.  slot and beta list the atom's points in increasing covered point.  The products are exact
+// (product and its rounding error by fma) and summed with compensation, across the lanes too: about FP64's
+// precision without its pipe (FP64 sums took 0.2 ms per field of 128 states and 64 atoms, FP64 only for
+// the sums across lanes 0.27 ms).
+constexpr int PJW = 8;
 template <int NP>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(32 * PJW)
     k_project_points(const float2* __restrict__ val, int npts, const int* __restrict__ sph_off,
                      const int* __restrict__ slot, const float* __restrict__ beta, int natoms, int n, float scale,
                      float2* __restrict__ proj) {
   chain_begin();
-  __shared__ double red[8][PJB * NP * 2];
-  const int I = blockIdx.x, b0 = blockIdx.y * PJB, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float s[PJB][NP][2] = {}, c[PJB][NP][2] = {};
-  for (int q = sph_off[I] + threadIdx.x; q < sph_off[I + 1]; q += 256) {
-    const int pt = slot[q];
+  const int I = blockIdx.x, lane = threadIdx.x & 31, b = blockIdx.y * PJW + (threadIdx.x >> 5);
+  if (b >= n) return;
+  const float2* vb = val + (size_t)b * npts;
+  SumPair t[NP][2];
+#pragma unroll 4
+  for (int q = sph_off[I] + lane; q < sph_off[I + 1]; q += 32) {
+    const float2 v = vb[slot[q]];
     float w[NP];
     if constexpr (NP == 4) {
-      const float4 t = *reinterpret_cast<const float4*>(beta + (size_t)q * 4);
-      w[0] = t.x;
-      w[1] = t.y;
-      w[2] = t.z;
-      w[3] = t.w;
+      const float4 f = *reinterpret_cast<const float4*>(beta + (size_t)q * 4);
+      w[0] = f.x;
+      w[1] = f.y;
+      w[2] = f.z;
+      w[3] = f.w;
     } else {
       w[0] = beta[q];
     }
 #pragma unroll
-    for (int k = 0; k < PJB; ++k)
-      if (b0 + k < n) {
-        const float2 v = val[(size_t)(b0 + k) * npts + pt];
-#pragma unroll
-        for (int l = 0; l < NP; ++l) {
-          add_product(s[k][l][0], c[k][l][0], w[l], v.x);
-          add_product(s[k][l][1], c[k][l][1], w[l], v.y);
-        }
-      }
+    for (int l = 0; l < NP; ++l) {
+      t[l][0].add_product(w[l], v.x);
+      t[l][1].add_product(w[l], v.y);
+    }
   }
 #pragma unroll
-  for (int k = 0; k < PJB; ++k)
+  for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
     for (int l = 0; l < NP; ++l)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        double t = (double)s[k][l][h] + (double)c[k][l][h];
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-        if (lane == 0) red[warp][(k * NP + l) * 2 + h] = t;
+        const float x = __shfl_xor_sync(0xffffffffu, t[l][h].s, o), e = __shfl_xor_sync(0xffffffffu, t[l][h].c, o);
+        t[l][h].add(x, e);
       }
-  __syncthreads();
-  const int e = threadIdx.x;                                         // (k, l)
-  if (e < PJB * NP && b0 + e / NP < n) {
-    double x = 0.0, y = 0.0;
-    for (int w = 0; w < 8; ++w) {
-      x += red[w][2 * e];
-      y += red[w][2 * e + 1];
+  if (lane == 0)
+#pragma unroll
+    for (int l = 0; l < NP; ++l) {
+      const double x = t[l][0].value(), y = t[l][1].value();
+      proj[((size_t)b * natoms + I) * NP + l] = make_float2((float)(x * scale), (float)(y * scale));
     }
-    proj[((size_t)(b0 + e / NP) * natoms + I) * NP + e % NP] = make_float2((float)(x * scale), (float)(y * scale));
-  }
 }
 
 // Setup: projector grid functions -> sphere coefficients (FP64), then rounded to complex64.
@@ -1787,12 +1781,12 @@ class FusedImpl final : public FusedOps {
 
   // The projections of the covered-point values in nlval_ (n states).
   void project(int n, float pscale, float2* out, cudaStream_t s) {
-    const dim3 grid(g_.natoms, (n + PJB - 1) / PJB);
+    const dim3 grid(g_.natoms, (n + PJW - 1) / PJW);
     if (g_.nproj == 4)
-      launch_chain(points(n), k_project_points<4>, grid, dim3(256), 0, s, nlval_, npts_, t_.sph_off, sph_slot_, sph_bz_,
+      launch_chain(points(n), k_project_points<4>, grid, dim3(32 * PJW), 0, s, nlval_, npts_, t_.sph_off, sph_slot_, sph_bz_,
                    g_.natoms, n, pscale, out);
     else
-      launch_chain(points(n), k_project_points<1>, grid, dim3(256), 0, s, nlval_, npts_, t_.sph_off, sph_slot_, sph_bz_,
+      launch_chain(points(n), k_project_points<1>, grid, dim3(32 * PJW), 0, s, nlval_, npts_, t_.sph_off, sph_slot_, sph_bz_,
                    g_.natoms, n, pscale, out);
   }
 
@@ -2031,7 +2025,11 @@ class FusedImpl final : public FusedOps {
     std::vector<int>& ent_off = h_ent_off_;
     std::vector<int>& ent_proj = h_ent_proj_;
     std::vector<float>& ent_beta = h_ent_beta_;
-    std::vector<int> slot_of(g.sph_idx.size(), 0);                    // covered point of each sphere point
+    // each atom's sphere points in the order of the covered points (so that a warp reads runs of them):
+    // their covered points and beta values (forces)
+    std::vector<int> next(g.sph_off.begin(), g.sph_off.end());
+    h_sph_slot_.resize(g.sph_idx.size());
+    h_sph_bz_.resize(g.sph_idx.size() * g.nproj);
     pt_off.assign(N_ + 1, 0);
     pt_xy.clear();
     ent_off.assign(1, 0);
@@ -2058,21 +2056,18 @@ class FusedImpl final : public FusedOps {
         pt_xy.push_back(g.cov_idx[c] / N_);
         for (int e = g.cov_off[c]; e < g.cov_off[c + 1]; ++e) {
           const int p = g.cov_ent[e];
-          slot_of[p] = (int)pt_xy.size() - 1;
+          const size_t at = (size_t)next[g.sph_atom[p]]++;
+          h_sph_slot_[at] = (int)pt_xy.size() - 1;
           ent_proj.push_back(g.sph_atom[p] * g.nproj);
-          for (int l = 0; l < g.nproj; ++l) ent_beta.push_back((float)g.sph_beta[(size_t)p * g.nproj + l]);
+          for (int l = 0; l < g.nproj; ++l) {
+            const float b = (float)g.sph_beta[(size_t)p * g.nproj + l];
+            ent_beta.push_back(b);
+            h_sph_bz_[at * g.nproj + l] = b;
+          }
         }
         ent_off.push_back((int)ent_proj.size());
       }
       pt_off[z + 1] = (int)pt_xy.size();
-    }
-    // each atom's sphere points in plane order: their covered points and beta values (forces)
-    h_sph_slot_.resize(g.sph_zorder.size());
-    h_sph_bz_.resize(g.sph_zorder.size() * g.nproj);
-    for (size_t q = 0; q < g.sph_zorder.size(); ++q) {
-      const int p = g.sph_zorder[q];
-      h_sph_slot_[q] = slot_of[p];
-      for (int l = 0; l < g.nproj; ++l) h_sph_bz_[q * g.nproj + l] = (float)g.sph_beta[(size_t)p * g.nproj + l];
     }
   }
   void upload_plane_lists() {
@@ -2214,7 +2209,7 @@ class FusedImpl final : public FusedOps {
   int nl_cap_ = 0;                    // most covered points of any plane
   std::vector<int> h_sph_slot_;
   std::vector<float> h_sph_bz_;
-  const int* sph_slot_ = nullptr;     // [npts_sph] covered point of each atom's sphere points, plane order
+  const int* sph_slot_ = nullptr;     // [npts_sph] covered point of each atom's sphere points, increasing
   const float* sph_bz_ = nullptr;     // [npts_sph][nproj] their beta values
   bool lists_ready_ = false;
   float2* colbuf1_ = nullptr;

@@ -3,6 +3,7 @@
 // periodic Poisson + Slater exchange, and the FP64 reductions for norms and energies.
 #include <type_traits>
 
+#include "exact_sum.cuh"
 #include "fft_device.cuh"
 #include "kernels.h"
 
@@ -236,40 +237,77 @@ __global__ void __launch_bounds__(128)
 // image sums [natoms][3][N] of the separable Gaussian, start [natoms][3] the first of the `cnt` grid
 // indices (mod N) around the atom outside which every factor is below 1e-20.  A warp per grid row of the
 // atom's box: the row's sum with the inner axis' factors, then one product with the two others'.  FP64
-// throughout, so the FP64 pipe bounds it: over the whole grid with a product per point, the 64 atoms of a
-// 96^3 cell took 0.72 ms.
+// arithmetic (conversions too) would bound it on FP32 fields, so there the FP64 factors are split into two
+// FP32 parts, the products are exact (with their rounding errors by fma) and the sums compensated, which
+// keeps about 45 bits: over the whole grid in FP64, the 64 atoms of a 96^3 cell took 0.72 ms, over the
+// boxes 0.27 ms, so 0.067 ms.
 template <typename T>
 __global__ void __launch_bounds__(RED_THREADS)
     k_local_force(const T* __restrict__ g, const double* __restrict__ xyz, const int* __restrict__ start, int cnt, int N,
                   double coef, double* __restrict__ partials, int zmajor) {
   chain_begin();
-  const int I = blockIdx.x, sl = blockIdx.y, lane = threadIdx.x & 31;
+  constexpr bool SPLIT = sizeof(T) == 4;
+  __shared__ float2 f0[128];                                         // the inner factors along the box, split
+  const int I = blockIdx.x, sl = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const size_t N3 = (size_t)N * N * N;
   // axes of the memory order, slowest first: [z][x][y] or [x][y][z]
   const int ax2 = zmajor ? 2 : 0, ax1 = zmajor ? 0 : 1, ax0 = zmajor ? 1 : 2;
   const double *T2 = xyz + ((size_t)I * 3 + ax2) * N, *T1 = xyz + ((size_t)I * 3 + ax1) * N,
                *T0 = xyz + ((size_t)I * 3 + ax0) * N;
   const int s2 = start[3 * I + ax2], s1 = start[3 * I + ax1], s0 = start[3 * I + ax0];
-  double acc[3] = {0.0, 0.0, 0.0};
-  const int rows = cnt * cnt, r0 = rows * sl / LOCAL_FORCE_SPLIT, r1 = rows * (sl + 1) / LOCAL_FORCE_SPLIT;
-  for (int r = r0 + (threadIdx.x >> 5); r < r1; r += RED_THREADS / 32) {
-    int j2 = s2 + r / cnt, j1 = s1 + r % cnt;
-    if (j2 >= N) j2 -= N;
-    if (j1 >= N) j1 -= N;
-    const T* row = g + ((size_t)j2 * N + j1) * N;
-    double t[3] = {0.0, 0.0, 0.0};
-    for (int i = lane; i < cnt; i += 32) {
-      int j0 = s0 + i;
-      if (j0 >= N) j0 -= N;
-      const double f = T0[j0];
-      t[0] = fma(f, (double)row[j0], t[0]);
-      t[1] = fma(f, (double)row[N3 + j0], t[1]);
-      t[2] = fma(f, (double)row[2 * N3 + j0], t[2]);
+  auto wrap = [&](int j) { return j >= N ? j - N : j; };
+  if (SPLIT) {
+    for (int i = threadIdx.x; i < cnt; i += RED_THREADS) {
+      const double f = T0[wrap(s0 + i)];
+      const float h = (float)f;
+      f0[i] = make_float2(h, (float)(f - (double)h));
     }
-    const double v = T2[j2] * T1[j1];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) acc[a] = fma(v, t[a], acc[a]);
+    __syncthreads();
   }
+  double acc[3] = {0.0, 0.0, 0.0};
+  SumPair S[3];
+  const int rows = cnt * cnt, r0 = rows * sl / LOCAL_FORCE_SPLIT, r1 = rows * (sl + 1) / LOCAL_FORCE_SPLIT;
+  for (int rb = r0 + 32 * warp; rb < r1; rb += RED_THREADS) {
+    // 32 rows of a warp: lane k forms the product of row k's two outer factors
+    const int mr = min(rb + lane, r1 - 1), m2 = wrap(s2 + mr / cnt), m1 = wrap(s1 + mr % cnt);
+    const double v = T2[m2] * T1[m1];
+    const float vh = (float)v, vl = (float)(v - (double)vh);
+    const int at = m2 * N + m1, nr = min(32, r1 - rb);
+    for (int k = 0; k < nr; ++k) {
+      const T* row = g + (size_t)__shfl_sync(0xffffffffu, at, k) * N;
+      if constexpr (SPLIT) {
+        const float wh = __shfl_sync(0xffffffffu, vh, k), wl = __shfl_sync(0xffffffffu, vl, k);
+        SumPair t[3];
+        for (int i = lane; i < cnt; i += 32) {
+          const int j0 = wrap(s0 + i);
+          const float2 f = f0[i];
+#pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            const float x = row[a * N3 + j0], p = f.x * x;
+            t[a].add(p, fmaf(f.x, x, -p) + f.y * x);
+          }
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const float p = wh * t[a].s;
+          S[a].add(p, fmaf(wh, t[a].s, -p) + (wl * t[a].s + wh * t[a].c));
+        }
+      } else {
+        const double w = __shfl_sync(0xffffffffu, v, k);
+        double t[3] = {0.0, 0.0, 0.0};
+        for (int i = lane; i < cnt; i += 32) {
+          const int j0 = wrap(s0 + i);
+          const double f = T0[j0];
+#pragma unroll
+          for (int a = 0; a < 3; ++a) t[a] = fma(f, (double)row[a * N3 + j0], t[a]);
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) acc[a] = fma(w, t[a], acc[a]);
+      }
+    }
+  }
+  if (SPLIT)
+    for (int a = 0; a < 3; ++a) acc[a] = S[a].value();
   block_sum<3>(acc);
   if (threadIdx.x == 0)
     for (int a = 0; a < 3; ++a) partials[((size_t)I * LOCAL_FORCE_SPLIT + sl) * 3 + a] = coef * acc[a];
@@ -512,37 +550,81 @@ __global__ void k_pulay_mix(T* __restrict__ nin, size_t N3, PulayMix<T> p) {
   }
 }
 
-// Teter-preconditioned SD, step 1 (one block per state): tr[b] = sum_g g2half |R|^2 and
-// r2[b] = sum_g |R|^2 of the residual R = hpsi - eig[b] psi.
+// Teter-preconditioned SD, step 1: the sums over g of g2half |R|^2 and |R|^2 of the residual
+// R = hpsi - eig psi, TETER_SPLIT blocks per state (part [n][TETER_SPLIT]).  On complex64 states eig is
+// split into two FP32 parts and R, its square and the sums carry their rounding errors (about 45 bits):
+// in FP64, one block per state, the pass took 0.17 ms on 96 states of 64^3, where the state arrays' bytes
+// take 8 us.
 template <typename T>
-__global__ void k_residual_kinetic(const cplx<T>* __restrict__ psi, const cplx<T>* __restrict__ hpsi,
-                                   const T* __restrict__ g2h, const double* __restrict__ eig, int nG,
-                                   double2* __restrict__ out) {
-  const int b = blockIdx.x;
+__global__ void __launch_bounds__(RED_THREADS)
+    k_residual_kinetic(const cplx<T>* __restrict__ psi, const cplx<T>* __restrict__ hpsi, const T* __restrict__ g2h,
+                       const double* __restrict__ eig, int nG, double2* __restrict__ part) {
+  const int b = blockIdx.y;
   const double e = eig[b];
+  const int g0 = (int)((long)nG * blockIdx.x / TETER_SPLIT), g1 = (int)((long)nG * (blockIdx.x + 1) / TETER_SPLIT);
   double acc[2] = {0.0, 0.0};
-  for (int g = threadIdx.x; g < nG; g += blockDim.x) {
-    const cplx<T> p = psi[(size_t)b * nG + g], h = hpsi[(size_t)b * nG + g];
-    const double rx = (double)h.x - e * (double)p.x, ry = (double)h.y - e * (double)p.y;
-    const double r2 = rx * rx + ry * ry;
-    acc[0] += (double)g2h[g] * r2;
-    acc[1] += r2;
+  if constexpr (std::is_same<T, float>::value) {
+    const float eh = (float)e, el = (float)(e - (double)eh);
+    SumPair tr, r2;
+    // r = h - e p as d + f, f of the order of d's rounding
+    auto residual = [&](float h, float p, float& d, float& f) {
+      const float m = eh * p, me = fmaf(eh, p, -m) + el * p;
+      d = h - m;
+      const float bp = d - h;
+      f = ((h - (d - bp)) - (m + bp)) - me;
+    };
+    for (int g = g0 + threadIdx.x; g < g1; g += RED_THREADS) {
+      const float2 p = psi[(size_t)b * nG + g], h = hpsi[(size_t)b * nG + g];
+      const float w = g2h[g];
+      float dx, fx, dy, fy;
+      residual(h.x, p.x, dx, fx);
+      residual(h.y, p.y, dy, fy);
+      SumPair q;                                                     // |r|^2
+      q.add_product(dx, dx);
+      q.add_product(dy, dy);
+      q.c += 2.f * (dx * fx + dy * fy);
+      r2.add(q.s, q.c);
+      const float k = w * q.s;
+      tr.add(k, fmaf(w, q.s, -k) + w * q.c);
+    }
+    acc[0] = tr.value();
+    acc[1] = r2.value();
+  } else {
+    for (int g = g0 + threadIdx.x; g < g1; g += RED_THREADS) {
+      const cplx<T> p = psi[(size_t)b * nG + g], h = hpsi[(size_t)b * nG + g];
+      const double rx = (double)h.x - e * (double)p.x, ry = (double)h.y - e * (double)p.y;
+      const double r2 = rx * rx + ry * ry;
+      acc[0] += (double)g2h[g] * r2;
+      acc[1] += r2;
+    }
   }
   block_sum<2>(acc);
-  if (threadIdx.x == 0) out[b] = make_double2(acc[0], acc[1]);
+  if (threadIdx.x == 0) part[(size_t)b * TETER_SPLIT + blockIdx.x] = make_double2(acc[0], acc[1]);
 }
 
 // Step 2: psi -= alpha_b K(g2half / T_b) R with T_b = max(tr / r2, tmin), alpha_b = 1 / (T_b + shift);
 // K(x) = (27 + 18x + 12x^2 + 8x^3) / (27 + 18x + 12x^2 + 8x^3 + 16x^4).  States with R = 0 stay.
 template <typename T>
 __global__ void k_teter_update(cplx<T>* __restrict__ psi, const cplx<T>* __restrict__ hpsi, const T* __restrict__ g2h,
-                               const double* __restrict__ eig, const double2* __restrict__ trr, double shift,
+                               const double* __restrict__ eig, const double2* __restrict__ part, double shift,
                                double tmin, int nG) {
   const int b = blockIdx.y;
-  const double2 q = trr[b];
-  if (!(q.y > 0.0)) return;                                          // uniform per block
-  const double t = fmax(q.x / q.y, tmin);
-  const T inv_t = (T)(1.0 / t), alpha = (T)(1.0 / (t + shift)), e = (T)eig[b];
+  __shared__ T sh[3];
+  if (threadIdx.x == 0) {
+    double2 q = make_double2(0.0, 0.0);
+    for (int i = 0; i < TETER_SPLIT; ++i) {
+      q.x += part[(size_t)b * TETER_SPLIT + i].x;
+      q.y += part[(size_t)b * TETER_SPLIT + i].y;
+    }
+    const bool live = q.y > 0.0;
+    const double t = live ? fmax(q.x / q.y, tmin) : 1.0;
+    sh[0] = (T)(1.0 / t);
+    sh[1] = live ? (T)(1.0 / (t + shift)) : T(-1);
+    sh[2] = (T)eig[b];
+  }
+  __syncthreads();
+  const T inv_t = sh[0], alpha = sh[1], e = sh[2];
+  if (alpha < T(0)) return;                                          // uniform per block
   for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < nG; g += gridDim.x * blockDim.x) {
     const T x = g2h[g] * inv_t;
     const T p = T(27) + x * (T(18) + x * (T(12) + x * T(8)));
@@ -897,9 +979,9 @@ void pulay_mix(T* nin, int N3, const PulayMix<T>& p, cudaStream_t s) {
 template <typename T>
 void teter_update(cplx<T>* psi, const cplx<T>* hpsi, const T* g2half, const double* eig, double2* trr, double shift,
                   double tmin, int nG, int n, cudaStream_t s) {
-  k_residual_kinetic<T><<<n, RED_THREADS, 0, s>>>(psi, hpsi, g2half, eig, nG, trr);
+  k_residual_kinetic<T><<<dim3(TETER_SPLIT, n), RED_THREADS, 0, s>>>(psi, hpsi, g2half, eig, nG, trr);
   KS_CHECK_LAUNCH();
-  k_teter_update<T><<<dim3(blocks_for((size_t)nG, 256, 64), n), 256, 0, s>>>(psi, hpsi, g2half, eig, trr, shift,
+  k_teter_update<T><<<dim3(blocks_for((size_t)nG, 1024, 64), n), 256, 0, s>>>(psi, hpsi, g2half, eig, trr, shift,
                                                                             tmin, nG);
   KS_CHECK_LAUNCH();
 }

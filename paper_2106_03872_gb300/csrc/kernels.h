@@ -121,7 +121,8 @@ template <typename T> void pulay_store(const T* nout, const T* nin, T* hn, T* hr
 template <typename T> void pulay_mix(T* nin, int N3, const PulayMix<T>& p, cudaStream_t s);
 // Teter-preconditioned SD update of n states [n][nG]: R = hpsi - eig psi, T_b = kinetic energy
 // of R_b (sum g2half |R|^2 / sum |R|^2) floored at tmin, psi_b -= K(g2half / T_b) R_b / (T_b + shift).
-// trr (device, n double2) receives (sum g2half |R|^2, sum |R|^2) per state.
+// trr (device, n TETER_SPLIT double2) receives partial (sum g2half |R|^2, sum |R|^2) of each state.
+constexpr int TETER_SPLIT = 8;
 template <typename T> void teter_update(cplx<T>* psi, const cplx<T>* hpsi, const T* g2half, const double* eig,
                                         double2* trr, double shift, double tmin, int nG, int n, cudaStream_t s);
 constexpr int HXC_BLOCKS = 296;
