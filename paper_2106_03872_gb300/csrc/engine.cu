@@ -428,6 +428,15 @@ template <typename T> class Engine final : public EngineBase {
     hpsi_valid_ = false;
   }
 
+  // grid_ = Omega^{1/2} psi(r) of nb packed states (plain path)
+  void to_real(const C* packed, int nb, cudaStream_t s) {
+    if constexpr (sizeof(T) == 8) {
+      if (plane64_inverse(packed, grid_, ginv_, t_, nb, s)) return;
+    }
+    fft_z_from_sphere<T>(packed, grid_, ginv_, t_, nb, s);
+    for (int ax = 1; ax >= 0; --ax) fft_axis<T>(grid_, nb, g_.N, ax, +1, t_.tw, s);
+  }
+
   // ------------------------------------------------------------------------------------------
   // H psi (Eq. 2): G -> r, V psi + V_NL psi on the grid, r -> G, keep S, + |G|^2/2 c.
   // ------------------------------------------------------------------------------------------
@@ -451,8 +460,7 @@ template <typename T> class Engine final : public EngineBase {
       const C* in = psi + (size_t)b0 * g_.nG;
       {
         ProfScope f(prof, "fft_lines", s);
-        fft_z_from_sphere<T>(in, grid_, ginv_, t_, nb, s);
-        for (int ax = 1; ax >= 0; --ax) fft_axis<T>(grid_, nb, N, ax, +1, t_.tw, s);
+        to_real(in, nb, s);
       }
       // grid holds psi' = Omega^{1/2} psi.  p = dV sum beta psi = dV Omega^{-1/2} sum beta psi'.
       nl_project<T>(grid_, t_, proj_, nb, T(g_.dV) * rs, s);
@@ -461,8 +469,13 @@ template <typename T> class Engine final : public EngineBase {
       nl_add<T>(grid_, t_, proj_, nb, T(g_.D * std::sqrt(g_.omega)), s);
       {
         ProfScope f(prof, "fft_lines", s);
-        for (int ax = 0; ax < 2; ++ax) fft_axis<T>(grid_, nb, N, ax, -1, t_.tw, s);
-        fft_z_to_sphere<T>(grid_, in, hpsi + (size_t)b0 * g_.nG, ginv_, t_, nb, T(1.0 / double(N3)), s);
+        C* out = hpsi + (size_t)b0 * g_.nG;
+        bool done = false;
+        if constexpr (sizeof(T) == 8) done = plane64_forward(grid_, in, out, ginv_, t_, nb, 1.0 / double(N3), s);
+        if (!done) {
+          for (int ax = 0; ax < 2; ++ax) fft_axis<T>(grid_, nb, N, ax, -1, t_.tw, s);
+          fft_z_to_sphere<T>(grid_, in, out, ginv_, t_, nb, T(1.0 / double(N3)), s);
+        }
       }
     }
   }
@@ -497,8 +510,7 @@ template <typename T> class Engine final : public EngineBase {
     const T scale = T(1.0 / g_.omega);
     for (int b0 = 0; b0 < n; b0 += batch_) {
       const int nb = std::min(batch_, n - b0);
-      fft_z_from_sphere<T>(psi + (size_t)b0 * g_.nG, grid_, ginv_, t_, nb, s);
-      for (int ax = 1; ax >= 0; --ax) fft_axis<T>(grid_, nb, N, ax, +1, t_.tw, s);
+      to_real(psi + (size_t)b0 * g_.nG, nb, s);
       density_accumulate<T>(grid_, occ_ + b0, nout, (int)N3, nb, scale, b0 == 0, s);
     }
   }

@@ -36,6 +36,13 @@ template <typename T> void fft_z_from_sphere(const cplx<T>* psi, cplx<T>* grid, 
                                              int nb, cudaStream_t s);
 template <typename T> void fft_z_to_sphere(cplx<T>* grid, const cplx<T>* psi, cplx<T>* hpsi, const int* ginv,
                                            const DevTables<T>& t, int nb, T scale, cudaStream_t s);
+// The same transforms in whole (y, z) planes on the FP64 path: grid = psi(r) Omega^{1/2} of nb packed
+// states, and hpsi = scale (forward transform of grid, destroyed) + |G|^2/2 psi.  False (nothing done) for
+// the grids without compiled planes.
+bool plane64_inverse(const double2* psi, double2* grid, const int* ginv, const DevTables<double>& t, int nb,
+                     cudaStream_t s);
+bool plane64_forward(double2* grid, const double2* psi, double2* hpsi, const int* ginv, const DevTables<double>& t,
+                     int nb, double scale, cudaStream_t s);
 void invert_index(const int* gidx, int nG, int* ginv, size_t N3, cudaStream_t s);
 // grid[b][gidx[g]] = psi[b][g] (grid must be zeroed before).
 template <typename T> void scatter_sphere(const cplx<T>* psi, cplx<T>* grid, const DevTables<T>& t, int nb, cudaStream_t s);

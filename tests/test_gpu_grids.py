@@ -47,3 +47,23 @@ def test_fused_grid(ks, meas, N, L, natoms, ns):
     meas("N=%d ETRS state" % N, rel(g.get_states(), q2), 5e-5)
     meas("N=%d ETRS norm and energy" % N, max(abs(norms[0] / n_ref - 1), abs(energies[0] / e_ref - 1)), 1e-4)
     g.close()
+
+
+@pytest.mark.parametrize("N,L,natoms,ns", [(24, 10.0, 3, 1), (36, 12.0, 3, 9), (54, 20.0, 5, 3), (72, 28.0, 4, 2),
+                                           (96, 30.0, 4, 2)])
+def test_fp64_planes(ks, meas, N, L, natoms, ns):
+    """FP64 H psi and density through whole (y, z) planes: 1e-12, as on every FP64 path."""
+    cell = inputs.small_cell(L, N, natoms, ns, 800 + N, depth=-3.0)
+    ref = ko.Cell(cell)
+    c = inputs.random_coeffs(800 + N, ns, ref.nG)
+    g = ks.Grid(cell, prec="fp64")
+    psi = torch.from_numpy(c).to("cuda")
+    h = torch.full_like(psi, float("nan"))
+    g.apply_h(psi.data_ptr(), h.data_ptr(), ns)
+    torch.cuda.synchronize()
+    meas("N=%d FP64 H psi" % N, rel(h.cpu().numpy(), ko.apply_h(ref, c)), 1e-12)
+    g.set_states(c)
+    n = torch.empty((N, N, N), dtype=torch.float64, device="cuda")
+    g.density(n.data_ptr())
+    meas("N=%d FP64 density" % N, rel(n.cpu().numpy(), ko.density(ref, c)), 1e-12)
+    g.close()
