@@ -14,7 +14,72 @@
 
 namespace ks {
 
+void StreamSet::create() {
+  int lo = 0, hi = 0;
+  KS_CUDA(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+  KS_CUDA(cudaStreamCreateWithPriority(&side, cudaStreamNonBlocking, hi));
+  for (cudaEvent_t& e : ev) KS_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+}
+
+void StreamSet::destroy() {
+  if (main) cudaStreamDestroy(main);
+  if (side) cudaStreamDestroy(side);
+  for (cudaEvent_t e : ev)
+    if (e) cudaEventDestroy(e);
+  *this = StreamSet{};
+}
+
+void StreamHolder::acquire(DevicePool* pool) {
+  pool_ = pool;
+  held_ = true;
+  if (pool_)
+    set_ = pool_->take_streams();
+  else
+    set_.create();
+}
+
+StreamHolder::~StreamHolder() {
+  if (!held_) return;
+  if (set_.main) cudaStreamSynchronize(set_.main);
+  if (set_.side) cudaStreamSynchronize(set_.side);
+  if (pool_)
+    pool_->give_streams(set_);
+  else
+    set_.destroy();
+}
+
+StreamSet DevicePool::take_streams() {
+  {
+    std::lock_guard<std::mutex> lk(mu_);
+    if (!idle_.empty()) {
+      StreamSet set = idle_.back();
+      idle_.pop_back();
+      return set;
+    }
+  }
+  StreamSet set;
+  try {
+    set.create();
+  } catch (...) {
+    set.destroy();
+    throw;
+  }
+  return set;
+}
+
+void DevicePool::give_streams(StreamSet set) {
+  {
+    std::lock_guard<std::mutex> lk(mu_);
+    if ((int)idle_.size() < StreamSet::KEEP) {
+      idle_.push_back(set);
+      return;
+    }
+  }
+  set.destroy();
+}
+
 DevicePool::~DevicePool() {
+  for (auto& set : idle_) set.destroy();
   for (auto& sl : slabs_) cudaFree(sl.base);
 }
 
@@ -244,10 +309,13 @@ template <typename T> class Engine final : public EngineBase {
     // side stream (highest priority, non-blocking): the CholQR factor that overlaps H psi, and
     // the setup work here and at atom moves (table uploads, V_loc, the projector block), which
     // so neither waits behind other engines' kernels nor serialises on the legacy stream
-    int lo = 0, hi = 0;
-    KS_CUDA(cudaDeviceGetStreamPriorityRange(&lo, &hi));
-    KS_CUDA(cudaStreamCreateWithPriority(&aux_, cudaStreamNonBlocking, hi));
+    streams_.acquire(pool);
+    aux_ = streams_->side;
     setup_ = aux_;
+    ev_gram_ = streams_->ev[0];
+    ev_hraw_ = streams_->ev[1];
+    ev_chol_ = streams_->ev[2];
+    ev_ritz_ = streams_->ev[3];
     const int N = g_.N, nG = g_.nG;
     const size_t N3 = (size_t)N * N * N;
     const size_t sn = (size_t)ns_ * nG;
@@ -345,23 +413,14 @@ template <typename T> class Engine final : public EngineBase {
     dots_ = alloc<double2>(ns_);
     norms_dev_ = alloc<double>(MAX_STEPS_CHUNK);
     energies_dev_ = alloc<double>(MAX_STEPS_CHUNK);
-    KS_CUDA(cudaEventCreateWithFlags(&ev_gram_, cudaEventDisableTiming));
-    KS_CUDA(cudaEventCreateWithFlags(&ev_hraw_, cudaEventDisableTiming));
-    KS_CUDA(cudaEventCreateWithFlags(&ev_chol_, cudaEventDisableTiming));
-    KS_CUDA(cudaEventCreateWithFlags(&ev_ritz_, cudaEventDisableTiming));
     update_vloc(setup_);                                             // ends with a synchronisation
   }
 
-  ~Engine() override {
-    if (aux_) {
-      cudaStreamSynchronize(aux_);
-      cudaStreamDestroy(aux_);
-    }
-    if (ev_gram_) cudaEventDestroy(ev_gram_);
-    if (ev_hraw_) cudaEventDestroy(ev_hraw_);
-    if (ev_chol_) cudaEventDestroy(ev_chol_);
-    if (ev_ritz_) cudaEventDestroy(ev_ritz_);
+  cudaStream_t main_stream() override {
+    if (!streams_->main) KS_CUDA(cudaStreamCreateWithFlags(&streams_->main, cudaStreamNonBlocking));
+    return streams_->main;
   }
+  cudaEvent_t order_event() override { return streams_->ev[4]; }
 
   const HostGeometry& geo() const override { return g_; }
   int nstates() const override { return ns_; }
@@ -1548,6 +1607,7 @@ template <typename T> class Engine final : public EngineBase {
   ks_precision prec_;
   int ns_;
   DeviceArena arena_;
+  StreamHolder streams_;             // after the arena: waits for its streams before the memory goes back
   DevTables<T> t_;
   std::unique_ptr<FusedOps> fused_;
   T* vloc_ = nullptr;

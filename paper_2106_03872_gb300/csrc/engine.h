@@ -10,6 +10,20 @@
 
 namespace ks {
 
+// The streams and events of one request's engine.  Creating and destroying them takes locks of the CUDA
+// context that a thread gets only when the others' launches and waits let it: with eight workers stepping,
+// one creation or destruction waited 30 to 125 ms, most of a request's start and retirement.  A server
+// therefore keeps them between requests (DevicePool), at most StreamSet::KEEP idle ones.
+struct StreamSet {
+  static constexpr int EVENTS = 5;
+  static constexpr int KEEP = 64;
+  cudaStream_t main = nullptr;      // a request's work (created on first use)
+  cudaStream_t side = nullptr;      // the engine's side stream, highest priority
+  cudaEvent_t ev[EVENTS] = {};
+  void create();                    // side stream and events
+  void destroy();
+};
+
 // Device memory shared by the engines of a server: slabs obtained with cudaMalloc as the pool
 // grows and kept until the pool is destroyed; blocks of 256-byte granularity handed out first
 // fit from per-slab free lists and returned without cudaFree.  cudaFree synchronises the whole
@@ -22,6 +36,9 @@ class DevicePool {
   ~DevicePool();
   void* alloc(size_t bytes);
   void free(void* p);
+  // A stream set (idle or new), and its return once its streams are idle.
+  StreamSet take_streams();
+  void give_streams(StreamSet set);
   size_t reserved() const;   // bytes obtained from the device
   size_t in_use() const;     // bytes handed out
   long grows() const;        // slabs obtained (cudaMalloc calls)
@@ -41,6 +58,22 @@ class DevicePool {
   size_t reserved_ = 0, in_use_ = 0;
   long grows_ = 0;
   double grow_s_ = 0;
+  std::vector<StreamSet> idle_;
+};
+
+// Owns an engine's stream set: from the pool and back to it, or created and destroyed.  Waits for the side
+// stream before it lets go.
+class StreamHolder {
+ public:
+  ~StreamHolder();
+  void acquire(DevicePool* pool);
+  StreamSet& operator*() { return set_; }
+  StreamSet* operator->() { return &set_; }
+
+ private:
+  DevicePool* pool_ = nullptr;
+  StreamSet set_;
+  bool held_ = false;
 };
 
 // Device allocation owned by an engine; every allocation is counted for admission.  With a pool,
@@ -153,6 +186,9 @@ class EngineBase {
                          double* energy_out, cudaStream_t s) = 0;
   virtual void randomize_states(uint64_t seed, cudaStream_t s) = 0;
   virtual void set_option(int option, int value) = 0;
+  // the engine's own stream for a server's request (non-blocking), and an event to order others after it
+  virtual cudaStream_t main_stream() = 0;
+  virtual cudaEvent_t order_event() = 0;
 };
 
 // pool (may be null): the engine's device memory comes from it.

@@ -126,12 +126,8 @@ void finish(ks_server_s* s, Request* r, ks_status st, const std::string& err) {
       st = e.st;
     }
   }
-  if (r->stream) cudaStreamSynchronize(r->stream);   // the engine's blocks go back to the pool idle
-  r->eng.reset();
-  if (r->stream) {
-    cudaStreamDestroy(r->stream);
-    r->stream = nullptr;
-  }
+  r->eng.reset();            // waits for its streams: its blocks and streams go back to the pool idle
+  r->stream = nullptr;
   std::lock_guard<std::mutex> lk(s->mu);
   r->finished = true;
   r->status = st;
@@ -145,8 +141,8 @@ void finish(ks_server_s* s, Request* r, ks_status st, const std::string& err) {
 // Create the engine and initial states of an admitted request (worker thread, no lock).
 void start(ks_server_s* s, Request* r) {
   const auto t0 = Clock::now();
-  KS_CUDA(cudaStreamCreateWithFlags(&r->stream, cudaStreamNonBlocking));
   r->eng = make_engine(r->desc, s->pool.get());
+  r->stream = r->eng->main_stream();
   const auto t1 = Clock::now();
   if (!r->c0.empty()) {
     r->eng->set_states(r->c0.data(), r->stream);
@@ -171,11 +167,9 @@ void td_group_quantum(const std::vector<Request*>& g) {
   for (Request* r : g) es.push_back(r->eng.get());
   cudaStream_t s0 = g[0]->stream;
   for (size_t i = 1; i < g.size(); ++i) {
-    cudaEvent_t ev;
-    KS_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    const cudaEvent_t ev = g[i]->eng->order_event();
     KS_CUDA(cudaEventRecord(ev, g[i]->stream));
     KS_CUDA(cudaStreamWaitEvent(s0, ev, 0));
-    KS_CUDA(cudaEventDestroy(ev));
   }
   std::vector<double> nrm(g.size()), e(g.size());
   td_step_engines(es, g[0]->dt, 1, nrm.data(), e.data(), s0);      // synchronous on s0
