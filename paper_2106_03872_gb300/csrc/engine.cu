@@ -410,7 +410,7 @@ template <typename T> class Engine final : public EngineBase {
     trr_ = alloc<double2>((size_t)ns_ * TETER_SPLIT);
     dipoles_dev_ = alloc<double>(3 * MAX_STEPS_CHUNK);
     parts_ = alloc<double>(4);
-    dots_ = alloc<double2>(ns_);
+    dots_ = alloc<double>((size_t)ns_ * DOT_SPLIT);
     norms_dev_ = alloc<double>(MAX_STEPS_CHUNK);
     energies_dev_ = alloc<double>(MAX_STEPS_CHUNK);
     update_vloc(setup_);                                             // ends with a synchronisation
@@ -1667,7 +1667,7 @@ template <typename T> class Engine final : public EngineBase {
   double* pulay_out_ = nullptr;
   double* dipoles_dev_ = nullptr;   // [MAX_STEPS_CHUNK][3] dipoles of a chunk of real-time steps
   double* parts_ = nullptr;
-  double2* dots_ = nullptr;
+  double* dots_ = nullptr;
   double* norms_dev_ = nullptr;
   double* energies_dev_ = nullptr;
 };

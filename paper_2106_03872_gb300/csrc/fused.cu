@@ -430,8 +430,10 @@ template <> struct TPlan<128> { static constexpr bool ok = true; static constexp
 // for every member of a packed H application too, the packed kernel spilling 68 bytes and taking
 // 0.683 against 0.614 ms per gs96-sized block; at N = 128 the packed kernel (20 bytes of spills)
 // runs for single-cell H applications too, the single-cell one spilling 112 bytes and taking
-// 6.75 against 6.44 ms per td128 block.
+// 6.75 against 6.44 ms per td128 block.  At N = 32 a packed application runs each member's CTA-wide plane
+// kernel (k_plane), which needs no projector values: 13.4 + 5.6 us with the team kernel at 24 states.
 template <int N> struct PlaneForm {
+  static constexpr bool cta_per_member = N == 32;
   static constexpr bool single_per_member = N == 96;
   static constexpr bool packed_for_single = N == 128;
 };
@@ -1611,22 +1613,26 @@ class FusedImpl final : public FusedOps {
 
   // The per-cell part of an H application: the projections p_Il = sum_G conj(b_Il(G)) c_G of the
   // block (tensor cores), scaled for the plane kernel, and the projector values they give.
-  void pre_h(const float2* psi, int n, cudaStream_t s) {
+  // `values`: the plane kernel that follows reads them (the team kernel; the CTA-wide one sums the
+  // projectors itself).
+  void pre_h(const float2* psi, int n, bool values, cudaStream_t s) {
     if (nprojtot_ > 0) {
       {
         ProfScope ps(prof_, "proj_gemm", s);
         tc_overlap(B_, g_.nG, psi, g_.nG, nprojtot_, n, g_.nG, part_, part_elems_, nullptr, err_, s, nullptr, Bimg_, pf_,
                    (float)(g_.D * std::sqrt(g_.omega)));
       }
-      if (npts_ > 0 && nlval_) {
-        ProfScope ps(prof_, "nl_values", s);
-        const dim3 grid((npts_ + 255) / 256, (n + NLB - 1) / NLB);
-        if (g_.nproj == 4)
-          launch_chain(points(n), k_nl_values<true>, grid, dim3(256), 0, s, pf_, nprojtot_, n, nl_, npts_, nlval_);
-        else
-          launch_chain(points(n), k_nl_values<false>, grid, dim3(256), 0, s, pf_, nprojtot_, n, nl_, npts_, nlval_);
-      }
+      if (values) nl_values(n, s);
     }
+  }
+  void nl_values(int n, cudaStream_t s) {
+    if (npts_ == 0 || !nlval_) return;
+    ProfScope ps(prof_, "nl_values", s);
+    const dim3 grid((npts_ + 255) / 256, (n + NLB - 1) / NLB);
+    if (g_.nproj == 4)
+      launch_chain(points(n), k_nl_values<true>, grid, dim3(256), 0, s, pf_, nprojtot_, n, nl_, npts_, nlval_);
+    else
+      launch_chain(points(n), k_nl_values<false>, grid, dim3(256), 0, s, pf_, nprojtot_, n, nl_, npts_, nlval_);
   }
 
   static bool same_geometry(const FusedImpl* a, const FusedImpl* b) {
@@ -1643,9 +1649,17 @@ class FusedImpl final : public FusedOps {
       FusedImpl* f = static_cast<FusedImpl*>(it.ops);
       if (!same_geometry(f0, f)) fail(KS_ERR_ARG, "packed H application: the members' grids differ");
       if (it.n < 1 || it.n > f->ns_) fail(KS_ERR_ARG, "packed H application: member with %d states", it.n);
-      f->pre_h(it.psi, it.n, s);
+      f->pre_h(it.psi, it.n, group_values(f->N_), s);
     }
     f0->dispatch([&](auto tag) { group_launch<decltype(tag)::value>(items, s); });
+  }
+
+  // whether the plane kernel of packed H applications reads the projector values
+  static bool group_values(int N) {
+    switch (N) {
+      case 48: case 54: case 64: case 72: case 96: case 108: case 128: return true;
+      default: return false;
+    }
   }
 
   template <int N> static void group_launch(const std::vector<FusedGroupItem>& items, cudaStream_t s) {
@@ -1699,7 +1713,12 @@ class FusedImpl final : public FusedOps {
         }
         {
           ProfScope ps(f0->prof_, "plane", s);
-          if constexpr (PlaneForm<N>::single_per_member) {
+          if constexpr (PlaneForm<N>::cta_per_member) {
+            for (size_t k = a; k < std::min(items.size(), a + GMAX); ++k) {
+              FusedImpl* f = static_cast<FusedImpl*>(items[k].ops);
+              f->template launch_plane<N>(items[k].n, f->colbuf1_, f->pf_, s, 1);
+            }
+          } else if constexpr (PlaneForm<N>::single_per_member) {
             for (size_t k = a; k < std::min(items.size(), a + GMAX); ++k) {
               FusedImpl* f = static_cast<FusedImpl*>(items[k].ops);
               f->template launch_plane_team_single<N>(items[k].n, s);
@@ -1719,7 +1738,8 @@ class FusedImpl final : public FusedOps {
   }
 
   void apply_h(const float2* psi, float2* hpsi, int n, cudaStream_t s, const TaylorEpi* te) override {
-    pre_h(psi, n, s);
+    const bool decided = !team_density() || tune_peek(tune_key("plane", n)) == 1;
+    pre_h(psi, n, !decided, s);
     zinv(psi, n, s);
     {
       ProfScope ps(prof_, "plane", s);
@@ -1879,8 +1899,10 @@ class FusedImpl final : public FusedOps {
     if constexpr (TPlan<N>::ok) {
       if (team_smem<N>(team_cap()) > SMEM_MAX) return 1;
       static const char* names[2] = {"team", "cta"};
-      return tune_choice(tune_key("plane", n), 2, [&](int c) { launch_plane<N>(n, colbuf1_, pf_, s, c); }, s,
-                         names);
+      return tune_choice(tune_key("plane", n), 2, [&](int c) {
+        if (c == 0 && nprojtot_ > 0) nl_values(n, s);                 // part of the team kernel's cost
+        launch_plane<N>(n, colbuf1_, pf_, s, c);
+      }, s, names);
     }
     return 1;
   }

@@ -637,50 +637,51 @@ __global__ void k_teter_update(cplx<T>* __restrict__ psi, const cplx<T>* __restr
   }
 }
 
+// Re <a_b|b_b> of each state b over DOT_SPLIT slices, one block each.  complex64 states: FP32 products
+// summed in FP32 over runs of 8 of a thread's elements, the runs summed in FP64 (FP64 arithmetic runs at
+// 1/64 of the FP32 rate: per element it took 3 ms per 512-state td128 block; each run carries at most 16
+// FP32 roundings).  A run's loads are issued together: with one block a state, a load at a time, 24 states
+// of 32^3 took 15 us and 96 of 48^3 40 us.
 template <typename T>
-__global__ void k_state_dots(const cplx<T>* __restrict__ a, const cplx<T>* __restrict__ bb, int nG,
-                             double2* __restrict__ dots) {
+__global__ void __launch_bounds__(RED_THREADS)
+    k_state_dots(const cplx<T>* __restrict__ a, const cplx<T>* __restrict__ bb, int nG, double* __restrict__ dots) {
   chain_begin();
-  const int b = blockIdx.x;
-  double acc[2] = {0.0, 0.0};
+  const int b = blockIdx.y;
+  const int g0 = (int)((long)nG * blockIdx.x / DOT_SPLIT), g1 = (int)((long)nG * (blockIdx.x + 1) / DOT_SPLIT);
+  const cplx<T>*pa = a + (size_t)b * nG, *pb = bb + (size_t)b * nG;
+  double acc[1] = {0.0};
   if constexpr (std::is_same<T, float>::value) {
-    // complex64 states: FP32 products summed in FP32 over runs of 8 of a thread's elements, the
-    // runs summed in FP64 (FP64 arithmetic runs at 1/64 of the FP32 rate: per element it took
-    // 3 ms per 512-state td128 block; each run carries at most 16 FP32 roundings)
-    float p0 = 0.f, p1 = 0.f;
-    int k = 0;
-    for (int g = threadIdx.x; g < nG; g += blockDim.x) {
-      const cplx<T> x = a[(size_t)b * nG + g], y = bb[(size_t)b * nG + g];
-      p0 = fmaf(x.x, y.x, p0);
-      p0 = fmaf(x.y, y.y, p0);
-      p1 = fmaf(x.x, y.y, p1);
-      p1 = fmaf(-x.y, y.x, p1);
-      if (++k == 8) {
-        acc[0] += (double)p0;
-        acc[1] += (double)p1;
-        p0 = p1 = 0.f;
-        k = 0;
+    for (int g = g0 + threadIdx.x; g < g1; g += 8 * RED_THREADS) {
+      float2 x[8], y[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int i = g + k * RED_THREADS;
+        x[k] = i < g1 ? pa[i] : make_float2(0.f, 0.f);
+        y[k] = i < g1 ? pb[i] : make_float2(0.f, 0.f);
       }
+      float p = 0.f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) p = fmaf(x[k].y, y[k].y, fmaf(x[k].x, y[k].x, p));
+      acc[0] += (double)p;
     }
-    acc[0] += (double)p0;
-    acc[1] += (double)p1;
   } else {
-    for (int g = threadIdx.x; g < nG; g += blockDim.x) {
-      const cplx<T> x = a[(size_t)b * nG + g], y = bb[(size_t)b * nG + g];
-      acc[0] += (double)x.x * y.x + (double)x.y * y.y;
-      acc[1] += (double)x.x * y.y - (double)x.y * y.x;
-    }
+    for (int g = g0 + threadIdx.x; g < g1; g += RED_THREADS)
+      acc[0] += (double)pa[g].x * pb[g].x + (double)pa[g].y * pb[g].y;
   }
-  block_sum<2>(acc);
-  if (threadIdx.x == 0) dots[b] = make_double2(acc[0], acc[1]);
+  block_sum<1>(acc);
+  if (threadIdx.x == 0) dots[(size_t)b * DOT_SPLIT + blockIdx.x] = acc[0];
 }
 
 __global__ void __launch_bounds__(RED_THREADS)
-    k_weighted_energy(const double2* __restrict__ dots, const double* __restrict__ occ, int nb,
+    k_weighted_energy(const double* __restrict__ dots, const double* __restrict__ occ, int nb,
                       const double* __restrict__ parts, double* __restrict__ out) {
   chain_begin();
   double e[1] = {0.0};
-  for (int b = threadIdx.x; b < nb; b += RED_THREADS) e[0] += occ[b] * dots[b].x;
+  for (int b = threadIdx.x; b < nb; b += RED_THREADS) {
+    double d = 0.0;
+    for (int i = 0; i < DOT_SPLIT; ++i) d += dots[(size_t)b * DOT_SPLIT + i];
+    e[0] += occ[b] * d;
+  }
   block_sum<1>(e);
   if (threadIdx.x == 0) out[0] = parts ? e[0] - parts[0] + parts[1] - parts[2] : e[0];
 }
@@ -1010,14 +1011,19 @@ __global__ void k_minmax_partials(const double* __restrict__ v, size_t n, double
 }
 
 __global__ void k_minmax_finish(const double* __restrict__ partials, int nblocks, double* __restrict__ out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
   double lo = INFINITY, hi = -INFINITY;
-  for (int b = 0; b < nblocks; ++b) {
+  for (int b = threadIdx.x; b < nblocks; b += 32) {
     lo = fmin(lo, partials[2 * b]);
     hi = fmax(hi, partials[2 * b + 1]);
   }
-  out[0] = lo;
-  out[1] = hi;
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  if (threadIdx.x == 0) {
+    out[0] = lo;
+    out[1] = hi;
+  }
 }
 
 void minmax(const double* v, size_t n, double* partials, int nblocks, double* out, cudaStream_t s) {
@@ -1032,11 +1038,11 @@ void sum_partials(const double* partials, int nblocks, double scale, double* out
 }
 
 template <typename T>
-void state_dots(const cplx<T>* a, const cplx<T>* b, int nG, int nb, double2* dots, cudaStream_t s) {
-  launch_chain(8 * (size_t)nb * nG, k_state_dots<T>, dim3(nb), dim3(RED_THREADS), 0, s, a, b, nG, dots);
+void state_dots(const cplx<T>* a, const cplx<T>* b, int nG, int nb, double* dots, cudaStream_t s) {
+  launch_chain(8 * (size_t)nb * nG, k_state_dots<T>, dim3(DOT_SPLIT, nb), dim3(RED_THREADS), 0, s, a, b, nG, dots);
 }
 
-void weighted_energy(const double2* dots, const double* occ, int nb, const double* parts, double* out, cudaStream_t s) {
+void weighted_energy(const double* dots, const double* occ, int nb, const double* parts, double* out, cudaStream_t s) {
   launch_chain(1, k_weighted_energy, dim3(1), dim3(RED_THREADS), 0, s, dots, occ, nb, parts, out);
 }
 
@@ -1102,7 +1108,7 @@ void real_to_double(const T* in, double* out, size_t n, cudaStream_t s) {
                                cudaStream_t, bool);                                                            \
   template void grad_packed<T>(const cplx<T>*, cplx<T>*, const DevTables<T>&, int, int, cudaStream_t);          \
   template void vloc_from_axes<T>(const double*, int, int, double, T*, double*, cudaStream_t);                  \
-  template void state_dots<T>(const cplx<T>*, const cplx<T>*, int, int, double2*, cudaStream_t);                \
+  template void state_dots<T>(const cplx<T>*, const cplx<T>*, int, int, double*, cudaStream_t);                 \
   template void axpy2<T>(cplx<T>*, double2, cplx<T>*, double2, const cplx<T>*, const cplx<T>*, size_t, cudaStream_t);           \
   template void random_states<T>(cplx<T>*, size_t, uint64_t, cudaStream_t);                                     \
   template void from_c128<T>(const double2*, cplx<T>*, size_t, cudaStream_t);                                   \

@@ -134,10 +134,11 @@ template <typename T> void teter_update(cplx<T>* psi, const cplx<T>* hpsi, const
                                         double2* trr, double shift, double tmin, int nG, int n, cudaStream_t s);
 constexpr int HXC_BLOCKS = 296;
 
-// dots[b] = sum_g conj(a[b][g]) b[b][g] (FP64 accumulation, fixed order)
-template <typename T> void state_dots(const cplx<T>* a, const cplx<T>* b, int nG, int nb, double2* dots, cudaStream_t s);
-// out[0] = sum_b occ[b] Re(dots[b]) - parts[0] + parts[1] - parts[2]   (parts may be NULL)
-void weighted_energy(const double2* dots, const double* occ, int nb, const double* parts, double* out, cudaStream_t s);
+// dots[b][i] = the i-th of DOT_SPLIT slices of sum_g Re(conj(a[b][g]) b[b][g]) (fixed order)
+constexpr int DOT_SPLIT = 8;
+template <typename T> void state_dots(const cplx<T>* a, const cplx<T>* b, int nG, int nb, double* dots, cudaStream_t s);
+// out[0] = sum_b occ[b] dots[b] - parts[0] + parts[1] - parts[2]   (parts may be NULL)
+void weighted_energy(const double* dots, const double* occ, int nb, const double* parts, double* out, cudaStream_t s);
 
 // acc1 += a1 * w; acc2 += a2 * w  (complex constants; acc2 may be NULL).  With base non-NULL
 // the accumulators start from it instead: acc1 = base + a1 w, acc2 = base + a2 w.

@@ -26,6 +26,12 @@ std::map<std::string, Decision>& decisions() {
 
 }  // namespace
 
+int tune_peek(const std::string& key) {
+  std::lock_guard<std::mutex> lk(g_mu);
+  auto it = decisions().find(key);
+  return it != decisions().end() ? it->second.choice : -1;
+}
+
 int tune_choice(const std::string& key, int ncand, const std::function<void(int)>& run, cudaStream_t s,
                 const char* const* names) {
   {

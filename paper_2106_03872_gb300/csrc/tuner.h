@@ -17,6 +17,8 @@ namespace ks {
 // Cached after the first call; thread-safe.
 int tune_choice(const std::string& key, int ncand, const std::function<void(int)>& run, cudaStream_t s,
                 const char* const* names);
+// The kept choice of a key, or -1 while it has not been timed.
+int tune_peek(const std::string& key);
 
 // The log of every decision so far: [{"key": ..., "ms": {name: ms, ...}, "choice": name}, ...].
 std::string tune_log_json();
