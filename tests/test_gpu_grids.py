@@ -1,4 +1,4 @@
-"""GPU: the fused path on the grids of 54, 72 and 108 points (6 x 9, 6 x 12 and 6 x 18 team plans, whose
+"""GPU: the fused path on the grids of 54, 72 and 108 points (6 x 9, 12 x 6 and 6 x 18 team plans, whose
 elements straddle the bitmap words) against the oracle."""
 import numpy as np
 import pytest
