@@ -431,11 +431,13 @@ template <> struct TPlan<128> { static constexpr bool ok = true; static constexp
 // for every member of a packed H application too, the packed kernel spilling 68 bytes and taking
 // 0.683 against 0.614 ms per gs96-sized block; at N = 128 the packed kernel (20 bytes of spills)
 // runs for single-cell H applications too, the single-cell one spilling 112 bytes and taking
-// 6.75 against 6.44 ms per td128 block.  At N = 32 a packed application runs each member's CTA-wide plane
-// kernel (k_plane), which needs no projector values: 13.4 + 5.6 us with the team kernel at 24 states.
+// 6.75 against 6.44 ms per td128 block.  At N = 32 every member runs alone, those of at most CTA_STATES states
+// by the CTA-wide plane kernel (k_plane), which needs no projector values: 7.8 us a plane pass of 8 states
+// against 10.8 with them, 38.4 against 35.5 at 128.  20 real-time steps, team against CTA-wide: 8.83 and
+// 8.76 ms at 65 states, 9.71 and 9.78 at 81, 10.42 and 10.57 at 96, 12.57 and 12.98 at 128.
 template <int N> struct PlaneForm {
-  static constexpr bool cta_per_member = N == 32;
-  static constexpr bool single_per_member = N == 96;
+  static constexpr int CTA_STATES = N == 32 ? 80 : 0;
+  static constexpr bool single_per_member = N == 96 || N == 32;
   static constexpr bool packed_for_single = N == 128;
 };
 
@@ -1650,17 +1652,19 @@ class FusedImpl final : public FusedOps {
       FusedImpl* f = static_cast<FusedImpl*>(it.ops);
       if (!same_geometry(f0, f)) fail(KS_ERR_ARG, "packed H application: the members' grids differ");
       if (it.n < 1 || it.n > f->ns_) fail(KS_ERR_ARG, "packed H application: member with %d states", it.n);
-      f->pre_h(it.psi, it.n, group_values(f->N_), s);
+      f->pre_h(it.psi, it.n, f->group_values(it.n), s);
     }
     f0->dispatch([&](auto tag) { group_launch<decltype(tag)::value>(items, s); });
   }
 
-  // whether the plane kernel of packed H applications reads the projector values
-  static bool group_values(int N) {
-    switch (N) {
-      case 48: case 54: case 64: case 72: case 96: case 108: case 128: return true;
-      default: return false;
-    }
+  // whether the plane kernel of a packed H application's member of n states reads the projector values
+  bool group_values(int n) {
+    bool team = false;
+    dispatch([&](auto tag) {
+      constexpr int N = decltype(tag)::value;
+      team = TPlan<N>::ok && n > PlaneForm<N>::CTA_STATES;
+    });
+    return team;
   }
 
   template <int N> static void group_launch(const std::vector<FusedGroupItem>& items, cudaStream_t s) {
@@ -1714,15 +1718,13 @@ class FusedImpl final : public FusedOps {
         }
         {
           ProfScope ps(f0->prof_, "plane", s);
-          if constexpr (PlaneForm<N>::cta_per_member) {
+          if constexpr (PlaneForm<N>::single_per_member) {
             for (size_t k = a; k < std::min(items.size(), a + GMAX); ++k) {
               FusedImpl* f = static_cast<FusedImpl*>(items[k].ops);
-              f->template launch_plane<N>(items[k].n, f->colbuf1_, f->pf_, s, 1);
-            }
-          } else if constexpr (PlaneForm<N>::single_per_member) {
-            for (size_t k = a; k < std::min(items.size(), a + GMAX); ++k) {
-              FusedImpl* f = static_cast<FusedImpl*>(items[k].ops);
-              f->template launch_plane_team_single<N>(items[k].n, s);
+              if (items[k].n <= PlaneForm<N>::CTA_STATES)
+                f->template launch_plane<N>(items[k].n, f->colbuf1_, f->pf_, s, 1);
+              else
+                f->template launch_plane_team_single<N>(items[k].n, s);
             }
           } else {
             launch_chain(f0->points(s0), k_plane_team_group<N>, dim3(N, s0), dim3(TCfg<N>::PT), smem, s, gd, f0->ncols_, f0->t_.col_xy,

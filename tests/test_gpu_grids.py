@@ -67,3 +67,10 @@ def test_fp64_planes(ks, meas, N, L, natoms, ns):
     g.density(n.data_ptr())
     meas("N=%d FP64 density" % N, rel(n.cpu().numpy(), ko.density(ref, c)), 1e-12)
     g.close()
+
+
+@pytest.mark.parametrize("ns", [1, 80, 81, 128])
+def test_realtime_32_plane_forms(ks, meas, ns):
+    """One ETRS step on 32^3 either side of the line between the plane kernel's two forms (bounds of
+    test_fused_grid)."""
+    test_fused_grid(ks, meas, 32, 10.0, 3, ns)
