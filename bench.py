@@ -269,8 +269,9 @@ def measured_traffic(name):
     return NCU_TRAFFIC_GS96["bytes"].get(name)
 
 
-# Stages that run as single-CTA kernels on the side stream, concurrently with the main stream's
-# whole-GPU kernels: rated against one SM's share of the peak, not chosen as the dominant kernel
+# Stages on the side stream, concurrent with the main stream's whole-GPU kernels: chains of
+# dependent steps in one CTA or a small cluster between short launches over more of the GPU; rated
+# against one SM's share of the peak, not chosen as the dominant kernel
 SIDE_STREAM = ("cholesky", "subspace", "eigh", "rr_step", "rot_prep", "ritz_values")
 
 
@@ -340,7 +341,7 @@ def roofline(entries, geo, pk, steps):
     pipeline is rated against HBM on the algorithmic bytes of the whole H psi it serves (one launch
     processes the block's states), with its share of the nominal FFT flops against the measured
     FP32 rate beside it; other stages by their own model.  Returns it, its name, and the
-    side-stream single-SM stages rated against one SM's share of the peak."""
+    side-stream stages rated against one SM's share of the peak."""
     leaf = {k: v for k, v in entries.items() if k != "apply_h" and k not in SIDE_STREAM}
     if not leaf:
         return None, None, []
@@ -587,8 +588,8 @@ def main_gpu(args):
         gp.set_states(c0)
         tp, _, pe = timed_steps(gp, 3, 1, lambda: gp.block_iteration(1, stream, precond="teter"), profile=True)
         tf, _, fe = timed_steps(gp, 2, 1, lambda: gp.forces(stream), profile=False)
-        forces = {"workload": "gs96, forces on the 64 atoms from the 128 states (Eq. 11): 4 full-grid transforms "
-                              "per state, real-space projections, separable local term",
+        forces = {"workload": "gs96, forces on the 64 atoms from the 128 states (Eq. 11): derivative planes "
+                              "of every state, real-space projections, separable local term",
                   "ms_per_call": statistics.mean(tf)}
         teter = {"workload": "gs96, one Teter-preconditioned block iteration per call",
                  "ms_per_iteration": statistics.mean(tp),
