@@ -14,11 +14,24 @@
 
 namespace ks {
 
-void StreamSet::create() {
-  int lo = 0, hi = 0;
-  KS_CUDA(cudaDeviceGetStreamPriorityRange(&lo, &hi));
-  KS_CUDA(cudaStreamCreateWithPriority(&side, cudaStreamNonBlocking, hi));
-  for (cudaEvent_t& e : ev) KS_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+StreamSet StreamSet::create() {
+  StreamSet set;
+  try {
+    int lo = 0, hi = 0;
+    KS_CUDA(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+    KS_CUDA(cudaStreamCreateWithPriority(&set.side, cudaStreamNonBlocking, hi));
+    for (cudaEvent_t& e : set.ev) KS_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  } catch (...) {
+    set.destroy();
+    throw;
+  }
+  return set;
+}
+
+bool StreamSet::complete() const {
+  for (cudaEvent_t e : ev)
+    if (!e) return false;
+  return side != nullptr;
 }
 
 void StreamSet::destroy() {
@@ -30,12 +43,9 @@ void StreamSet::destroy() {
 }
 
 void StreamHolder::acquire(DevicePool* pool) {
+  set_ = pool ? pool->take_streams() : StreamSet::create();
   pool_ = pool;
-  held_ = true;
-  if (pool_)
-    set_ = pool_->take_streams();
-  else
-    set_.create();
+  held_ = true;                      // only now is there a set to wait for and to give back
 }
 
 StreamHolder::~StreamHolder() {
@@ -57,18 +67,11 @@ StreamSet DevicePool::take_streams() {
       return set;
     }
   }
-  StreamSet set;
-  try {
-    set.create();
-  } catch (...) {
-    set.destroy();
-    throw;
-  }
-  return set;
+  return StreamSet::create();
 }
 
 void DevicePool::give_streams(StreamSet set) {
-  {
+  if (set.complete()) {
     std::lock_guard<std::mutex> lk(mu_);
     if ((int)idle_.size() < StreamSet::KEEP) {
       idle_.push_back(set);

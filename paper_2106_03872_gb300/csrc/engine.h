@@ -20,7 +20,8 @@ struct StreamSet {
   cudaStream_t main = nullptr;      // a request's work (created on first use)
   cudaStream_t side = nullptr;      // the engine's side stream, highest priority
   cudaEvent_t ev[EVENTS] = {};
-  void create();                    // side stream and events
+  static StreamSet create();        // side stream and events; nothing is left behind when it throws
+  bool complete() const;            // all of them are there
   void destroy();
 };
 
@@ -36,7 +37,7 @@ class DevicePool {
   ~DevicePool();
   void* alloc(size_t bytes);
   void free(void* p);
-  // A stream set (idle or new), and its return once its streams are idle.
+  // A stream set (idle or new), and its return once its streams are idle (an incomplete one is destroyed).
   StreamSet take_streams();
   void give_streams(StreamSet set);
   size_t reserved() const;   // bytes obtained from the device
