@@ -610,21 +610,22 @@ __global__ void k_teter_update(cplx<T>* __restrict__ psi, const cplx<T>* __restr
                                double tmin, int nG) {
   const int b = blockIdx.y;
   __shared__ T sh[3];
+  __shared__ bool live;                                              // R != 0
   if (threadIdx.x == 0) {
     double2 q = make_double2(0.0, 0.0);
     for (int i = 0; i < TETER_SPLIT; ++i) {
       q.x += part[(size_t)b * TETER_SPLIT + i].x;
       q.y += part[(size_t)b * TETER_SPLIT + i].y;
     }
-    const bool live = q.y > 0.0;
-    const double t = live ? fmax(q.x / q.y, tmin) : 1.0;
+    live = q.y > 0.0;
+    const double t = fmax(q.x / q.y, tmin);
     sh[0] = (T)(1.0 / t);
-    sh[1] = live ? (T)(1.0 / (t + shift)) : T(-1);
+    sh[1] = (T)(1.0 / (t + shift));                                  // negative for a coupling D below -(t + V's span)
     sh[2] = (T)eig[b];
   }
   __syncthreads();
+  if (!live) return;                                                 // uniform per block
   const T inv_t = sh[0], alpha = sh[1], e = sh[2];
-  if (alpha < T(0)) return;                                          // uniform per block
   for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < nG; g += gridDim.x * blockDim.x) {
     const T x = g2h[g] * inv_t;
     const T p = T(27) + x * (T(18) + x * (T(12) + x * T(8)));
