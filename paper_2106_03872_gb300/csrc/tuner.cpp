@@ -40,6 +40,13 @@ int tune_choice(const std::string& key, int ncand, const std::function<void(int)
     if (it != decisions().end()) return it->second.choice;
   }
   if (ncand <= 1) return 0;
+  // a stream under capture cannot be timed (its events never complete): the first candidate, and the key
+  // stays undecided
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return 0;
+  }
   constexpr int REPS = 3;
   cudaEvent_t a, b;
   KS_CUDA(cudaEventCreate(&a));

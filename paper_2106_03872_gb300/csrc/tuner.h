@@ -14,7 +14,8 @@
 namespace ks {
 
 // Index of the fastest of ncand candidates for `key`: run(c) launches candidate c on stream s.
-// Cached after the first call; thread-safe.
+// Cached after the first call; thread-safe.  On a stream under capture an undecided key gives the
+// first candidate, untimed.
 int tune_choice(const std::string& key, int ncand, const std::function<void(int)>& run, cudaStream_t s,
                 const char* const* names);
 // The kept choice of a key, or -1 while it has not been timed.

@@ -35,3 +35,32 @@ def test_teter_step_of_negative_length(ks, meas, prec, tol):
     g.block_iteration(1, precond="teter")
     meas("states after a step of negative length", rel(g.get_states(), ko.block_iteration_teter(ref, c, 1)[1]), tol)
     g.close()
+
+
+@pytest.mark.parametrize("N,L", [(54, 16.875), (96, 30.0)])
+def test_first_call_under_capture(ks, meas, N, L):
+    """H psi and the density captured into a graph by the first calls of their size class (130 states: no
+    other test's): nothing is timed on the capturing stream.  Bounds of the fused grids' parity tests."""
+    ns = 130
+    cell = inputs.small_cell(L, N, 2, ns, 72, depth=-3.0)
+    g = ks.Grid(cell, prec="bf16x3")
+    c = inputs.random_coeffs(72, 2, g.nG)
+    ref = ko.Cell(cell)
+    psi = torch.from_numpy(c).to("cuda", torch.complex64).repeat(ns // 2, 1)
+    h, n = torch.zeros_like(psi), torch.zeros((N, N, N), dtype=torch.float32, device="cuda")
+    g.set_states(np.tile(c, (ns // 2, 1)))
+    torch.cuda.synchronize()
+    graph, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=s):
+        g.apply_h(psi.data_ptr(), h.data_ptr(), ns, stream=s)
+        g.density(n.data_ptr(), stream=s)
+    for _ in range(2):
+        h.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+    got = h.cpu().numpy().astype(np.complex128)
+    expect = ko.apply_h(ref, c)
+    for k in (0, 1, ns - 2, ns - 1):
+        meas("N=%d captured H psi" % N, rel(got[k], expect[k % 2]), 2e-5)
+    meas("N=%d captured density" % N, rel(n.cpu().numpy().astype(float), ns // 2 * ko.density(ref, c)), 1e-5)
+    g.close()
