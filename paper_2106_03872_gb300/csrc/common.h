@@ -183,5 +183,7 @@ void build_geometry(const ks_cell_desc& d, HostGeometry& g);
 // for new positions pos [natoms][3] of the same atoms.  V_loc, vmin and vmax are the
 // engine's to fill (on the device).
 void build_atoms(const double* pos, HostGeometry& g);
+// Grid steps from its centre beyond which a Gaussian of this width is below 1e-20 (at most N).
+int gaussian_half_box(double width, double h, int N);
 
 }  // namespace ks

@@ -1509,7 +1509,7 @@ template <typename T> class Engine final : public EngineBase {
         }
     KS_CUDA(cudaMemcpyAsync(fxyz_, xyz.data(), xyz.size() * sizeof(double), cudaMemcpyHostToDevice, s));
     // the grid indices around each atom outside which its factor is below 1e-20 (the local force's box)
-    const int hw = (int)std::ceil(g_.vloc_width * std::sqrt(2.0 * std::log(1e20)) / g_.h);
+    const int hw = gaussian_half_box(g_.vloc_width, g_.h, N);
     fcnt_ = std::min(N, 2 * hw + 2);
     std::vector<int> first(3 * (size_t)na);
     for (int i = 0; i < 3 * na; ++i)

@@ -206,6 +206,10 @@ void build_atoms(const double* pos, HostGeometry& g) {
 
 }
 
+int gaussian_half_box(double width, double h, int N) {
+  return (int)std::min<double>(N, std::ceil(width * std::sqrt(2.0 * std::log(1e20)) / h));   // any width > 0, inf too
+}
+
 void build_geometry(const ks_cell_desc& d, HostGeometry& g) {
   if (d.natoms < 0 || (d.natoms > 0 && !d.pos)) fail(KS_ERR_ARG, "natoms=%d with pos=%p", d.natoms, (const void*)d.pos);
   if (d.nproj != 1 && d.nproj != 4) fail(KS_ERR_ARG, "nproj must be 1 or 4, got %d", d.nproj);

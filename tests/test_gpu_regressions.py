@@ -64,3 +64,19 @@ def test_first_call_under_capture(ks, meas, N, L):
         meas("N=%d captured H psi" % N, rel(got[k], expect[k % 2]), 2e-5)
     meas("N=%d captured density" % N, rel(n.cpu().numpy().astype(float), ns // 2 * ko.density(ref, c)), 1e-5)
     g.close()
+
+
+@pytest.mark.parametrize("width", [4e7, 1e11, np.inf])
+def test_forces_of_a_flat_local_potential(ks, meas, width):
+    """Widths whose box of grid points overflowed an integer: V_loc is constant, so the local sums cancel to
+    the rounding of V times the gradient density (FP64 1e-12; FP32 gradients of a few 6e-8: 1e-6)."""
+    cell = dict(inputs.small_cell(10.0, 24, 2, 3, 73, depth=-0.1), vloc_width=width)
+    ref = ko.Cell(cell)
+    q, _ = ko.cholqr(inputs.random_coeffs(73, 3, ref.nG))
+    F_ref = ko.forces(ref, q)
+    scale = np.max(np.abs(F_ref)) + np.max(np.abs(ref.vloc))
+    for prec, tol in (("fp64", 1e-12), ("bf16x3", 1e-6)):
+        g = ks.Grid(cell, prec=prec)
+        g.set_states(q)
+        meas("width %g, %s" % (width, prec), np.max(np.abs(g.forces() - F_ref)), tol * scale)
+        g.close()
