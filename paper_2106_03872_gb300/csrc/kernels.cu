@@ -240,7 +240,9 @@ __global__ void __launch_bounds__(128)
 // arithmetic (conversions too) would bound it on FP32 fields, so there the FP64 factors are split into two
 // FP32 parts, the products are exact (with their rounding errors by fma) and the sums compensated, which
 // keeps about 45 bits: over the whole grid in FP64, the 64 atoms of a 96^3 cell took 0.72 ms, over the
-// boxes 0.27 ms, so 0.067 ms.
+// boxes 0.27 ms, so 0.067 ms.  On FP64 fields a warp takes four rows at a time: a row at a time, waiting for
+// each row's loads, 27 atoms of a 48^3 cell, whose boxes are the whole grid, took 0.155 ms (and the plain
+// sum over the grid 0.055 ms); four at a time 0.050 ms.
 template <typename T>
 __global__ void __launch_bounds__(RED_THREADS)
     k_local_force(const T* __restrict__ g, const double* __restrict__ xyz, const int* __restrict__ start, int cnt, int N,
@@ -266,16 +268,18 @@ __global__ void __launch_bounds__(RED_THREADS)
   }
   double acc[3] = {0.0, 0.0, 0.0};
   SumPair S[3];
+  constexpr int WARPS = RED_THREADS / 32;
   const int rows = cnt * cnt, r0 = rows * sl / LOCAL_FORCE_SPLIT, r1 = rows * (sl + 1) / LOCAL_FORCE_SPLIT;
-  for (int rb = r0 + 32 * warp; rb < r1; rb += RED_THREADS) {
+  const int w0 = r0 + (r1 - r0) * warp / WARPS, w1 = r0 + (r1 - r0) * (warp + 1) / WARPS;
+  for (int rb = w0; rb < w1; rb += 32) {
     // 32 rows of a warp: lane k forms the product of row k's two outer factors
-    const int mr = min(rb + lane, r1 - 1), m2 = wrap(s2 + mr / cnt), m1 = wrap(s1 + mr % cnt);
+    const int mr = min(rb + lane, w1 - 1), m2 = wrap(s2 + mr / cnt), m1 = wrap(s1 + mr % cnt);
     const double v = T2[m2] * T1[m1];
     const float vh = (float)v, vl = (float)(v - (double)vh);
-    const int at = m2 * N + m1, nr = min(32, r1 - rb);
-    for (int k = 0; k < nr; ++k) {
-      const T* row = g + (size_t)__shfl_sync(0xffffffffu, at, k) * N;
-      if constexpr (SPLIT) {
+    const int at = m2 * N + m1, nr = min(32, w1 - rb);
+    if constexpr (SPLIT) {
+      for (int k = 0; k < nr; ++k) {
+        const T* row = g + (size_t)__shfl_sync(0xffffffffu, at, k) * N;
         const float wh = __shfl_sync(0xffffffffu, vh, k), wl = __shfl_sync(0xffffffffu, vl, k);
         SumPair t[3];
         for (int i = lane; i < cnt; i += 32) {
@@ -292,17 +296,33 @@ __global__ void __launch_bounds__(RED_THREADS)
           const float p = wh * t[a].s;
           S[a].add(p, fmaf(wh, t[a].s, -p) + (wl * t[a].s + wh * t[a].c));
         }
-      } else {
-        const double w = __shfl_sync(0xffffffffu, v, k);
-        double t[3] = {0.0, 0.0, 0.0};
+      }
+    } else {
+      // RB rows at a time, their loads issued together
+      constexpr int RB = 4;
+      for (int k = 0; k < nr; k += RB) {
+        const T* row[RB];
+        double w[RB], t[RB][3] = {};
+#pragma unroll
+        for (int q = 0; q < RB; ++q) {
+          const int kq = min(k + q, nr - 1);                         // past the rows: the last one again, not added
+          row[q] = g + (size_t)__shfl_sync(0xffffffffu, at, kq) * N;
+          w[q] = __shfl_sync(0xffffffffu, v, kq);
+        }
         for (int i = lane; i < cnt; i += 32) {
           const int j0 = wrap(s0 + i);
           const double f = T0[j0];
 #pragma unroll
-          for (int a = 0; a < 3; ++a) t[a] = fma(f, (double)row[a * N3 + j0], t[a]);
+          for (int q = 0; q < RB; ++q)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) t[q][a] = fma(f, (double)row[q][a * N3 + j0], t[q][a]);
         }
 #pragma unroll
-        for (int a = 0; a < 3; ++a) acc[a] = fma(w, t[a], acc[a]);
+        for (int q = 0; q < RB; ++q)
+          if (k + q < nr) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) acc[a] = fma(w[q], t[q][a], acc[a]);
+          }
       }
     }
   }

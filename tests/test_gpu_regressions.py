@@ -80,3 +80,21 @@ def test_forces_of_a_flat_local_potential(ks, meas, width):
         g.set_states(q)
         meas("width %g, %s" % (width, prec), np.max(np.abs(g.forces() - F_ref)), tol * scale)
         g.close()
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-12), ("bf16x3", 1e-4)])
+@pytest.mark.parametrize("N,L,face", [(48, 15.0, 0.1), (64, 20.0, 19.9), (72, 30.0, 0.0)])
+def test_local_force_boxes(ks, meas, prec, tol, N, L, face):
+    """The local force over boxes that are the whole grid (48 points) or a part of it that wraps around the
+    cell's faces, with occupations of every size.  Bounds of the force parity tests."""
+    cell = inputs.small_cell(L, N, 2, 3, 74, depth=-3.0)
+    cell["pos"][0] = [face, L - 0.3, 0.5 * L]
+    occ = np.array([2.0, 1.25, 0.5])
+    ref = ko.Cell(dict(cell, occ=occ))
+    q, _ = ko.cholqr(inputs.random_coeffs(74, 3, ref.nG))
+    q = ko.block_iteration(ref, q, 2)[1]
+    F_ref = ko.forces(ref, q)
+    g = ks.Grid(cell, prec=prec, occ=occ)
+    g.set_states(q)
+    meas("N=%d forces" % N, np.max(np.abs(g.forces() - F_ref)), tol * np.max(np.abs(F_ref)))
+    g.close()
