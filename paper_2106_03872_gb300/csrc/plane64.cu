@@ -7,6 +7,10 @@
 // The FP64 pipe bounds them (two lanes a clock per SM: the transforms of an H application of 8 states on
 // 24^3 take 22 us of it); as six passes through HBM with run-time lengths they took 15, 15 and 10 us a
 // pass there, the whole H application 88 us; with these it takes 78 us.
+//
+// Only the planes that hold columns are launched, 2 xr + 1 of N: with the others' CTAs in the grid, which
+// left at once, the scheduler put two planes on some multiprocessors and none on others (3 states on 54^3
+// 275 -> 208 us an H application, 6 states on 36^3 160 -> 115 us).
 #include "fft_device.cuh"
 #include "kernels.h"
 
@@ -23,6 +27,8 @@ template <int N> struct P64 {
 };
 
 __device__ __forceinline__ bool in_band(int x, int N, int xr) { return x <= xr || x >= N - xr; }
+// The p-th x-plane that holds columns, p < 2 xr + 1; the others are zero and the x lines do not read them.
+__device__ __forceinline__ int band_plane(int p, int N, int xr) { return p <= xr ? p : N - (2 * xr + 1) + p; }
 
 template <int N>
 __global__ void __launch_bounds__(P64<N>::PT)
@@ -32,8 +38,7 @@ __global__ void __launch_bounds__(P64<N>::PT)
   extern __shared__ __align__(16) double2 p64sm[];
   chain_begin();
   double2 *tw = p64sm, *P = p64sm + N;                               // [y][z]
-  const int x = blockIdx.x, b = blockIdx.y;
-  if (!in_band(x, N, xr)) return;                                    // a plane of zeros: the x lines do not read it
+  const int x = band_plane(blockIdx.x, N, xr), b = blockIdx.y;
   for (int t = threadIdx.x; t < N; t += PT) tw[t] = twg[t];
   const int* gi = ginv + x * N * N;
   for (int e = threadIdx.x; e < N * N; e += PT) {
@@ -79,8 +84,7 @@ __global__ void __launch_bounds__(P64<N>::PT)
   extern __shared__ __align__(16) double2 p64sm[];
   chain_begin();
   double2 *tw = p64sm, *P = p64sm + N;                               // [y][z]
-  const int x = blockIdx.x, b = blockIdx.y;
-  if (!in_band(x, N, xr)) return;                                    // no sphere points
+  const int x = band_plane(blockIdx.x, N, xr), b = blockIdx.y;
   for (int t = threadIdx.x; t < N; t += PT) tw[t] = twg[t];
   const double2* in = grid + ((size_t)b * N + x) * N * N;
   for (int e = threadIdx.x; e < N * N; e += PT) P[(e / N) * ld + e % N] = in[e];
@@ -98,19 +102,51 @@ __global__ void __launch_bounds__(P64<N>::PT)
   }
 }
 
+// Whether nb states go through planes.  Their launch fills the GPU in steps of one plane an SM; where it
+// leaves most of the last step empty, the line passes, which spread evenly, are faster: they win from
+// LINES times as many plane slots as the nb N planes of the whole grids (us of an H application, planes and
+// lines: 150 and 94 for 1 state on 48^3, slots 3.2 times the planes; 174 and 134 for 1 on 54^3, 2.8; 163 and
+// 127 for 1 on 64^3, 2.4; 279 and 252 for 1 on 72^3, 2.1, and 507 and 450 for 3 with 61 planes each, 1.41;
+// level for 2 on 36^3, 2.1; but 186 and 235 for 2 on 54^3, 1.41, and 352 and 372 for 1 on 96^3, 1.58).  Up to
+// 32 points the launches count, two less with planes.
+constexpr int SMS = 152;
+template <int N> bool planes_pay(int nb, int xr) {
+  constexpr double LINES = N == 72 ? 1.4 : 2.2;
+  const long planes = (long)nb * (2 * xr + 1), slots = (planes + SMS - 1) / SMS * SMS;
+  return N <= 32 || slots <= LINES * nb * N;
+}
+
+// The element count that decides on a chained launch (launch_chain) of the forward passes.  Where mid-sized
+// work leaves SMs idle, the planes of the last pass, set up early, pile up on them and then run several to
+// an SM while the others have none: 3 us of launch latency hidden, up to 70 us lost (H application of 2
+// states on 72^3 374 us chained, 300 not; 6 on 36^3 147 and 111; 2 on 64^3 220 and 178).  Chained: the
+// smallest work (24^3, 4 states: 57 and 68 us), grids from 48 points on whose planes fill the SMs (64^3, 4
+// states: 288 and 300), and 96 points, whose planes take an SM's whole shared memory (1 state: 338 and 352).
+// The inverse passes are level at every size and always chained.
+template <int N> size_t chain_elems(int nb, int xr) {
+  const size_t pts = (size_t)nb * N * N * N;
+  const bool chain = pts <= (size_t(1) << 17) || N >= 96 || (N >= 48 && (long)nb * (2 * xr + 1) >= SMS);
+  return chain ? pts : CHAIN_ELEMS + 1;
+}
+
 template <int N> struct NTag {
   static constexpr int value = N;
 };
-template <typename F> bool with_n(int N, F&& f) {
+template <typename F> bool with_planes(int N, int nb, int xr, F&& f) {
+  auto go = [&](auto tag) {
+    if (!planes_pay<decltype(tag)::value>(nb, xr)) return false;
+    f(tag);
+    return true;
+  };
   switch (N) {
-    case 24: f(NTag<24>{}); return true;
-    case 32: f(NTag<32>{}); return true;
-    case 36: f(NTag<36>{}); return true;
-    case 48: f(NTag<48>{}); return true;
-    case 54: f(NTag<54>{}); return true;
-    case 64: f(NTag<64>{}); return true;
-    case 72: f(NTag<72>{}); return true;
-    case 96: f(NTag<96>{}); return true;
+    case 24: return go(NTag<24>{});
+    case 32: return go(NTag<32>{});
+    case 36: return go(NTag<36>{});
+    case 48: return go(NTag<48>{});
+    case 54: return go(NTag<54>{});
+    case 64: return go(NTag<64>{});
+    case 72: return go(NTag<72>{});
+    case 96: return go(NTag<96>{});
     default: return false;
   }
 }
@@ -119,7 +155,7 @@ template <typename F> bool with_n(int N, F&& f) {
 
 bool plane64_inverse(const double2* psi, double2* grid, const int* ginv, const DevTables<double>& t, int nb,
                      cudaStream_t s) {
-  return with_n(t.N, [&](auto tag) {
+  return with_planes(t.N, nb, t.xr, [&](auto tag) {
     constexpr int N = decltype(tag)::value;
     static bool attr = false;
     if (!attr) {
@@ -127,7 +163,8 @@ bool plane64_inverse(const double2* psi, double2* grid, const int* ginv, const D
       attr = true;
     }
     const size_t pts = (size_t)nb * N * N * N;
-    launch_chain(pts, k_p64_inv<N>, dim3(N, nb), dim3(P64<N>::PT), P64<N>::SMEM, s, psi, t.nG, ginv, t.xr, grid, t.tw);
+    launch_chain(pts, k_p64_inv<N>, dim3(2 * t.xr + 1, nb), dim3(P64<N>::PT), P64<N>::SMEM, s, psi, t.nG, ginv,
+                 t.xr, grid, t.tw);
     launch_chain(pts, k_p64_x<N, +1>, dim3((N + P64<N>::LB - 1) / P64<N>::LB, N, nb), dim3(P64<N>::PT), P64<N>::XSMEM, s,
                  grid, t.xr, t.tw);
   });
@@ -135,18 +172,18 @@ bool plane64_inverse(const double2* psi, double2* grid, const int* ginv, const D
 
 bool plane64_forward(double2* grid, const double2* psi, double2* hpsi, const int* ginv, const DevTables<double>& t,
                      int nb, double scale, cudaStream_t s) {
-  return with_n(t.N, [&](auto tag) {
+  return with_planes(t.N, nb, t.xr, [&](auto tag) {
     constexpr int N = decltype(tag)::value;
     static bool attr = false;
     if (!attr) {
       KS_CUDA(cudaFuncSetAttribute(k_p64_fwd<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P64<N>::SMEM));
       attr = true;
     }
-    const size_t pts = (size_t)nb * N * N * N;
+    const size_t pts = chain_elems<N>(nb, t.xr);
     launch_chain(pts, k_p64_x<N, -1>, dim3((N + P64<N>::LB - 1) / P64<N>::LB, N, nb), dim3(P64<N>::PT), P64<N>::XSMEM, s,
                  grid, t.xr, t.tw);
-    launch_chain(pts, k_p64_fwd<N>, dim3(N, nb), dim3(P64<N>::PT), P64<N>::SMEM, s, grid, psi, hpsi, t.nG, ginv, t.g2half,
-                 t.xr, scale, t.tw);
+    launch_chain(pts, k_p64_fwd<N>, dim3(2 * t.xr + 1, nb), dim3(P64<N>::PT), P64<N>::SMEM, s, grid, psi, hpsi, t.nG,
+                 ginv, t.g2half, t.xr, scale, t.tw);
   });
 }
 

@@ -98,3 +98,25 @@ def test_local_force_boxes(ks, meas, prec, tol, N, L, face):
     g.set_states(q)
     meas("N=%d forces" % N, np.max(np.abs(g.forces() - F_ref)), tol * np.max(np.abs(F_ref)))
     g.close()
+
+
+@pytest.mark.parametrize("N,L,ns", [(32, 13.3, 1), (36, 11.25, 2), (36, 11.25, 3), (48, 20.0, 1), (48, 20.0, 2), (54, 16.875, 1),
+                                    (54, 22.5, 4), (64, 20.0, 1), (64, 26.6, 3), (72, 30.0, 1), (72, 22.5, 3),
+                                    (72, 30.0, 3), (72, 30.0, 4), (96, 30.0, 1), (108, 33.75, 2), (128, 40.0, 1)])
+def test_fp64_routes(ks, meas, N, L, ns):
+    """FP64 H psi and density either side of the line between whole planes and line passes, and on the grids
+    that have line passes only: 1e-12, as on every FP64 path."""
+    cell = inputs.small_cell(L, N, 3, ns, 75, depth=-3.0)
+    ref = ko.Cell(cell)
+    c = inputs.random_coeffs(75, ns, ref.nG)
+    g = ks.Grid(cell, prec="fp64")
+    psi = torch.from_numpy(c).to("cuda")
+    h = torch.full_like(psi, float("nan"))
+    g.apply_h(psi.data_ptr(), h.data_ptr(), ns)
+    torch.cuda.synchronize()
+    meas("N=%d, %d states: H psi" % (N, ns), rel(h.cpu().numpy(), ko.apply_h(ref, c)), 1e-12)
+    g.set_states(c)
+    n = torch.empty((N, N, N), dtype=torch.float64, device="cuda")
+    g.density(n.data_ptr())
+    meas("N=%d, %d states: density" % (N, ns), rel(n.cpu().numpy(), ko.density(ref, c)), 1e-12)
+    g.close()
