@@ -774,7 +774,9 @@ inline unsigned blocks_for(size_t n, int threads, unsigned cap = 152u * 16u) {
 // ------------------------------------------------------------------------------------------
 // Lines per CTA: as many as its shared memory holds, but fewer where the launch would leave
 // multiprocessors without a CTA (24^3 with 8 states: 54 CTAs of 85 lines took 18 us a pass in FP64, whose
-// pipe on every SM needs 4 us); at least 16 of a strided pass, whose rows are then 128 or 256 bytes.
+// pipe on every SM needs 4 us); at least 16 of a strided pass, whose rows are then 128 or 256 bytes.  The
+// tiles of a strided pass are equal, in whole sectors: 34 lines of 36 would leave every second CTA 2 (FP64
+// forces of 8 states on 36^3 0.55 ms a call, in equal tiles 0.51 ms).
 template <typename T, int MODE>
 static void fft_lines(cplx<T>* grid, int nb, int N, int axis, int sign, const cplx<T>* tw, const SphereEnd<T>& sp,
                       cudaStream_t s) {
@@ -783,7 +785,10 @@ static void fft_lines(cplx<T>* grid, int nb, int N, int axis, int sign, const cp
   const int B = axis == 2 ? 1 : (axis == 1 ? N : N * N);
   const long lines = (long)nb * N * N;
   int TB = std::max(1, std::min<int>(LINE_ELEMS / N, (int)std::max<long>(16, lines / (2 * 152))));
-  if (B > 1 && TB > B) TB = B;
+  if (B > 1) {
+    const int ntb = (B + TB - 1) / TB, sector = 32 / (int)sizeof(cplx<T>);
+    TB = std::min(TB, ((B + ntb - 1) / ntb + sector - 1) / sector * sector);
+  }
   const long nblocks = (B == 1) ? (nouter + TB - 1) / TB : nouter * ((B + TB - 1) / TB);
   const size_t smem = (size_t)(N + TB * (N + 1)) * sizeof(cplx<T>);
   launch_chain((size_t)lines * N, k_fft_lines<T, MODE>, dim3((unsigned)nblocks), dim3(LINE_THREADS), smem, s, grid, N,
