@@ -43,7 +43,8 @@ __device__ __forceinline__ void block_sum(double (&v)[NV]) {
 // Packed sphere coefficients at either end of a z pass (axis 2): ginv [N^3] is the packed index of a grid
 // point, or -1.  Reading them there saves the grid's clearing and the scatter, and keeping only S on the
 // way out the gather with the kinetic term: three launches and two passes over the grids of an H
-// application.
+// application.  A CTA whose lines hold no point of S (two thirds of them) transforms nothing: with all lines
+// transformed, 12 FP64 states on 108^3 took 5.51 ms an H application, against 5.37 ms with the gather; now 4.55.
 template <typename T> struct SphereEnd {
   const int* ginv = nullptr;
   const cplx<T>* psi = nullptr;    // packed states [b][nG] (read: the transform's input; written: T c)
@@ -71,18 +72,32 @@ __global__ void __launch_bounds__(LINE_THREADS) k_fft_lines(cplx<T>* __restrict_
   int lines;
   size_t base;
   long a0 = 0;
+  const int NN = N * N;
+  // packed index of element k of line a0 + l (axis 2; the lines of a batch fit an int), or -1
+  auto sphere_index = [&](int l, int k) { return sp.ginv[((int)a0 + l) % NN * N + k]; };
   if (B == 1) {
     a0 = (long)blockIdx.x * TB;
     lines = (int)min((long)TB, nouter - a0);
     base = (size_t)a0 * N;
+    bool any = false;                                                // a point of S on these lines
+    if constexpr (MODE == LINES_TO_SPHERE) {
+      for (int e = threadIdx.x; e < lines * N; e += blockDim.x) any |= sphere_index(e / N, e % N) >= 0;
+      if (!__syncthreads_or(any)) return;
+    }
     for (int e = threadIdx.x; e < lines * N; e += blockDim.x) {
       const int l = e / N, k = e - (e / N) * N;
       if constexpr (MODE == LINES_FROM_SPHERE) {
-        const long line = a0 + l, st = line / ((long)N * N);
-        const int g = sp.ginv[(line - st * N * N) * N + k];
+        const int st = ((int)a0 + l) / NN, g = sphere_index(l, k);
+        any |= g >= 0;
         s[l * ld + k] = g >= 0 ? sp.psi[(size_t)st * sp.nG + g] : mk<C>(T(0), T(0));
       } else {
         s[l * ld + k] = data[base + (size_t)l * N + k];
+      }
+    }
+    if constexpr (MODE == LINES_FROM_SPHERE) {
+      if (!__syncthreads_or(any)) {
+        for (int e = threadIdx.x; e < lines * N; e += blockDim.x) data[base + e] = mk<C>(T(0), T(0));
+        return;
       }
     }
   } else {
@@ -103,10 +118,9 @@ __global__ void __launch_bounds__(LINE_THREADS) k_fft_lines(cplx<T>* __restrict_
       const int l = e / N, k = e - (e / N) * N;
       const C u = s[l * ld + k];
       if constexpr (MODE == LINES_TO_SPHERE) {
-        const long line = a0 + l, st = line / ((long)N * N);
-        const int g = sp.ginv[(line - st * N * N) * N + k];
+        const int g = sphere_index(l, k);
         if (g >= 0) {
-          const size_t i = (size_t)st * sp.nG + g;
+          const size_t i = (size_t)(((int)a0 + l) / NN) * sp.nG + g;
           const C c = sp.psi[i];
           const T kin = sp.g2h[g];
           sp.hpsi[i] = mk<C>(u.x * sp.scale + kin * c.x, u.y * sp.scale + kin * c.y);
