@@ -49,7 +49,8 @@ typedef enum {
  *   KS_FP64          complex128 states, FP64 FFTs, FP64 everything (correctness anchor).
  *   KS_MIXED_BF16X3  complex64 states and FFTs; projector and Gram/rotation GEMMs on the
  *                    tensor cores with each FP32 operand split into two bf16 terms (3
- *                    products), FP32 accumulation; the Cholesky factor and the subspace
+ *                    products), FP32 accumulation (projections of grids of 8, 12, 16, 54, 72
+ *                    and 108 points: sums over the grid); the Cholesky factor and the subspace
  *                    eigensolver in FP32 with FP64 refinement (FP64 Rayleigh quotients for the
  *                    reported eigenvalues; FP64 throughout with KS_OPT_FP64_SUBSPACE); norms
  *                    and energies in FP64. */

@@ -1271,9 +1271,12 @@ __global__ void __launch_bounds__(FCfg<N>::PT, FCfg<N>::PMIN)
 // at the plane's covered points to val[b][point] for the projections, so d psi never goes to the grid.
 // Full-grid stores of psi and three derivatives, four passes over the spheres in them and three passes
 // summing the products took 7.05 ms a call on 128 states of 96^3; this form takes 2.46 ms (a derivative
-// 0.46 ms, of which the density kernel's transforms are 0.42).
-template <int N, bool GRAD>
-__global__ void __launch_bounds__(TCfg<N>::PT, TCfg<N>::PMIN)
+// 0.46 ms, of which the density kernel's transforms are 0.42).  STORE = false: psi's covered points alone (the
+// projections of an H application on the grids of real_space_projections), planes without any left out.
+// On 54 points that form's blocks of 192 threads run four to an SM (two, with twice the registers: projections
+// of 24 states and 40 atoms 41 us, now 34 us).
+template <int N, bool GRAD, bool STORE = true>
+__global__ void __launch_bounds__(TCfg<N>::PT, STORE || N != 54 ? TCfg<N>::PMIN : 4)
     k_plane_force_team(const float2* __restrict__ colbuf, int ncols, const int* __restrict__ col_xy, int xr,
                        const int* __restrict__ rowym, int nstates, int chunk, const double* __restrict__ occ, int axis,
                        float g0, float2* __restrict__ grid, float* __restrict__ partial, TeamNL nl,
@@ -1290,6 +1293,7 @@ __global__ void __launch_bounds__(TCfg<N>::PT, TCfg<N>::PMIN)
   int* loff = reinterpret_cast<int*>(bits + N * NW);
   int* yms = loff + N;
   const int z = blockIdx.x, ch = blockIdx.y;
+  if (!GRAD && !STORE && nl.pt_off[z] == nl.pt_off[z + 1]) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int team = warp / W, wi = warp - team * W;
   const int l = team * 32 + lane;
@@ -1314,12 +1318,20 @@ __global__ void __launch_bounds__(TCfg<N>::PT, TCfg<N>::PMIN)
     for (int c = threadIdx.x; c < ncols; c += PT) {
       const int xy = col_xy[c];
       const int jx = xy / N, jy = xy - jx * N;
-      float2 v = src[c];
-      if (GRAD && axis < 2) {
-        const float G = g0 * (float)grid_freq(axis == 0 ? jx : jy, N);
-        v = make_float2(-G * v.y, G * v.x);
+      if constexpr (GRAD) {
+        float2 v = src[c];
+        if (axis < 2) {
+          const float G = g0 * (float)grid_freq(axis == 0 ? jx : jy, N);
+          v = make_float2(-G * v.y, G * v.x);
+        }
+        P[jx * ld + jy] = v;
+      } else {
+        cp_async8(P + jx * ld + jy, src + c);
       }
-      P[jx * ld + jy] = v;
+    }
+    if constexpr (!GRAD) {
+      cp_async_commit();
+      cp_async_wait_all();
     }
     __syncthreads();
     team_lines<N, +1, 1>(P, nband, RowOff<N>{xr}, tw, ColMask<N>{yms});
@@ -1367,7 +1379,7 @@ __global__ void __launch_bounds__(TCfg<N>::PT, TCfg<N>::PMIN)
           for (int r = 0; r < R2; ++r) u[r] = plane[(size_t)(j + r * R1) * N];
 #pragma unroll
           for (int r = 0; r < R2; ++r) accs[(j + r * R1) * N + l] += f2 * (v[r].x * u[r].x + v[r].y * u[r].y);
-        } else {
+        } else if constexpr (STORE) {
 #pragma unroll
           for (int r = 0; r < R2; ++r) plane[(size_t)(j + r * R1) * N] = v[r];
         }
@@ -1404,39 +1416,43 @@ __global__ void __launch_bounds__(256) k_add_partials(const float* __restrict__ 
   }
 }
 
-// proj[b][I][l] = scale sum over atom I's sphere points of beta_l val[b][slot], one warp per atom and
+// proj[b][I][l] = scale sum over atom I's sphere points of beta_l val[b][slot], S warps per atom and
 // state.  slot and beta list the atom's points in increasing covered point.  The products are exact
-// (product and its rounding error by fma) and summed with compensation, across the lanes too: about FP64's
-// precision without its pipe (FP64 sums took 0.2 ms per field of 128 states and 64 atoms, FP64 only for
-// the sums across lanes 0.27 ms).
+// (product and its rounding error by fma) and summed with compensation, across the lanes and warps too: about
+// FP64's precision without its pipe (FP64 sums took 0.2 ms per field of 128 states and 64 atoms, FP64 only for
+// the sums across lanes 0.27 ms).  Latency of the scattered loads bounds it: with one warp for the 1100 points
+// of an atom, 23 atoms and 37 states took 36 us (5.6 warps an SM), with four 13 us.
 constexpr int PJW = 8;
-template <int NP>
+template <int NP, int S>
 __global__ void __launch_bounds__(32 * PJW)
     k_project_points(const float2* __restrict__ val, int npts, const int* __restrict__ sph_off,
                      const int* __restrict__ slot, const float* __restrict__ beta, int natoms, int n, float scale,
                      float2* __restrict__ proj) {
+  __shared__ float2 red[PJW][NP][2];                                 // a warp's sums and their errors
   chain_begin();
-  const int I = blockIdx.x, lane = threadIdx.x & 31, b = blockIdx.y * PJW + (threadIdx.x >> 5);
-  if (b >= n) return;
-  const float2* vb = val + (size_t)b * npts;
+  const int I = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sl = warp % S;
+  const int b = blockIdx.y * (PJW / S) + warp / S;
   SumPair t[NP][2];
+  if (b < n) {
+    const float2* vb = val + (size_t)b * npts;
 #pragma unroll 4
-  for (int q = sph_off[I] + lane; q < sph_off[I + 1]; q += 32) {
-    const float2 v = vb[slot[q]];
-    float w[NP];
-    if constexpr (NP == 4) {
-      const float4 f = *reinterpret_cast<const float4*>(beta + (size_t)q * 4);
-      w[0] = f.x;
-      w[1] = f.y;
-      w[2] = f.z;
-      w[3] = f.w;
-    } else {
-      w[0] = beta[q];
-    }
+    for (int q = sph_off[I] + 32 * sl + lane; q < sph_off[I + 1]; q += 32 * S) {
+      const float2 v = vb[slot[q]];
+      float w[NP];
+      if constexpr (NP == 4) {
+        const float4 f = *reinterpret_cast<const float4*>(beta + (size_t)q * 4);
+        w[0] = f.x;
+        w[1] = f.y;
+        w[2] = f.z;
+        w[3] = f.w;
+      } else {
+        w[0] = beta[q];
+      }
 #pragma unroll
-    for (int l = 0; l < NP; ++l) {
-      t[l][0].add_product(w[l], v.x);
-      t[l][1].add_product(w[l], v.y);
+      for (int l = 0; l < NP; ++l) {
+        t[l][0].add_product(w[l], v.x);
+        t[l][1].add_product(w[l], v.y);
+      }
     }
   }
 #pragma unroll
@@ -1450,10 +1466,18 @@ __global__ void __launch_bounds__(32 * PJW)
       }
   if (lane == 0)
 #pragma unroll
-    for (int l = 0; l < NP; ++l) {
-      const double x = t[l][0].value(), y = t[l][1].value();
-      proj[((size_t)b * natoms + I) * NP + l] = make_float2((float)(x * scale), (float)(y * scale));
-    }
+    for (int l = 0; l < NP; ++l)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) red[warp][l][h] = make_float2(t[l][h].s, t[l][h].c);
+  __syncthreads();
+  if (sl == 0 && b < n && lane < NP) {
+    SumPair r[2];
+    for (int w = 0; w < S; ++w)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) r[h].add(red[warp + w][lane][h].x, red[warp + w][lane][h].y);
+    const double x = r[0].value(), y = r[1].value();
+    proj[((size_t)b * natoms + I) * NP + lane] = make_float2((float)(x * scale), (float)(y * scale));
+  }
 }
 
 // Setup: projector grid functions -> sphere coefficients (FP64), then rounded to complex64.
@@ -1581,12 +1605,14 @@ class FusedImpl final : public FusedOps {
       pois[m2] = (float)(4.0 * M_PI / (kf * kf * (double)m2)) * (float)(1.0 / (double)N3);
     pois_ = upload(pois);
     if (nprojtot_ > 0) {
-      B_ = alloc<float2>((size_t)nprojtot_ * g.nG);
-      Bimg_ = arena_.alloc(tc_overlap_image_bytes(nprojtot_, g.nG));
       pf_ = alloc<float2>((size_t)nprojtot_ * ns_);
-      part_elems_ = std::max<size_t>(tc_overlap_part_elems(nprojtot_, ns_, true), 4096);
-      part_ = alloc<double2>(part_elems_);
-      build_projector_block();
+      if (!real_space_projections()) {
+        B_ = alloc<float2>((size_t)nprojtot_ * g.nG);
+        Bimg_ = arena_.alloc(tc_overlap_image_bytes(nprojtot_, g.nG));
+        part_elems_ = std::max<size_t>(tc_overlap_part_elems(nprojtot_, ns_, true), 4096);
+        part_ = alloc<double2>(part_elems_);
+        build_projector_block();
+      }
     }
     nch_max_ = std::max((ns_ + density_chunk(0) - 1) / density_chunk(0), (ns_ + density_chunk(1) - 1) / density_chunk(1));
     dpartial_ = alloc<float>((size_t)nch_max_ * N3);
@@ -1614,19 +1640,53 @@ class FusedImpl final : public FusedOps {
     });
   }
 
-  // The per-cell part of an H application: the projections p_Il = sum_G conj(b_Il(G)) c_G of the
-  // block (tensor cores), scaled for the plane kernel, and the projector values they give.
+  // Grids whose projections are sums over the spheres' grid points, p_Il = dV sum_r beta_Il(r) psi(r), instead of
+  // products with the projector block on the tensor cores.  These grids are used at the accuracy of such
+  // sums, H psi within 4.4e-8 to 4.8e-8 of 64 bits; split-BF16 products keep 16 bits of their operands and round
+  // their FP32 accumulators towards zero, which took it to 4.7e-8 to 14e-8.  The sums need psi on the grid before
+  // the plane kernel adds their result there, an inverse plane pass more: H psi of 37 states on 72^3 (23 atoms)
+  // 177 -> 204 us, of 128 on 108^3 (64 atoms) 1.87 -> 2.27 ms, but of 24 on 108^3 at 10/24 bohr (40 atoms) 0.71
+  // -> 0.54 ms.  FP32 products on the CUDA cores were as accurate and took 220 us, 2.6 ms and 0.91 ms.  Without a
+  // projector block and its split image a handle of the first of these cells takes 100 MB less.
+  static constexpr bool real_space_projections(int N) { return N == 54 || N == 72 || N == 108; }
+  bool real_space_projections() const { return real_space_projections(N_); }
+  // The per-cell part of an H application: the projections p_Il of the block, scaled for the plane
+  // kernel, and the projector values they give (real_space_projections: of the block whose columns colbuf1_
+  // holds; psi is not read).
   // `values`: the plane kernel that follows reads them (the team kernel; the CTA-wide one sums the
   // projectors itself).
   void pre_h(const float2* psi, int n, bool values, cudaStream_t s) {
     if (nprojtot_ > 0) {
-      {
+      if (real_space_projections()) {
+        ProfScope ps(prof_, "project", s);
+        project_columns(n, s);
+      } else {
         ProfScope ps(prof_, "proj_gemm", s);
         tc_overlap(B_, g_.nG, psi, g_.nG, nprojtot_, n, g_.nG, part_, part_elems_, nullptr, err_, s, nullptr, Bimg_, pf_,
                    (float)(g_.D * std::sqrt(g_.omega)));
       }
       if (values) nl_values(n, s);
     }
+  }
+  // pf_ of the n states in colbuf1_ (nlval_ holds their covered points meanwhile)
+  void project_columns(int n, cudaStream_t s) {
+    if (npts_ == 0 || !nlval_) return;                                // no covered point reads pf_
+    dispatch([&](auto tag) {
+      constexpr int N = decltype(tag)::value;
+      if constexpr (real_space_projections(N)) {
+        static_assert(TPlan<N>::ok, "the kernel has team transforms");
+        const size_t smem = force_smem<N, false>();
+        static bool attr = false;
+        if (!attr) {
+          KS_CUDA(cudaFuncSetAttribute(k_plane_force_team<N, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem));
+          attr = true;
+        }
+        launch_chain(points(n), k_plane_force_team<N, false, false>, dim3(N, n), dim3(TCfg<N>::PT), smem, s, colbuf1_, ncols_,
+                     t_.col_xy, g_.xr, rowym_, n, 1, nullptr, 0, 0.f, nullptr, nullptr, team_nl(), nlval_, t_.tw);
+      }
+    });
+    project(n, (float)(g_.D * g_.dV), pf_, s);
   }
   void nl_values(int n, cudaStream_t s) {
     if (npts_ == 0 || !nlval_) return;
@@ -1652,7 +1712,7 @@ class FusedImpl final : public FusedOps {
       FusedImpl* f = static_cast<FusedImpl*>(it.ops);
       if (!same_geometry(f0, f)) fail(KS_ERR_ARG, "packed H application: the members' grids differ");
       if (it.n < 1 || it.n > f->ns_) fail(KS_ERR_ARG, "packed H application: member with %d states", it.n);
-      f->pre_h(it.psi, it.n, f->group_values(it.n), s);
+      if (!f->real_space_projections()) f->pre_h(it.psi, it.n, f->group_values(it.n), s);
     }
     f0->dispatch([&](auto tag) { group_launch<decltype(tag)::value>(items, s); });
   }
@@ -1716,6 +1776,11 @@ class FusedImpl final : public FusedOps {
           launch_chain(f0->points(s0), k_zinv_group<N>, dim3(ncb, z0), dim3(FCfg<N>::ZT), zsmem<N>(), s, gd, f0->g_.nG, f0->t_.col_off,
                        f0->t_.col_half, f0->ncols_, f0->t_.tw);
         }
+        if (f0->real_space_projections())
+          for (size_t k = a; k < std::min(items.size(), a + GMAX); ++k) {
+            FusedImpl* f = static_cast<FusedImpl*>(items[k].ops);
+            f->pre_h(items[k].psi, items[k].n, f->group_values(items[k].n), s);
+          }
         {
           ProfScope ps(f0->prof_, "plane", s);
           if constexpr (PlaneForm<N>::single_per_member) {
@@ -1742,8 +1807,9 @@ class FusedImpl final : public FusedOps {
 
   void apply_h(const float2* psi, float2* hpsi, int n, cudaStream_t s, const TaylorEpi* te) override {
     const bool decided = !team_density() || tune_peek(tune_key("plane", n)) == 1;
-    pre_h(psi, n, !decided, s);
+    if (!real_space_projections()) pre_h(psi, n, !decided, s);
     zinv(psi, n, s);
+    if (real_space_projections()) pre_h(psi, n, !decided, s);
     {
       ProfScope ps(prof_, "plane", s);
       dispatch([&](auto tag) {
@@ -1774,8 +1840,7 @@ class FusedImpl final : public FusedOps {
     dispatch([&](auto tag) {
       constexpr int N = decltype(tag)::value;
       if constexpr (TPlan<N>::ok) {
-        const size_t tables = (size_t)N * TCfg<N>::NW * 4 + 2 * (size_t)N * sizeof(int);
-        const size_t smem0 = plane_smem<N>() + tables, smem1 = smem0 + (size_t)N * N * sizeof(float);
+        const size_t smem0 = force_smem<N, false>(), smem1 = force_smem<N, true>();
         static bool attr = false;
         if (!attr) {
           KS_CUDA(cudaFuncSetAttribute(k_plane_force_team<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1802,15 +1867,22 @@ class FusedImpl final : public FusedOps {
     });
   }
 
+  template <int N, bool GRAD> static size_t force_smem() {
+    return plane_smem<N>() + (size_t)N * TCfg<N>::NW * 4 + 2 * (size_t)N * sizeof(int) +
+           (GRAD ? (size_t)N * N * sizeof(float) : 0);
+  }
   // The projections of the covered-point values in nlval_ (n states).
   void project(int n, float pscale, float2* out, cudaStream_t s) {
-    const dim3 grid(g_.natoms, (n + PJW - 1) / PJW);
-    if (g_.nproj == 4)
-      launch_chain(points(n), k_project_points<4>, grid, dim3(32 * PJW), 0, s, nlval_, npts_, t_.sph_off, sph_slot_, sph_bz_,
-                   g_.natoms, n, pscale, out);
+    // four warps per atom and state until one each fills the GPU (48 an SM)
+    if ((size_t)g_.natoms * n < 152 * 48)
+      g_.nproj == 4 ? launch_project<4, 4>(n, pscale, out, s) : launch_project<1, 4>(n, pscale, out, s);
     else
-      launch_chain(points(n), k_project_points<1>, grid, dim3(32 * PJW), 0, s, nlval_, npts_, t_.sph_off, sph_slot_, sph_bz_,
-                   g_.natoms, n, pscale, out);
+      g_.nproj == 4 ? launch_project<4, 1>(n, pscale, out, s) : launch_project<1, 1>(n, pscale, out, s);
+  }
+  template <int NP, int S> void launch_project(int n, float pscale, float2* out, cudaStream_t s) {
+    constexpr int states = PJW / S;                                  // per CTA
+    launch_chain(points(n), k_project_points<NP, S>, dim3(g_.natoms, (n + states - 1) / states), dim3(32 * PJW), 0, s, nlval_,
+                 npts_, t_.sph_off, sph_slot_, sph_bz_, g_.natoms, n, pscale, out);
   }
 
   void prepare_atoms() override {
@@ -1832,7 +1904,7 @@ class FusedImpl final : public FusedOps {
     arena_.release(sph_slot_);
     arena_.release(sph_bz_);
     upload_plane_lists();
-    if (nprojtot_ > 0) build_projector_block();
+    if (nprojtot_ > 0 && !real_space_projections()) build_projector_block();
     KS_CUDA(cudaStreamSynchronize(setup_));                           // the new lists have landed
   }
 
@@ -2241,7 +2313,7 @@ class FusedImpl final : public FusedOps {
   float2* colbuf2_ = nullptr;
   float* vplane_ = nullptr;
   const float* pois_ = nullptr;      // Poisson factor by |m|^2
-  float2* B_ = nullptr;
+  float2* B_ = nullptr;              // projector block (not with real_space_projections)
   void* Bimg_ = nullptr;             // B_ split into bf16 hi/lo operand tiles
   float2* pf_ = nullptr;
   const int* rowym_ = nullptr;       // [2 xr + 1] column range of each band row

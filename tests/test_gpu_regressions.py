@@ -120,3 +120,40 @@ def test_fp64_routes(ks, meas, N, L, ns):
     g.density(n.data_ptr())
     meas("N=%d, %d states: density" % (N, ns), rel(n.cpu().numpy(), ko.density(ref, c)), 1e-12)
     g.close()
+
+
+@pytest.mark.parametrize("N,h,natoms,ns", [(54, 0.3125, 1, 1), (54, 0.3125, 33, 5), (72, 0.375, 40, 3), (108, 10.0 / 24, 17, 2)])
+def test_projections_of_fp32_accuracy(ks, meas, N, h, natoms, ns):
+    """H psi of smooth states (large projections beside the kinetic part) on the grids of 54, 72 and 108 points
+    at the accuracy of sums over the grid: a coefficient's last two roundings, 2^-24 / sqrt(3) rms each, are
+    4.9e-8, the transforms and projections come to less: 6.5e-8.  (Split-BF16 projections: 7e-8 to 1.4e-7.)"""
+    cell = inputs.small_cell(N * h, N, natoms, ns, 76, depth=-3.0)
+    ref = ko.Cell(cell)
+    t = 0.5 + np.arange(ns)[:, None]
+    c = (inputs.random_coeffs(76, ns, ref.nG) * np.exp(-0.25 * ref.g2[None, :] / t)).astype(np.complex64)
+    g = ks.Grid(cell, prec="bf16x3")
+    psi = torch.from_numpy(c).to("cuda")
+    out = torch.empty_like(psi)
+    g.apply_h(psi.data_ptr(), out.data_ptr(), ns)
+    torch.cuda.synchronize()
+    meas("N=%d, %d atoms" % (N, natoms), rel(out.cpu().numpy().astype(complex), ko.apply_h(ref, c.astype(complex))), 6.5e-8)
+    g.close()
+
+
+@pytest.mark.parametrize("natoms,nproj,ns", [(1, 1, 1), (16, 4, 2), (5, 4, 3), (17, 4, 9), (73, 1, 99), (73, 1, 100)])
+def test_projection_groups(ks, meas, natoms, nproj, ns):
+    """Projections summed on the grid, either side of the lines between two and eight states a CTA (four and one
+    warps per atom and state), full and ragged groups, states of different sizes; bound of the fused grids'
+    H psi."""
+    cell = inputs.small_cell(16.875, 54, natoms, ns, 77, depth=-3.0, nproj=nproj)
+    ref = ko.Cell(cell)
+    c = inputs.random_coeffs(77, ns, ref.nG) * np.logspace(-3, 3, ns)[:, None]
+    g = ks.Grid(cell, prec="bf16x3")
+    buf = torch.zeros((ns + 1, ref.nG), dtype=torch.complex64, device="cuda")
+    buf[1:] = torch.from_numpy(c).to("cuda", torch.complex64)
+    out = torch.full_like(buf, float("nan"))
+    g.apply_h(buf[1:].data_ptr(), out[1:].data_ptr(), ns)
+    torch.cuda.synchronize()
+    got, expect = out[1:].cpu().numpy().astype(complex), ko.apply_h(ref, c)
+    meas("%d x %d" % (natoms * nproj, ns), max(rel(got[k], expect[k]) for k in range(ns)), 2e-5)
+    g.close()
