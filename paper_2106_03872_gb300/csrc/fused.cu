@@ -2117,59 +2117,66 @@ class FusedImpl final : public FusedOps {
   }
   void plane_lists_host() {
     const HostGeometry& g = g_;
-    std::vector<int>& pt_off = h_pt_off_;
-    std::vector<int>& pt_xy = h_pt_xy_;
-    std::vector<int>& ent_off = h_ent_off_;
-    std::vector<int>& ent_proj = h_ent_proj_;
-    std::vector<float>& ent_beta = h_ent_beta_;
-    // each atom's sphere points in the order of the covered points (so that a warp reads runs of them):
-    // their covered points and beta values (forces)
-    std::vector<int> next(g.sph_off.begin(), g.sph_off.end());
-    h_sph_slot_.resize(g.sph_idx.size());
-    h_sph_bz_.resize(g.sph_idx.size() * g.nproj);
-    pt_off.assign(N_ + 1, 0);
-    pt_xy.clear();
-    ent_off.assign(1, 0);
-    ent_proj.clear();
-    ent_beta.clear();
-    std::vector<std::vector<int>> byz(N_);
-    for (size_t c = 0; c < g.cov_idx.size(); ++c) byz[g.cov_idx[c] % N_].push_back((int)c);
-    // within a plane, points in (y, x) order, with the offset of each y-line (the team plane
-    // kernel finds a point's value by its line's offset and a bitmap of x)
-    std::vector<int>& line_off = h_line_off_;
-    line_off.assign((size_t)N_ * (N_ + 1), 0);
-    nl_cap_ = 0;
-    for (int z = 0; z < N_; ++z) {
-      std::vector<int>& v = byz[z];
-      std::stable_sort(v.begin(), v.end(), [&](int a, int b) {
-        const int xa = g.cov_idx[a] / N_, xb = g.cov_idx[b] / N_;       // jx*N + jy
-        return (xa % N_) != (xb % N_) ? (xa % N_) < (xb % N_) : (xa / N_) < (xb / N_);
-      });
-      int* lo = line_off.data() + (size_t)z * (N_ + 1);
-      for (int c : v) lo[(g.cov_idx[c] / N_) % N_ + 1]++;
-      for (int y = 0; y < N_; ++y) lo[y + 1] += lo[y];
-      nl_cap_ = std::max(nl_cap_, (int)v.size());
-      for (int c : v) {
-        pt_xy.push_back(g.cov_idx[c] / N_);
-        for (int e = g.cov_off[c]; e < g.cov_off[c + 1]; ++e) {
-          const int p = g.cov_ent[e];
-          const size_t at = (size_t)next[g.sph_atom[p]]++;
-          h_sph_slot_[at] = (int)pt_xy.size() - 1;
-          ent_proj.push_back(g.sph_atom[p] * g.nproj);
-          for (int l = 0; l < g.nproj; ++l) {
-            const float b = (float)g.sph_beta[(size_t)p * g.nproj + l];
-            ent_beta.push_back(b);
-            h_sph_bz_[at * g.nproj + l] = b;
-          }
-        }
-        ent_off.push_back((int)ent_proj.size());
-      }
-      pt_off[z + 1] = (int)pt_xy.size();
+    const int N = N_, np = g.nproj;
+    const size_t nc = g.cov_idx.size(), ne = g.cov_ent.size();
+    // planes in order, within a plane points in (y, x) order, with the offset of each y-line (the team plane
+    // kernel finds a point's value by its line's offset and a bitmap of x).  The geometry's points are in
+    // (x, y, z) order, so counting them by (z, y) leaves x increasing within a line (a sort by comparisons was
+    // most of a handle's creation: 40 atoms on 54^3 8.8 ms, counted 4.7).
+    std::vector<int> end((size_t)N * N + 1, 0), order(nc);            // by z N + y
+    for (size_t c = 0; c < nc; ++c) {
+      const int xy = g.cov_idx[c] / N, z = g.cov_idx[c] - xy * N;
+      ++end[(size_t)z * N + xy % N + 1];
     }
+    for (size_t k = 0; k < (size_t)N * N; ++k) end[k + 1] += end[k];
+    for (size_t c = 0; c < nc; ++c) {
+      const int xy = g.cov_idx[c] / N, z = g.cov_idx[c] - xy * N;
+      order[end[(size_t)z * N + xy % N]++] = (int)c;                  // end[k]: the line's start, then its end
+    }
+    h_pt_off_.assign(N + 1, 0);
+    h_line_off_.assign((size_t)N * (N + 1), 0);
+    nl_cap_ = 0;
+    for (int z = 0; z < N; ++z) {
+      h_pt_off_[z + 1] = end[(size_t)z * N + N - 1];
+      for (int y = 0; y < N; ++y) h_line_off_[(size_t)z * (N + 1) + y + 1] = end[(size_t)z * N + y] - h_pt_off_[z];
+      nl_cap_ = std::max(nl_cap_, h_pt_off_[z + 1] - h_pt_off_[z]);
+    }
+    h_pt_xy_.resize(nc);
+    h_ent_off_.resize(nc + 1);
+    h_ent_proj_.resize(ne);
+    h_ent_beta_.resize(ne * np);
+    // on the grids with team transforms each atom's sphere points in the order of the covered points (so that a
+    // warp reads runs of them): their covered points and beta values (project)
+    const bool spheres = team_density();
+    std::vector<int> next;
+    if (spheres) {
+      next.assign(g.sph_off.begin(), g.sph_off.end());
+      h_sph_slot_.resize(ne);
+      h_sph_bz_.resize(ne * np);
+    }
+    int at = 0;
+    for (size_t i = 0; i < nc; ++i) {
+      const int c = order[i];
+      h_pt_xy_[i] = g.cov_idx[c] / N;
+      h_ent_off_[i] = at;
+      for (int e = g.cov_off[c]; e < g.cov_off[c + 1]; ++e, ++at) {
+        const int p = g.cov_ent[e], atom = g.sph_atom[p];
+        h_ent_proj_[at] = atom * np;
+        for (int l = 0; l < np; ++l) h_ent_beta_[(size_t)at * np + l] = (float)g.sph_beta[(size_t)p * np + l];
+        if (spheres) {
+          const size_t q = (size_t)next[atom]++;
+          h_sph_slot_[q] = (int)i;
+          for (int l = 0; l < np; ++l) h_sph_bz_[q * np + l] = h_ent_beta_[(size_t)at * np + l];
+        }
+      }
+    }
+    h_ent_off_[nc] = at;
   }
   void upload_plane_lists() {
-    sph_slot_ = upload(h_sph_slot_);
-    sph_bz_ = upload(h_sph_bz_);
+    if (team_density()) {
+      sph_slot_ = upload(h_sph_slot_);
+      sph_bz_ = upload(h_sph_bz_);
+    }
     nl_.pt_off = upload(h_pt_off_);
     nl_.pt_xy = upload(h_pt_xy_);
     nl_.ent_off = upload(h_ent_off_);
