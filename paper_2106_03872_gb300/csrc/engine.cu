@@ -1030,8 +1030,8 @@ template <typename T> class Engine final : public EngineBase {
   }
 
   // ------------------------------------------------------------------------------------------
-  // Forces from the orbital gradients (Eq. 11, with the sign of -dE/dR_I), one state at a time
-  // through two full-grid buffers: psi(r) and d_alpha psi(r) from i G_alpha c.
+  // Forces from the orbital gradients (Eq. 11, with the sign of -dE/dR_I): psi(r) of a chunk of states on the
+  // grid and d_alpha psi(r) from i G_alpha c, on the grid too or by planes (FusedOps::force_chunk).
   //   local:    F_Ia -= dV sum_j v_I(r_j) g_a(r_j),  g_a = sum_k f_k 2 Re(conj(d_a psi_k) psi_k)
   //   nonlocal: F_Ia -= sum_k f_k sum_l 2 D Re(conj(q_Il,a) p_Il)
   // v_I is the atom's 27-image Gaussian, separable per axis.
@@ -1473,20 +1473,25 @@ template <typename T> class Engine final : public EngineBase {
     KS_CUDA(cudaMemcpy(v_host, vloc64_, (size_t)g_.N * g_.N * g_.N * sizeof(double), cudaMemcpyDeviceToHost));
   }
 
-  // Work buffers of the force evaluation (allocated on first use): full grids for a chunk of
-  // fb_ states (at most 2 GB for the two), their projections, the gradient densities.
+  // Work buffers of the force evaluation (allocated on first use): psi's full grids of a chunk of fb_ states
+  // and, off the grids with force_chunks, its gradient's (at most 2 GB), their projections, the gradient
+  // densities.  A call that ran out of memory on the way continues where it stopped.
   void force_buffers() {
-    if (fw_) return;
+    if (flocp_) return;                                              // the last one
     const int N = g_.N, na = g_.natoms, np = g_.nproj;
     const size_t N3 = (size_t)N * N * N;
-    fb_ = (int)std::max<size_t>(1, std::min<size_t>((size_t)ns_, (size_t(2048) << 20) / (2 * N3 * sizeof(C))));
-    fpsi_ = alloc<C>((size_t)fb_ * N3);
-    fw_ = alloc<C>((size_t)fb_ * N3);
-    fg_ = alloc<T>(3 * N3);
-    fp_ = alloc<C>((size_t)fb_ * na * np);
-    fq_ = alloc<C>((size_t)fb_ * na * np);
-    fnl_ = alloc<double>(3 * (size_t)na);
-    floc_ = alloc<double>(3 * (size_t)na);
+    const bool gradient = !(fused_ && fused_->force_chunks());
+    if (!fpsi_) {
+      fb_ = (int)std::max<size_t>(
+          1, std::min<size_t>((size_t)ns_, (size_t(2048) << 20) / ((gradient ? 2 : 1) * N3 * sizeof(C))));
+      fpsi_ = alloc<C>((size_t)fb_ * N3);
+    }
+    if (gradient && !fw_) fw_ = alloc<C>((size_t)fb_ * N3);
+    if (!fg_) fg_ = alloc<T>(3 * N3);
+    if (!fp_) fp_ = alloc<C>((size_t)fb_ * na * np);
+    if (!fq_) fq_ = alloc<C>((size_t)fb_ * na * np);
+    if (!fnl_) fnl_ = alloc<double>(3 * (size_t)na);
+    if (!floc_) floc_ = alloc<double>(3 * (size_t)na);
     flocp_ = alloc<double>(3 * (size_t)na * LOCAL_FORCE_SPLIT);
   }
 
@@ -1656,8 +1661,8 @@ template <typename T> class Engine final : public EngineBase {
   double* resid_dev_ = nullptr;     // SCF residual
   double* dip_partials_ = nullptr;  // dipole block partials
   double2* trr_ = nullptr;          // per-state residual kinetic sums of the preconditioned update
-  C* fw_ = nullptr;                 // forces: state and gradient grids of a chunk, accumulators,
-  C* fpsi_ = nullptr;               // projections (on first use)
+  C* fpsi_ = nullptr;               // forces (on first use): state grids of a chunk,
+  C* fw_ = nullptr;                 // gradient grids (off the grids with force_chunks), accumulators, projections
   int fb_ = 1;
   T* fg_ = nullptr;
   C *fp_ = nullptr, *fq_ = nullptr;

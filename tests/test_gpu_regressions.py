@@ -157,3 +157,18 @@ def test_projection_groups(ks, meas, natoms, nproj, ns):
     got, expect = out[1:].cpu().numpy().astype(complex), ko.apply_h(ref, c)
     meas("%d x %d" % (natoms * nproj, ns), max(rel(got[k], expect[k]) for k in range(ns)), 2e-5)
     g.close()
+
+
+@pytest.mark.parametrize("N,L,grids", [(64, 20.0, 1), (54, 16.875, 1), (36, 11.25, 2)])
+def test_force_buffers(ks, N, L, grids):
+    """The first force call allocates the states' full grids once, and the gradients' beside them only on grids
+    without team transforms: that many grids of the block, plus less than half a one for the rest."""
+    ns = 24
+    cell = inputs.small_cell(L, N, 2, ns, 78)
+    g = ks.Grid(cell, prec="bf16x3")
+    g.set_states(inputs.random_coeffs(78, ns, g.nG))
+    before = g.device_bytes()
+    g.forces()
+    grown, block = g.device_bytes() - before, 8 * ns * N ** 3
+    assert grids * block <= grown <= (grids + 0.5) * block
+    g.close()
