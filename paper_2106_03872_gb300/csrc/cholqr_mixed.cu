@@ -281,15 +281,13 @@ size_t cholesky_mixed_workspace(int n) { return (size_t)3 * n * n; }
 void cholesky_inverse_mixed(const double2* S, double2* M, int n, double tol, double2* work, int* status,
                             cudaStream_t s, float2* M32, bool refine) {
   if (n > C32_MAXN) fail(KS_ERR_ARG, "cholesky_inverse_mixed: n=%d > %d", n, C32_MAXN);
-  if (n <= SMALL_SUBSPACE) {
-    cholesky_small(S, M, n, tol, work, status, s, M32, refine);
-    return;
-  }
   double2* M1 = work;
   double2* T = work + (size_t)n * n;
   double2* S2 = work + (size_t)2 * n * n;
   auto factor = [&](int conj_out, double2* out, float2* out32) {
-    if (n <= 32)
+    if (n <= SMALL_SUBSPACE)
+      chol32_small(S, n, tol, conj_out, status, out, out32, s);
+    else if (n <= 32)
       launch_chol32<1, 256, 32>(S, n, tol, conj_out, status, out, out32, s);
     else if (n <= 64)
       launch_chol32<1, 512, 64>(S, n, tol, conj_out, status, out, out32, s);

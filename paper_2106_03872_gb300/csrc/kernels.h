@@ -202,8 +202,9 @@ void rr_step_mixed(const float2* Hraw, const float2* M, double alpha, int n, flo
 // Blocks of at most SMALL_SUBSPACE states take one-CTA kernels instead (subspace_small.cu), through
 // cholesky_inverse_mixed, eigh_mixed and rr_step_mixed.
 constexpr int SMALL_SUBSPACE = 16;
-void cholesky_small(const double2* S, double2* M, int n, double tol, double2* work, int* status, cudaStream_t s,
-                    float2* M32, bool refine);
+// Out = L^{-1} of S = L L^H in FP32 (conj(L^{-1}) when conj_out), and a complex64 copy to Out32 when given.
+void chol32_small(const double2* S, int n, double tol, int conj_out, int* status, double2* Out, float2* Out32,
+                  cudaStream_t s);
 void eigh_small(const double2* A, double2* V, int n, cudaStream_t s);
 void rr_step_small(const float2* Hraw, const float2* M, double alpha, int n, float2* Mcat, float2* Aout,
                    float2* Vout, int* perm, cudaStream_t s);

@@ -1,10 +1,9 @@
-// Subspace kernels for blocks of at most 16 states on the mixed path: the whole Rayleigh-Ritz step, and
-// the whole Cholesky factor, in one CTA each.  At these sizes the launches of the spread-out solver
+// Subspace kernels for blocks of at most 16 states on the mixed path: the eigensolver, the whole
+// Rayleigh-Ritz step and the Cholesky factor, in one CTA each.  At these sizes the launches of the spread-out solver
 // (eigh.cu) cost more than its parallelism saves: a Rayleigh-Ritz step of 8 states takes 36 us here and
-// 89 us there (at 16 states the eigensolver takes 92 and 81 us, about level).  Both round differently, and blocks this
-// small meet exactly degenerate levels most often (closed shells of free electrons).
+// 89 us there (at 16 states the eigensolver takes 92 and 81 us, about level).
 //
-// The eigensolver, FP32, matrix in shared memory:
+// The eigensolver, FP32, matrix in shared memory, a warp per row:
 //   1. Householder reduction to a real symmetric tridiagonal T, the update of step k-1 applied in the
 //      same pass over the trailing block as the product A v_k of step k (one barrier a step; every warp
 //      forms v_k itself from column k).
@@ -15,24 +14,20 @@
 //   4. Back-transformation, 8 threads per column.
 // The Rayleigh-Ritz step adds H_sub = conj(M) H_raw M^T before and the step matrix after, as
 // rr_step_mixed does (eigh.cu).
-#include <type_traits>
-
 #include "kernels.h"
 
 namespace ks {
 
 namespace {
 
-constexpr int EH_MAXN = 64;                                          // array bounds: rows 4 warp + u
-constexpr int EH_THREADS = 512;                                      // a warp per row
+constexpr int EH_MAXN = SMALL_SUBSPACE;
+constexpr int EH_THREADS = 512;                                      // a warp per row of the matrix
 constexpr int EH_WARPS = EH_THREADS / 32;
-static_assert(SMALL_SUBSPACE <= EH_WARPS, "a warp per row of the matrix");
+static_assert(EH_MAXN <= EH_WARPS && EH_MAXN <= 32, "a warp per row, a lane per column");
 constexpr unsigned FULL = 0xffffffffu;
-// shared memory: the matrix [EH_MAXN][EH_MAXN + 1], then the packed reflectors, whose region also
-// stages operand rows
+// shared memory: the matrix [n][n + 1], then packed reflectors or three staged n x n operands
 constexpr int EH_AREG = EH_MAXN * (EH_MAXN + 1);
-constexpr int EH_RREG = 64 * EH_MAXN;
-constexpr size_t EH_SMEM = (size_t)(EH_AREG + EH_RREG) * sizeof(float2);
+constexpr int EH_RREG = 3 * EH_MAXN * EH_MAXN;
 constexpr int SC_THREADS = 256;
 
 __device__ __forceinline__ float2 cm(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
@@ -77,166 +72,56 @@ __device__ __forceinline__ int sturm_count(const float* d, const float* e2, int 
   return c;
 }
 
-// Phase 0 of the Rayleigh-Ritz variant: A = conj(M) H_raw M^T (FP32), Hermitian part, in the
-// [n][ld] matrix region; R (EH_RREG float2) stages operand chunks.  M is lower triangular.
-// Thread (warp w, lane): rows 4w + u (u < 4), columns lane + 32v (v < 4), 16 accumulators; each
-// element's sum runs over k in ascending order (terms of M's zero triangle add exact zeros).
-constexpr int RR_KC = 16, RR_MLD = EH_MAXN + 1;
-constexpr int RR_V = EH_MAXN / 32;                            // column slots of a lane
+// A = conj(M) H_raw M^T (FP32), its Hermitian part, in the [n][n + 1] matrix region, and to Aout.  R stages
+// H_raw, M (lower triangular, zeros stored) and H_raw M^T; each sum runs over k in ascending order.
 __device__ __forceinline__ void subspace_matrix_small(const float2* __restrict__ Hraw, const float2* __restrict__ M, int n,
                                                 float2* A, float2* R, float2* __restrict__ Aout) {
-  const int ld = n + 1;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const float2 zero = make_float2(0.f, 0.f);
-  float2 acc[4][RR_V];
-  // T = H_raw M^T: T_ij = sum_k H_ik M_jk
-  float2* Hs = R;                                                    // [EH_MAXN][RR_KC]: H_i,k0+kk
-  float2* Mt = R + EH_MAXN * RR_KC;                                  // [RR_KC][RR_MLD]: M_j,k0+kk
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int v = 0; v < RR_V; ++v) acc[u][v] = zero;
-  for (int k0 = 0; k0 < n; k0 += RR_KC) {
-    __syncthreads();
-    for (int e = t; e < EH_MAXN * RR_KC; e += EH_THREADS) {
-      const int i = e / RR_KC, k = k0 + e % RR_KC;
-      Hs[e] = (i < n && k < n) ? Hraw[i * n + k] : zero;
-    }
-    for (int e = t; e < EH_MAXN * RR_KC; e += EH_THREADS) {
-      const int j = e / RR_KC, kk = e % RR_KC, k = k0 + kk;
-      Mt[kk * RR_MLD + j] = (j < n && k < n) ? M[j * n + k] : zero;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < RR_KC; ++kk) {
-      float2 hv[4], mv[RR_V];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) hv[u] = Hs[(4 * warp + u) * RR_KC + kk];
-#pragma unroll
-      for (int v = 0; v < RR_V; ++v) mv[v] = Mt[kk * RR_MLD + lane + 32 * v];
-#pragma unroll
-      for (int v = 0; v < RR_V; ++v)
-        if (32 * v + 31 >= k0)                                       // M_jk = 0 for every j of group v
-#pragma unroll
-          for (int u = 0; u < 4; ++u) acc[u][v] = cfma(acc[u][v], hv[u], mv[v]);
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int v = 0; v < RR_V; ++v) {
-      const int i = 4 * warp + u, j = lane + 32 * v;
-      if (i < n && j < n) A[i * ld + j] = acc[u][v];
-    }
-  // A = conj(M) T: A_ij = sum_{k <= i} conj(M_ik) T_kj, all rows at once (written after the sums)
-  float2* Ms = R;                                                    // [EH_MAXN][RR_KC]: M_i,k0+kk
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int v = 0; v < RR_V; ++v) acc[u][v] = zero;
-  for (int k0 = 0; k0 < n; k0 += RR_KC) {
-    __syncthreads();
-    for (int e = t; e < EH_MAXN * RR_KC; e += EH_THREADS) {
-      const int i = e / RR_KC, k = k0 + e % RR_KC;
-      Ms[e] = (i < n && k < n) ? M[i * n + k] : zero;
-    }
-    __syncthreads();
-    const int kend = min(RR_KC, n - k0);
-    if (4 * warp + 3 >= k0) {                                        // M_ik = 0 for every row i of the warp
-      for (int kk = 0; kk < kend; ++kk) {
-        const int k = k0 + kk;
-        float2 ma[4], tv[RR_V];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) ma[u] = Ms[(4 * warp + u) * RR_KC + kk];
-#pragma unroll
-        for (int v = 0; v < RR_V; ++v) {
-          const int j = lane + 32 * v;
-          tv[v] = j < n ? A[k * ld + j] : zero;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-          for (int v = 0; v < RR_V; ++v) acc[u][v] = cfmac(acc[u][v], ma[u], tv[v]);
-      }
-    }
+  const int ld = n + 1, t = threadIdx.x, i = t / n, j = t - i * n;
+  const bool in = t < n * n;
+  float2 *Hs = R, *Ms = Hs + EH_MAXN * EH_MAXN, *Ts = Ms + EH_MAXN * EH_MAXN;
+  if (in) {
+    Hs[t] = Hraw[t];
+    Ms[t] = M[t];
   }
   __syncthreads();
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int v = 0; v < RR_V; ++v) {
-      const int i = 4 * warp + u, j = lane + 32 * v;
-      if (i < n && j < n) A[i * ld + j] = acc[u][v];
-    }
+  float2 acc = make_float2(0.f, 0.f);
+  if (in) {
+    for (int k = 0; k < n; ++k) acc = cfma(acc, Hs[i * n + k], Ms[j * n + k]);
+    Ts[t] = acc;
+  }
   __syncthreads();
-  // Hermitian part (one thread per pair), real diagonal
-  for (int i = warp; i < n; i += EH_WARPS)
-    for (int j = lane; j <= i; j += 32) {
-      const float2 a = A[i * ld + j], b = A[j * ld + i];
-      const float2 h = make_float2(0.5f * (a.x + b.x), i == j ? 0.f : 0.5f * (a.y - b.y));
-      A[i * ld + j] = h;
-      A[j * ld + i] = make_float2(h.x, -h.y);
-    }
+  acc = make_float2(0.f, 0.f);
+  if (in) {
+    for (int k = 0; k < n; ++k) acc = cfmac(acc, Ms[i * n + k], Ts[k * n + j]);
+    A[i * ld + j] = acc;
+  }
   __syncthreads();
-  for (int i = warp; i < n; i += EH_WARPS)
-    for (int j = lane; j < n; j += 32) Aout[i * n + j] = A[i * ld + j];
+  float2 h = acc;
+  if (in) {                                                          // Hermitian part, real diagonal
+    const float2 b = A[j * ld + i];
+    h = make_float2(0.5f * (acc.x + b.x), i == j ? 0.f : 0.5f * (acc.y - b.y));
+  }
+  __syncthreads();
+  if (in) {
+    A[i * ld + j] = h;
+    Aout[t] = h;
+  }
 }
 
-// Phase 5 of the Rayleigh-Ritz variant: with V staged in the matrix region (V_kr at k ld + r),
-// C = Vt M (C_rj = sum_{k >= j} V_kr M_kj, k ascending) and Mcat row rank(r) =
-// [(1 + alpha lam_r) C_r | -alpha C_r].  Thread: rows r = 4w + u, columns lane + 32v.
+// With the vectors V in the matrix region (V_kr at k ld + r): C = Vt M (C_rj = sum_k V_kr M_kj, k ascending) and
+// Mcat row rank(r) = [(1 + alpha lam_r) C_r | -alpha C_r].
 __device__ __forceinline__ void step_matrix_small(const float2* Vs, const float2* __restrict__ M, int n, const float* lam,
                                             const int* rank, float alpha, float2* R, float2* __restrict__ Mcat) {
-  const int ld = n + 1;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const float2 zero = make_float2(0.f, 0.f);
-  float2* Ms = R;                                                    // [RR_KC][EH_MAXN]: M rows k0..
-  float2 acc[4][RR_V];
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int v = 0; v < RR_V; ++v) acc[u][v] = zero;
-  for (int k0 = 0; k0 < n; k0 += RR_KC) {
-    __syncthreads();
-    for (int e = t; e < RR_KC * EH_MAXN; e += EH_THREADS) {
-      const int k = k0 + e / EH_MAXN, j = e % EH_MAXN;
-      Ms[e] = (k < n && j < n) ? M[k * n + j] : zero;
-    }
-    __syncthreads();
-    const int kend = min(RR_KC, n - k0);
-    for (int kr = 0; kr < kend; ++kr) {
-      const int k = k0 + kr;
-      float2 vr[4], mv[RR_V];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int r = 4 * warp + u;
-        vr[u] = r < n ? Vs[k * ld + r] : zero;
-      }
-#pragma unroll
-      for (int v = 0; v < RR_V; ++v) mv[v] = Ms[kr * EH_MAXN + lane + 32 * v];
-#pragma unroll
-      for (int v = 0; v < RR_V; ++v)
-        if (32 * v <= k)                                             // M_kj = 0 for j > k
-#pragma unroll
-          for (int u = 0; u < 4; ++u) acc[u][v] = cfma(acc[u][v], vr[u], mv[v]);
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int r = 4 * warp + u;
-    if (r < n) {
-      const float f = 1.f + alpha * lam[r];
-      float2* row = Mcat + (size_t)rank[r] * 2 * n;
-#pragma unroll
-      for (int v = 0; v < RR_V; ++v) {
-        const int j = lane + 32 * v;
-        if (j < n) {
-          row[j] = make_float2(f * acc[u][v].x, f * acc[u][v].y);
-          row[n + j] = make_float2(-alpha * acc[u][v].x, -alpha * acc[u][v].y);
-        }
-      }
-    }
-  }
+  const int ld = n + 1, t = threadIdx.x, r = t / n, j = t - r * n;
+  if (t < n * n) R[t] = M[t];
+  __syncthreads();
+  if (t >= n * n) return;
+  float2 c = make_float2(0.f, 0.f);
+  for (int k = 0; k < n; ++k) c = cfma(c, Vs[k * ld + r], R[k * n + j]);
+  const float f = 1.f + alpha * lam[r];
+  float2* row = Mcat + (size_t)rank[r] * 2 * n;
+  row[j] = make_float2(f * c.x, f * c.y);
+  row[n + j] = make_float2(-alpha * c.x, -alpha * c.y);
 }
 
 // Inputs and outputs of the Rayleigh-Ritz variant (all device pointers, row-major, FP32).
@@ -253,14 +138,13 @@ struct RRStep {
 template <bool RR>
 __global__ void __launch_bounds__(EH_THREADS, 1)
     k_eigh_small(const double2* __restrict__ H, int n, double2* __restrict__ Vout, RRStep rr) {
-  extern __shared__ __align__(16) unsigned char esm[];
-  const int ld = n + 1;
-  float2* A = reinterpret_cast<float2*>(esm);                       // [n][ld]
-  float2* R = A + EH_AREG;                                          // packed reflectors
+  __shared__ __align__(16) float2 A[EH_AREG];                        // [n][ld]
+  __shared__ float2 R[EH_RREG];                                      // packed reflectors
   __shared__ float d[EH_MAXN], e[EH_MAXN], e2[EH_MAXN], lam[EH_MAXN];
   __shared__ float2 tau[EH_MAXN], wvp[2][EH_MAXN], red[2][32];
   __shared__ int blk_lo[EH_MAXN], blk_hi[EH_MAXN];
   __shared__ float s_err[EH_WARPS];
+  const int ld = n + 1;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
 
   if (t < 64) red[t >> 5][t & 31] = make_float2(0.f, 0.f);           // entries without a warp stay zero
@@ -278,58 +162,48 @@ __global__ void __launch_bounds__(EH_THREADS, 1)
   // ---- 1. tridiagonalization ---------------------------------------------------------------
   // Entering step k, A[k:, k:] holds the updates of steps < k-1; the update of step k-1
   // (v_{k-1} at R + rprev, w_{k-1} = wvp[(k-1)&1] + ap v_{k-1}) is still to be applied.
-  // Lane-owned indices: rows / columns k+1+lane+32q.
+  // A lane owns row / column j = k+1+lane, a warp row k+1+warp.
   int rprev = 0, roff = 0;
   for (int k = 0; k + 1 < n; ++k) {
     const int m = n - k - 1;
     const bool hp = k > 0;
     const int pb = (k + 1) & 1;                                     // buffer of step k-1
-    float2 ap = make_float2(0.f, 0.f);
+    const int j = k + 1 + lane, i = k + 1 + warp;
+    const float2 zero = make_float2(0.f, 0.f);
+    float2 ap = zero;
     if (hp) {
       const float2 s = warp_sum(red[pb][lane]);
       const float2 h = cm(tau[k - 1], s);
       ap = make_float2(-0.5f * h.x, -0.5f * h.y);
     }
-    // pending-update vectors at the lane's indices and at k
-    float2 vp[4], wp[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int j = k + 1 + lane + 32 * q;
-      vp[q] = make_float2(0.f, 0.f);
-      wp[q] = make_float2(0.f, 0.f);
-      if (hp && j < n) {
-        vp[q] = R[rprev + j - k];
-        wp[q] = cadd(wvp[pb][j], cm(ap, vp[q]));
-      }
+    // pending-update vectors at the lane's index and at k
+    float2 vp = zero, wp = zero;
+    if (hp && j < n) {
+      vp = R[rprev + j - k];
+      wp = cadd(wvp[pb][j], cm(ap, vp));
     }
-    const float2 wk = hp ? cadd(wvp[pb][k], ap) : make_float2(0.f, 0.f);   // v_{k-1}[k] = 1
-    // column k after the pending update: x_i = A_ik - (v_i conj(w_k) + w_i)
-    float2 x[4];
+    const float2 wk = hp ? cadd(wvp[pb][k], ap) : zero;              // v_{k-1}[k] = 1
+    // column k after the pending update: x_j = A_jk - (v_j conj(w_k) + w_j)
+    float2 x = zero;
     float xn2 = 0.f;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int i = k + 1 + lane + 32 * q;
-      x[q] = make_float2(0.f, 0.f);
-      if (i < n) {
-        const float2 a = A[i * ld + k];
-        const float2 u = cadd(make_float2(vp[q].x * wk.x + vp[q].y * wk.y, vp[q].y * wk.x - vp[q].x * wk.y), wp[q]);
-        x[q] = csub(a, u);
-        if (q > 0 || lane > 0) xn2 += x[q].x * x[q].x + x[q].y * x[q].y;
-      }
+    if (j < n) {
+      const float2 u = cadd(make_float2(vp.x * wk.x + vp.y * wk.y, vp.y * wk.x - vp.x * wk.y), wp);
+      x = csub(A[j * ld + k], u);
+      if (lane > 0) xn2 = x.x * x.x + x.y * x.y;
     }
     for (int o = 16; o > 0; o >>= 1) xn2 += __shfl_xor_sync(FULL, xn2, o);
-    const float2 al = make_float2(__shfl_sync(FULL, x[0].x, 0), __shfl_sync(FULL, x[0].y, 0));
-    float2 tk, sc = make_float2(0.f, 0.f);
+    const float2 al = make_float2(__shfl_sync(FULL, x.x, 0), __shfl_sync(FULL, x.y, 0));
+    float2 tk, sc = zero;
     float ek;
     const float s2 = al.x * al.x + al.y * al.y + xn2;
     if (xn2 == 0.f && al.y == 0.f) {
-      tk = make_float2(0.f, 0.f);
+      tk = zero;
       ek = al.x;
     } else if (s2 < 1e-30f) {
       // a column already reduced up to rounding noise (|x| < 1e-15): no reflection and a zero
       // off-diagonal element, which moves eigenvalues by < 1e-15; forming the reflector from
       // such a column would underflow its squares and divide by zero
-      tk = make_float2(0.f, 0.f);
+      tk = zero;
       ek = 0.f;
     } else {
       const float beta = -copysignf(sqrtf(al.x * al.x + al.y * al.y + xn2), al.x);
@@ -340,76 +214,43 @@ __global__ void __launch_bounds__(EH_THREADS, 1)
       sc = make_float2(dn.x * inv, -dn.y * inv);
       ek = beta;
     }
-    float2 vk[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int i = k + 1 + lane + 32 * q;
-      vk[q] = (q == 0 && lane == 0) ? make_float2(1.f, 0.f) : (i < n ? cm(x[q], sc) : make_float2(0.f, 0.f));
-    }
+    const float2 vk = lane == 0 ? make_float2(1.f, 0.f) : (j < n ? cm(x, sc) : zero);
     if (warp == 0) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int i = k + 1 + lane + 32 * q;
-        if (i < n) R[roff + i - k - 1] = vk[q];
-      }
+      if (j < n) R[roff + lane] = vk;
       if (lane == 0) {
         tau[k] = tk;
         e[k] = ek;
         d[k] = A[k * ld + k].x - 2.f * wk.x;
       }
     }
-    // trailing block: apply the update of step k-1, then w'_i = tau_k sum_j A_ij v_j; the
-    // four rows' sums are reduced together so their shuffle latencies overlap
-    float2 acc[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int i = k + 1 + warp + 32 * r;
-      acc[r] = make_float2(0.f, 0.f);
-      if (i < n) {                                                   // warp-uniform
-        float2 vi = make_float2(0.f, 0.f), wi = make_float2(0.f, 0.f);
+    // trailing block: apply the update of step k-1 to row i, then w'_i = tau_k sum_j A_ij v_j
+    float2 acc = zero;
+    if (i < n) {                                                     // warp-uniform
+      float2 vi = zero, wi = zero;
+      if (hp) {
+        vi = R[rprev + i - k];
+        wi = cadd(wvp[pb][i], cm(ap, vi));
+      }
+      if (j < n) {
+        float2 a = A[i * ld + j];
         if (hp) {
-          vi = R[rprev + i - k];
-          wi = cadd(wvp[pb][i], cm(ap, vi));
+          // v_i conj(w_j) + w_i conj(v_j)
+          a.x -= (vi.x * wp.x + vi.y * wp.y) + (wi.x * vp.x + wi.y * vp.y);
+          a.y -= (vi.y * wp.x - vi.x * wp.y) + (wi.y * vp.x - wi.x * vp.y);
         }
-        float2* arow = A + i * ld;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int j = k + 1 + lane + 32 * q;
-          if (j < n) {
-            float2 a = arow[j];
-            if (hp) {
-              // v_i conj(w_j) + w_i conj(v_j)
-              a.x -= (vi.x * wp[q].x + vi.y * wp[q].y) + (wi.x * vp[q].x + wi.y * vp[q].y);
-              a.y -= (vi.y * wp[q].x - vi.x * wp[q].y) + (wi.y * vp[q].x - wi.x * vp[q].y);
-            }
-            if (i == j) a.y = 0.f;
-            arow[j] = a;
-            acc[r].x += a.x * vk[q].x - a.y * vk[q].y;
-            acc[r].y += a.x * vk[q].y + a.y * vk[q].x;
-          }
-        }
+        if (i == j) a.y = 0.f;
+        A[i * ld + j] = a;
+        acc = make_float2(a.x * vk.x - a.y * vk.y, a.x * vk.y + a.y * vk.x);
       }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        acc[r].x += __shfl_xor_sync(FULL, acc[r].x, o);
-        acc[r].y += __shfl_xor_sync(FULL, acc[r].y, o);
-      }
-    float2 pw = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int i = k + 1 + warp + 32 * r;
-      // v_k at row i lives in lane (i - k - 1) & 31 = warp, slot r
-      const float2 vr = make_float2(__shfl_sync(FULL, vk[r].x, warp), __shfl_sync(FULL, vk[r].y, warp));
-      if (i < n) {
-        const float2 w = cm(tk, acc[r]);
-        if (lane == 0) wvp[k & 1][i] = w;
-        const float2 c = cmc(w, vr);
-        pw.x += c.x;
-        pw.y += c.y;
-      }
+    acc = warp_sum(acc);
+    // v_k at row i lives in lane i - k - 1 = warp
+    const float2 vr = make_float2(__shfl_sync(FULL, vk.x, warp), __shfl_sync(FULL, vk.y, warp));
+    float2 pw = zero;
+    if (i < n) {
+      const float2 w = cm(tk, acc);
+      if (lane == 0) wvp[k & 1][i] = w;
+      pw = cmc(w, vr);
     }
     if (lane == 0) red[k & 1][warp] = pw;
     rprev = roff;
@@ -493,12 +334,13 @@ __global__ void __launch_bounds__(EH_THREADS, 1)
   __syncthreads();
 
   // ---- 3. eigenvectors of T ----------------------------------------------------------------
-  // Z (real, [n][zld]) in the upper half of the A region; D- pivots [n][n] and later
-  // Z^T Z in the lower half.
+  // Z (real, [n][zld]) in the second half of the A region; D- pivots [n][n] and later
+  // Z^T Z in the first.
   const int zld = n + 1;
   const float tiny = 1e-30f + 1e-13f * tnorm;                        // pivot floor
-  float* Zr = reinterpret_cast<float*>(esm) + EH_MAXN * EH_MAXN;
-  float* low = reinterpret_cast<float*>(esm);
+  float* low = reinterpret_cast<float*>(A);
+  float* Zr = low + EH_MAXN * EH_MAXN;
+  static_assert(EH_MAXN * EH_MAXN + EH_AREG <= 2 * EH_AREG, "both fit");
   for (int idx = t; idx < n * zld; idx += EH_THREADS) Zr[idx] = 0.f;
   __syncthreads();
   if (t < n) {
@@ -607,72 +449,36 @@ __global__ void __launch_bounds__(EH_THREADS, 1)
   }
   __syncthreads();
   // Newton-Schulz: G = Z^T Z; while max |G - I| > 2e-6: Z <- 1.5 Z - 0.5 Z G.
-  // Thread tiles: rows warp + 32u, columns lane + 32v (u, v < 4).  The Rayleigh-Ritz variant
-  // skips it: its vectors only span the next iterate, whose CholQR orthonormalises the block,
-  // and outside degenerate clusters (handled above) they are orthogonal to eps |T| / gap
-  // <= 6e-3, a condition number of the step matrix within 1.01.
+  // Thread: row warp, column lane.  The Rayleigh-Ritz variant skips it: its vectors only span the next
+  // iterate, whose CholQR orthonormalises the block, and outside degenerate clusters (handled above) they
+  // are orthogonal to eps |T| / gap <= 6e-3, a condition number of the step matrix within 1.01.
   if constexpr (!RR) {
     float* G = low;                                                  // [n][n]
+    const bool in = warp < n && lane < n;
     for (int it = 0; it < 4; ++it) {
-      float g[4][4] = {};
-      for (int i = 0; i < n; ++i) {
-        float za[4], zb[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int a = warp + 32 * u, b = lane + 32 * u;
-          za[u] = a < n ? Zr[i * zld + a] : 0.f;
-          zb[u] = b < n ? Zr[i * zld + b] : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-          for (int v = 0; v < 4; ++v) g[u][v] += za[u] * zb[v];
+      float g = 0.f, err = 0.f;
+      if (in) {
+        for (int i = 0; i < n; ++i) g += Zr[i * zld + warp] * Zr[i * zld + lane];
+        G[warp * n + lane] = g;
+        err = fabsf(g - (warp == lane ? 1.f : 0.f));
       }
-      float err = 0.f;
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          const int a = warp + 32 * u, b = lane + 32 * v;
-          if (a < n && b < n) {
-            G[a * n + b] = g[u][v];
-            err = fmaxf(err, fabsf(g[u][v] - (a == b ? 1.f : 0.f)));
-          }
-        }
       for (int o = 16; o > 0; o >>= 1) err = fmaxf(err, __shfl_xor_sync(FULL, err, o));
       if (lane == 0) s_err[warp] = err;
       __syncthreads();
       float emax = 0.f;
       for (int w = 0; w < EH_WARPS; ++w) emax = fmaxf(emax, s_err[w]);
       if (!(emax > 2e-6f)) break;                                    // uniform
-      float z[4][4] = {};
-      for (int b = 0; b < n; ++b) {
-        float zr[4], gb[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int i = warp + 32 * u, a = lane + 32 * u;
-          zr[u] = i < n ? Zr[i * zld + b] : 0.f;
-          gb[u] = a < n ? G[b * n + a] : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-          for (int v = 0; v < 4; ++v) z[u][v] += zr[u] * gb[v];
-      }
+      float z = 0.f;
+      if (in)
+        for (int b = 0; b < n; ++b) z += Zr[warp * zld + b] * G[b * n + lane];
       __syncthreads();
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          const int i = warp + 32 * u, a = lane + 32 * v;
-          if (i < n && a < n) Zr[i * zld + a] = 1.5f * Zr[i * zld + a] - 0.5f * z[u][v];
-        }
+      if (in) Zr[warp * zld + lane] = 1.5f * Zr[warp * zld + lane] - 0.5f * z;
       __syncthreads();
     }
   }
 
   // ---- 4. V = H_0 ... H_{n-2} Z ------------------------------------------------------------
-  // thread (column j = t / 8, s = t % 8) holds rows s + 8p, p < 16.  The reflectors are
+  // thread (column j = t / 8, s = t % 8) holds rows s + 8p, p < 2.  The reflectors are
   // expanded into a zero-padded [n-1][EH_MAXN] layout in the A region (v_k[i] = 0 for i <= k
   // and i >= n), so no row needs a bounds test.
   {
@@ -977,146 +783,26 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
 #undef XL
 }
 
-// Triangular products on 8 x 8 output tiles (64 threads, one output each), K staged through
-// shared memory in chunks of 32 with coalesced loads:
-//   MODE 0: C = S M^H             C_ij = sum_{k <= j} S_ik conj(M_jk)          (all tiles, FP64)
-//   MODE 1: C = M T (lower part)  C_ij = sum_{k <= i} M_ik T_kj, i >= j          (FP64)
-//   MODE 2: C = conj(B - Phi(A - I) B) with A = S2 (lower) and B = M1:
-//           C_ij = conj(B_ij - sum_{j <= k <= i} Phi_ik B_kj), Phi_ik = A_ik for k < i and
-//           (A_ii - 1)/2 for k = i; i >= j, 0 above; C = I once *status is set.  Phi is
-//           O(eps_32 kappa), so FP32 products keep the 24-bit accuracy of the rotation.
-// MODE 2 also writes an FP32 copy of C to C32 when it is given.
-template <int MODE>
-__global__ void __launch_bounds__(64) k_tri_small(const double2* __restrict__ A, const double2* __restrict__ B,
-                                                    int n, const int* __restrict__ status, double2* __restrict__ C,
-                                                    float2* __restrict__ C32) {
-  constexpr int KC = 32;
-  __shared__ double2 As[8][KC + 1];
-  __shared__ double2 Bs[8][KC + 1];                                  // Bs[j][k]
-  const int ty = threadIdx.x >> 3, tx = threadIdx.x & 7;
-  const int I = blockIdx.y * 8, J = blockIdx.x * 8;
-  const int i = I + ty, j = J + tx;
-  if (MODE == 2 && *status != 0) {
-    if (i < n && j < n) {
-      C[(size_t)i * n + j] = make_double2(i == j ? 1.0 : 0.0, 0.0);
-      if (C32) C32[(size_t)i * n + j] = make_float2(i == j ? 1.f : 0.f, 0.f);
-    }
-    return;
-  }
-  if (MODE != 0 && J > I) {                                          // strictly upper tile
-    if (MODE == 2 && i < n && j < n) {
-      C[(size_t)i * n + j] = make_double2(0.0, 0.0);
-      if (C32) C32[(size_t)i * n + j] = make_float2(0.f, 0.f);
-    }
-    return;
-  }
-  // k range of the tile
-  const int k0 = MODE == 2 ? J : 0;
-  const int k1 = min(n, MODE == 0 ? J + 8 : I + 8);
-  using R = typename std::conditional<MODE == 2, float, double>::type;
-  R re = 0, im = 0;
-  for (int kc = k0; kc < k1; kc += KC) {
-    for (int e = threadIdx.x; e < 8 * KC; e += 64) {
-      const int r = e / KC, k = kc + e % KC;
-      As[r][e % KC] = (I + r < n && k < k1) ? A[(size_t)(I + r) * n + k] : make_double2(0.0, 0.0);
-      if (MODE == 0) {
-        Bs[r][e % KC] = (J + r < n && k < k1) ? B[(size_t)(J + r) * n + k] : make_double2(0.0, 0.0);
-      } else {
-        const int kk = kc + e / 8, jj = e % 8;                        // B rows k, columns J..J+7
-        Bs[jj][e / 8] = (kk < k1 && J + jj < n) ? B[(size_t)kk * n + J + jj] : make_double2(0.0, 0.0);
-      }
-    }
-    __syncthreads();
-    const int kend = min(KC, k1 - kc);
-    for (int kk = 0; kk < kend; ++kk) {
-      const int k = kc + kk;
-      const double2 a = As[ty][kk], b = Bs[tx][kk];
-      if (MODE == 0) {
-        if (k <= j) {
-          re += a.x * b.x + a.y * b.y;
-          im += a.y * b.x - a.x * b.y;
-        }
-      } else if (MODE == 1) {
-        if (k <= i) {
-          re += a.x * b.x - a.y * b.y;
-          im += a.x * b.y + a.y * b.x;
-        }
-      } else {
-        if (k >= j && k <= i) {
-          R ax = (R)a.x, ay = (R)a.y;
-          if (k == i) {                                              // Phi_ii = (A_ii - 1) / 2
-            ax = (R)(0.5 * (a.x - 1.0));
-            ay = 0;
-          }
-          const R bx = (R)b.x, by = (R)b.y;
-          re += ax * bx - ay * by;
-          im += ax * by + ay * bx;
-        }
-      }
-    }
-    __syncthreads();
-  }
-  if (i >= n || j >= n) return;
-  if (MODE == 0) {
-    C[(size_t)i * n + j] = make_double2((double)re, (double)im);
-  } else if (MODE == 1) {
-    if (j <= i) C[(size_t)i * n + j] = make_double2((double)re, (double)im);
-  } else {
-    double2 c = make_double2(0.0, 0.0);
-    if (j <= i) {
-      const double2 bij = B[(size_t)i * n + j];
-      c = make_double2(bij.x - (double)re, -(bij.y - (double)im));
-    }
-    C[(size_t)i * n + j] = c;
-    if (C32) C32[(size_t)i * n + j] = make_float2((float)c.x, (float)c.y);
-  }
-}
-
 }  // namespace
 
 void eigh_small(const double2* A, double2* V, int n, cudaStream_t s) {
   if (n > SMALL_SUBSPACE || n < 1) fail(KS_ERR_ARG, "eigh_small: n=%d not in [1, %d]", n, SMALL_SUBSPACE);
-  static bool attr = false;
-  if (!attr) {
-    KS_CUDA(cudaFuncSetAttribute(k_eigh_small<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EH_SMEM));
-    attr = true;
-  }
-  k_eigh_small<false><<<1, EH_THREADS, EH_SMEM, s>>>(A, n, V, RRStep{});
+  k_eigh_small<false><<<1, EH_THREADS, 0, s>>>(A, n, V, RRStep{});
   KS_CHECK_LAUNCH();
 }
 
 void rr_step_small(const float2* Hraw, const float2* M, double alpha, int n, float2* Mcat, float2* Aout,
                    float2* Vout, int* perm, cudaStream_t s) {
   if (n > SMALL_SUBSPACE || n < 1) fail(KS_ERR_ARG, "rr_step_small: n=%d not in [1, %d]", n, SMALL_SUBSPACE);
-  static bool attr = false;
-  if (!attr) {
-    KS_CUDA(cudaFuncSetAttribute(k_eigh_small<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EH_SMEM));
-    attr = true;
-  }
   const RRStep rr{Hraw, M, (float)alpha, Mcat, Aout, Vout, perm};
-  k_eigh_small<true><<<1, EH_THREADS, EH_SMEM, s>>>(nullptr, n, nullptr, rr);
+  k_eigh_small<true><<<1, EH_THREADS, 0, s>>>(nullptr, n, nullptr, rr);
   KS_CHECK_LAUNCH();
 }
 
-void cholesky_small(const double2* S, double2* M, int n, double tol, double2* work, int* status, cudaStream_t s,
-                    float2* M32, bool refine) {
-  if (n > SMALL_SUBSPACE || n < 1) fail(KS_ERR_ARG, "cholesky_small: n=%d not in [1, %d]", n, SMALL_SUBSPACE);
-  double2* M1 = work;
-  double2* T = work + (size_t)n * n;
-  double2* S2 = work + (size_t)2 * n * n;
-  if (!refine) {                                                     // the FP32 factor itself
-    k_chol_small<<<1, SC_THREADS, 0, s>>>(S, n, tol, 1, status, M, M32);
-    KS_CHECK_LAUNCH();
-    return;
-  }
-  const dim3 grid((n + 7) / 8, (n + 7) / 8);
-  k_chol_small<<<1, SC_THREADS, 0, s>>>(S, n, tol, 0, status, M1, nullptr);
-  KS_CHECK_LAUNCH();
-  k_tri_small<0><<<grid, 64, 0, s>>>(S, M1, n, status, T, nullptr);
-  KS_CHECK_LAUNCH();
-  k_tri_small<1><<<grid, 64, 0, s>>>(M1, T, n, status, S2, nullptr);   // S2 = M1 S M1^H (lower)
-  KS_CHECK_LAUNCH();
-  k_tri_small<2><<<grid, 64, 0, s>>>(S2, M1, n, status, M, M32);
+void chol32_small(const double2* S, int n, double tol, int conj_out, int* status, double2* Out, float2* Out32,
+                  cudaStream_t s) {
+  if (n > SMALL_SUBSPACE || n < 1) fail(KS_ERR_ARG, "chol32_small: n=%d not in [1, %d]", n, SMALL_SUBSPACE);
+  k_chol_small<<<1, SC_THREADS, 0, s>>>(S, n, tol, conj_out, status, Out, Out32);
   KS_CHECK_LAUNCH();
 }
 
