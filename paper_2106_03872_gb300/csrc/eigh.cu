@@ -602,7 +602,8 @@ __global__ void __launch_bounds__(256) k_rr_product(const float2* __restrict__ A
 }
 
 // Reported eigenvalues of the Rayleigh-Ritz variant: FP64 Rayleigh quotients of the FP32
-// eigenvectors on the FP32 subspace matrix (of its Hermitian part, the real part of the quotient), eig[perm[j]] = Re(v_j^H A v_j) / (v_j^H v_j).
+// eigenvectors on the FP32 subspace matrix (of its Hermitian part, the real part of the quotient),
+// eig[perm[j]] = Re(v_j^H A v_j) / (v_j^H v_j).
 __global__ void k_ritz_values(const float2* __restrict__ A, const float2* __restrict__ V, const int* __restrict__ perm,
                               int n, double* __restrict__ eig) {
   const int j = blockIdx.x;

@@ -689,7 +689,7 @@ template <typename T> class Engine final : public EngineBase {
     // reorganised around the linearity of H:
     //  - S = psi^H psi and H_raw = psi^H (H psi) are formed on the raw block; the factor M of S,
     //    H_sub = conj(M) H_raw M^T, its eigenvectors Vt, C = Vt M and the step matrix
-    //    Mcat = [(I + alpha Lambda) C | -alpha C] run on the side stream (one SM), while
+    //    Mcat = [(I + alpha Lambda) C | -alpha C] run on the side stream, while
     //  - the main stream applies H to H psi (H^2 psi);
     //  - then psi <- Mcat [psi; H psi] and H psi <- Mcat [H psi; H^2 psi].
     // On the mixed path with n <= 128 the side stream's Rayleigh-Ritz step runs in FP32
@@ -1637,10 +1637,10 @@ template <typename T> class Engine final : public EngineBase {
   double* eig_ = nullptr;
   double* lam_ = nullptr;
   void* ehw_ = nullptr;      // workspace of the FP32 eigensolver
-  double2* chw_ = nullptr;   // two-pass FP32 Cholesky workspace (mixed path)
+  double2* chw_ = nullptr;   // FP32 Cholesky factor and its FP64 refinement (mixed path)
   double2 *mT_ = nullptr, *mC_ = nullptr, *mF_ = nullptr;   // subspace products, FP64 factor scratch
   double2* mCat_ = nullptr;                                   // [n][2n] steepest-descent step matrix
-  // one-CTA Rayleigh-Ritz step of the block iteration (FP32 operands and results)
+  // Rayleigh-Ritz step of the block iteration in FP32 (operands and results)
   float2 *hraw32_ = nullptr, *m32_ = nullptr, *mcat32_ = nullptr, *aexp_ = nullptr, *vexp_ = nullptr;
   int* perm_ = nullptr;
   cudaStream_t setup_ = nullptr;     // = aux_: setup work at creation and at atom moves

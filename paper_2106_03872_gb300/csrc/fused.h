@@ -55,7 +55,8 @@ class FusedOps {
   // out[b][z][x][y] = Omega^{1/2} psi_b(r) on the grid (plane-major: z slowest), the unscaled
   // inverse transform of n packed states, by the pruned z-columns and the in-SMEM y, x passes.
   virtual void real_space(const float2* psi, int n, float2* out, cudaStream_t s) = 0;
-  // Forces (Eq. 11) of a chunk of n packed states, on the grids with a team plan (force_chunks): fg[a] += sum_b 2 occ[b] Re(conj(d_a psi_b) psi_b) for a = x, y, z (fg [3][N^3], planes [z][x][y]),
+  // Forces (Eq. 11) of a chunk of n packed states, on the grids with a team plan (force_chunks):
+  // fg[a] += sum_b 2 occ[b] Re(conj(d_a psi_b) psi_b) for a = x, y, z (fg [3][N^3], planes [z][x][y]),
   // fnl -= the projectors' part (w and fnl as nl_force, projections scaled by pscale).  gz: i G_z c of the
   // states (packed); grid [n][N^3], p and q [n][natoms nproj] work.
   virtual bool force_chunks() const = 0;

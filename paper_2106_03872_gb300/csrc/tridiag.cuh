@@ -1,5 +1,5 @@
 // Householder reduction of a Hermitian FP32 matrix to real symmetric tridiagonal form by a cluster of
-// CTAs (eigh_cluster.cu).
+// CTAs (eigh.cu).
 //
 // The reflector H_k = I - tau_k v_k v_k^H (v_k[k+1] = 1) maps A[k+1:, k] to (beta_k, 0, ...) with real
 // beta_k; the trailing block takes A -= v w^H + w v^H, w = w' - (tau/2)(w'^H v) v, w' = tau A v.  The
