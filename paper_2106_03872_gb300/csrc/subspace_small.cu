@@ -1,7 +1,8 @@
 // Subspace kernels for blocks of at most 16 states on the mixed path: the eigensolver, the whole
-// Rayleigh-Ritz step and the Cholesky factor, in one CTA each.  At these sizes the launches of the spread-out solver
-// (eigh.cu) cost more than its parallelism saves: a Rayleigh-Ritz step of 8 states takes 36 us here and
-// 89 us there (at 16 states the eigensolver takes 92 and 81 us, about level).
+// Rayleigh-Ritz step and the Cholesky factor, in one CTA each.  The chain of dependent steps bounds them; at
+// these sizes the launches of the spread-out solver (eigh.cu) cost more than its parallelism saves: kernel time of
+// a Rayleigh-Ritz step 19 us at 8 and 37 us at 16 states in one launch, where seven launches take 54 us at 17; of
+// the eigensolver 20 and 36 us, where ten take 60 us.
 //
 // The eigensolver, FP32, matrix in shared memory, a warp per row:
 //   1. Householder reduction to a real symmetric tridiagonal T, the update of step k-1 applied in the
